@@ -1,0 +1,306 @@
+// The FP64 tile march of the D2Q9 step.  Internal header of kernels_d2q9.cu.
+//
+// What bounds it: the FP64 pipe.  GB300 issues one FP64 warp instruction per
+// 16 cycles and SM (about 630 G operations/s on the chip), so a node update
+// costs its FP64 operations and nothing else: loads, shared memory, index
+// arithmetic and barriers hide behind them.  The march is therefore written
+// for the fewest FP64 operations, not for bytes or registers:
+//  * vertical second differences v = (phi_N - phi) + (phi_S - phi) and first
+//    differences d = phi_N - phi_S are formed once per node and shared with
+//    the neighbour columns through shared-memory rings: the Laplacian is
+//    h + (2/3) v + (1/6)(v_E + v_W) with h the horizontal second difference,
+//    and the gradient (1/2)(phi_E - phi_W) + (1/12)(v_E - v_W),
+//    (1/3) d + (1/12)(d_E + d_W).  Every term stays a difference of
+//    neighbours, so a uniform phase still gives exact zeros;
+//  * one reciprocal of rho tau_g serves 1/rho and 1/tau_g;
+//  * each collision is one multiply-add per population on coefficients
+//    formed once per node and direction class;
+//  * the halo columns of both thread rows are one warp's extra work instead
+//    of two warps'.
+// About 153 FP64 operations per node against about 250 in the form shared with
+// the FP32 kernel before.  Measured with per-step launches, whole runs of 40
+// and 400 steps: 1024 x 1024 505 -> 363 us per step (the operations alone take
+// 255 us), 16 x 128 16.5 -> 9.9 us.
+#pragma once
+
+// shared memory of one FP64 tile march
+template <int TX>
+struct TileSmem64 {
+    static constexpr int RP = 8;        // phi ring: rows t .. t + 3 read, t + 4, t + 5 next
+    static constexpr int RV = 4;        // v, d and mu rings: four rows alive
+    static constexpr int WP = TX + 4;   // phi, v, d ring width (halo 2)
+    static constexpr int WM = TX + 2;   // mu ring width (halo 1)
+    static constexpr int NT = TX * 2;
+    double phs[RP * WP], vs[RV * WP], ds[RV * WP], mus[RV * WM];
+    double red[7][(NT + 31) / 32];
+    int bad;
+};
+
+// 1/x to about one rounding: the hardware's 20-bit estimate r and one step of
+// Householder's third-order iteration, e = 1 - x r, r (1 + e + e^2), whose
+// error is e^3 < 2^-57.  x = rho tau_g, positive and of order one.
+__device__ __forceinline__ double rcp64(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(fma(e, e, e), r, r);
+}
+
+// One tile: columns [x0, x0 + TX), rows [y0, yend), marching in direction dir
+// (see d2q9_tile, which this replaces for FP64 storage).
+template <int TX, int PASS, bool NC>
+__device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
+                                            const StepParams<double> &P, const PassArgs &a, int x0,
+                                            int y0, int yend, int dir, int part)
+{
+    using SM = TileSmem64<TX>;
+    constexpr int WP = SM::WP, WM = SM::WM, NT = SM::NT, NW = (NT + 31) / 32;
+    constexpr bool NEED_S = (PASS & (PASS_STATE | PASS_DIAG)) != 0;
+    double(*const dacc)[NT] = reinterpret_cast<double(*)[NT]>(dyn);
+    double(*const facc)[NT] = dacc + 4;
+    const int tx = threadIdx.x, ty = threadIdx.y, lin = ty * TX + tx;
+    const int nx = P.nx, ny = P.ny;
+    const unsigned N = (unsigned)P.N;
+    const bool small = ny < 4;
+    const double *__restrict__ fsrc = static_cast<const double *>(a.f_src);
+    const double *__restrict__ gsrc = static_cast<const double *>(a.g_src);
+
+    const int xo = x0 + tx;
+    const bool col_ok = xo < nx;
+    // columns past the grid's last one are needed up to the stencil's reach
+    // (two columns); warps wholly beyond it skip the FP64 work
+    const bool col_phi = xo < nx + 2;
+    const unsigned xO = wrapi(xo, nx), xOm = wrapi(xo - 1, nx), xOp = wrapi(xo + 1, nx);
+    // halo work of both thread rows: the last 8 threads, 4 halo columns each
+    // (ring index 0, 1, TX + 2, TX + 3); column k of thread row q
+    const int hk = lin - (NT - 8);
+    const bool halo = hk >= 0;
+    const int hq = (hk >> 2) & 1, hc = hk & 3;
+    const int jH = hc < 2 ? hc : TX + hc;
+    const int cH = x0 - 2 + jH;
+    // (a ragged last strip never reads the ring past its own columns + 2)
+    const bool halo_phi = halo && cH < nx + 2;
+    const unsigned xH = wrapi(cH, nx), xHm = wrapi(cH - 1, nx), xHp = wrapi(cH + 1, nx);
+    // mu halo: columns ring index 0 and TX + 1 (phi ring 1 and TX + 2)
+    const bool halo_mu = halo && (hc == 1 || hc == 2) && cH < nx + 1;
+
+    const int first = dir > 0 ? y0 : yend - 1;
+    const int nout = yend - y0;
+    const double beta4 = 4.0 * P.beta, hd = 0.5 * (P.phil - P.phiv), q0 = hd * hd;
+    const double kap = P.kappa, k23 = P.kappa * (2.0 / 3.0), k16 = P.kappa * (1.0 / 6.0);
+
+    // ring rows of march coordinate m >= -2
+    auto prow = [&](int m) { return sm.phs + ((m + 2) & 7) * WP; };
+    auto vrow = [&](int m) { return sm.vs + ((m + 4) & 3) * WP; };
+    auto drow = [&](int m) { return sm.ds + ((m + 4) & 3) * WP; };
+    auto mrow = [&](int m) { return sm.mus + ((m + 4) & 3) * WM; };
+
+    struct Rows {
+        unsigned rm, r0, rp;
+    };
+    auto rows_of = [&](int m) {
+        const int row = first + dir * m;
+        Rows r;
+        r.rm = (unsigned)wrap_row(row - 1, ny, small) * nx;
+        r.r0 = (unsigned)wrap_row(row, ny, small) * nx;
+        r.rp = (unsigned)wrap_row(row + 1, ny, small) * nx;
+        return r;
+    };
+    // phi rows mb + ty (own columns, keeping the pulls and their sum) and the
+    // halo columns of rows mb, mb + 1
+    auto phi_rows = [&](int mb, double v[9], double &s) {
+        if (col_phi) {
+            const Rows r = rows_of(mb + ty);
+            pull9<NC>(fsrc, N, r.rm, r.r0, r.rp, xOm, xO, xOp, v);
+            s = sum_moving(v);
+            prow(mb + ty)[tx + 2] = v[0] + s;
+        }
+        if (halo_phi) {
+            const Rows r = rows_of(mb + hq);
+            double h[9];
+            pull9<NC>(fsrc, N, r.rm, r.r0, r.rp, xHm, xH, xHp, h);
+            prow(mb + hq)[jH] = h[0] + sum_moving(h);
+        }
+    };
+    // v and d (in +y) of one ring element of row m
+    auto vd_at = [&](int m, int j) {
+        const double *pm = prow(m - dir), *p0 = prow(m), *pp = prow(m + dir);
+        const double n = pp[j], s = pm[j], c = p0[j];
+        vrow(m)[j] = (n - c) + (s - c);
+        drow(m)[j] = n - s;
+    };
+    auto vd_rows = [&](int mb) {
+        if (col_phi) vd_at(mb + ty, tx + 2);
+        if (halo_phi) vd_at(mb + hq, jH);
+    };
+    // Eq. chemical_potencial; j is the phi ring index.  The double-well
+    // derivative is 4 beta t (t^2 - (dphi/2)^2) with t = phi - phibar
+    auto mu_at = [&](int m, int j) {
+        const double *p0 = prow(m), *v = vrow(m);
+        const double c = p0[j];
+        const double h = (p0[j + 1] - c) + (p0[j - 1] - c);
+        const double t = c - P.phibar;
+        double mu = (beta4 * t) * fma(t, t, -q0);
+        mu = fma(-kap, h, mu);
+        mu = fma(-k23, v[j], mu);
+        mrow(m)[j - 1] = fma(-k16, v[j + 1] + v[j - 1], mu);
+    };
+    auto mu_rows = [&](int mb) {
+        if (xo < nx + 1) mu_at(mb + ty, tx + 2);
+        if (halo_mu) mu_at(mb + hq, jH);
+    };
+
+    if (PASS & PASS_DIAG) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dacc[q][lin] = 0.0;
+        facc[0][lin] = 0.0;
+        facc[1][lin] = INFINITY;
+        facc[2][lin] = -INFINITY;
+        if (lin == 0) sm.bad = 0;  // read after the march's barriers
+    }
+
+    // prologue: phi rows -2 .. 1, v, d and mu rows -1, 0
+    double fcur[9], fnext[9], scur = 0.0, snext = 0.0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) fcur[i] = fnext[i] = 0.0;
+    phi_rows(-2, fnext, snext);
+    phi_rows(0, fcur, scur);
+    __syncthreads();
+    vd_rows(-1);
+    __syncthreads();
+    mu_rows(-1);
+
+    for (int t = 0; t < nout; t += 2) {
+        const int m = t + ty, row = first + dir * m;
+        const bool out_ok = col_ok && m < nout;
+        const Rows r = rows_of(m);
+        double gv[9], Sprev = 0.0;
+        if (out_ok) {
+            pull9<NC>(gsrc, N, r.rm, r.r0, r.rp, xOm, xO, xOp, gv);
+            if (NEED_S)
+                Sprev = NC ? __ldcs(static_cast<const double *>(a.S) + (r.r0 + xo))
+                           : __ldcg(static_cast<const double *>(a.S) + (r.r0 + xo));
+        }
+        phi_rows(t + 2, fnext, snext);
+        __syncthreads();
+        vd_rows(t + 1);
+        __syncthreads();
+        mu_rows(t + 1);
+        __syncthreads();
+        if (out_ok) {
+            const double *p0 = prow(m), *v = vrow(m), *dd = drow(m);
+            const double *mm = mrow(m - dir), *m0 = mrow(m), *mp = mrow(m + dir);
+            const int j = tx + 2, k = tx + 1;
+            const double phi = fcur[0] + scur;
+            const double mu = m0[k];
+            // q = 2 grad(phi)
+            const double qx = fma(1.0 / 6.0, v[j + 1] - v[j - 1], p0[j + 1] - p0[j - 1]);
+            const double qy = fma(1.0 / 6.0, dd[j + 1] + dd[j - 1], (2.0 / 3.0) * dd[j]);
+            // F = -phi grad(mu) + G with grad(mu) = (1/3)[axis + (1/4) diagonal]
+            const double da = mp[k + 1] - mm[k - 1], db = mm[k + 1] - mp[k - 1];
+            const double f3 = (-1.0 / 3.0) * phi;
+            const double Fx = fma(f3, fma(0.25, da + db, m0[k + 1] - m0[k - 1]), P.G[0]);
+            const double Fy = fma(f3, fma(0.25, da - db, mp[k] - mm[k]), P.G[1]);
+            const double dphi = phi - P.phiv;
+            const double rho = fma(P.drho, dphi, P.rhov);
+            const double taug = fma(3.0 * P.dnu, dphi, fma(3.0, P.nuv, 0.5));
+            const double inv = rcp64(rho * taug);
+            const double irho = inv * taug, itg = inv * rho;
+            // rho u = sum_i c_i g_i + F/2
+            const double ga = gv[5] - gv[7], gb = gv[8] - gv[6];
+            const double jx = (gv[2] - gv[4]) + (ga + gb), jy = (gv[3] - gv[1]) + (ga - gb);
+            const double ux = fma(0.5, Fx, jx) * irho, uy = fma(0.5, Fy, jy) * irho;
+            const double S2 = fma(ux, qx, uy * qy);  // 2 u.grad(phi)
+            const double uu = fma(ux, ux, uy * uy), ruu = rho * uu;
+            // 3p = (9/5)[sum_{i!=0} g_i + u.grad(rho)/2 - (2/3) rho |u|^2]
+            const double p3 =
+                1.8 * fma(-2.0 / 3.0, ruu, fma(0.25 * P.drho, S2, sum_moving(gv)));
+
+            if (PASS & PASS_DIAG) {
+                dacc[0][lin] += phi;
+                dacc[1][lin] = fma(0.5, ruu, dacc[1][lin]);
+                dacc[2][lin] = fma(0.5, S2, dacc[2][lin]);
+                dacc[3][lin] += Sprev;
+                facc[0][lin] = fmax(facc[0][lin], uu);
+                facc[1][lin] = fmin(facc[1][lin], mu);
+                facc[2][lin] = fmax(facc[2][lin], mu);
+                if (!isfinite(phi) || !isfinite(p3) || !isfinite(uu) || !isfinite(mu)) sm.bad = 1;
+            }
+            const unsigned n = r.r0 + xo;
+            if (PASS & PASS_MACROS) {
+                if (a.out_phi) a.out_phi[n] = phi;
+                if (a.out_p) a.out_p[n] = p3 * (1.0 / 3.0);
+                if (a.out_mu) a.out_mu[n] = mu;
+                if (a.out_u) {
+                    a.out_u[n] = ux;
+                    a.out_u[(size_t)N + n] = uy;
+                }
+            }
+            if (PASS & PASS_MACROS_T) {
+                static_cast<double *>(a.mt_phi)[n] = phi;
+                static_cast<double *>(a.mt_p)[n] = p3 * (1.0 / 3.0);
+                static_cast<double *>(a.mt_mu)[n] = mu;
+                static_cast<double *>(a.mt_u)[n] = ux;
+                static_cast<double *>(a.mt_u)[(size_t)N + n] = uy;
+            }
+            if (PASS & PASS_STATE) {
+                double *__restrict__ fd = static_cast<double *>(a.f_dst);
+                double *__restrict__ gd = static_cast<double *>(a.g_dst);
+                static_cast<double *>(a.S_out)[n] = 0.5 * S2;
+                // Eq. BGK with Eqs. H_i, F_i: f* = f (1 - 1/tau_f) + z w_i + w_i b_i Sh,
+                // z = alpha mu / tau_f, Sh = 1.5 S - 0.5 S_prev, b = -2, -1/2, 1;
+                // the rest population through f_0 - f_0^eq = (5/9) alpha mu - sum f_i
+                const double Sh = fma(0.75, S2, -0.5 * Sprev);
+                const double itf = P.inv_tauf, omf = 1.0 - itf;
+                const double z = (itf * P.alpha) * mu;
+                fd[n] = fma(itf, scur, fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, fcur[0])));
+                const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
+#pragma unroll
+                for (int i = 1; i < 9; ++i) fd[i * N + n] = fma(omf, fcur[i], i < 5 ? ka : kd);
+                // Eq. BGK-NS with Eqs. G_i, GGi.  Per direction pair: even part
+                // E = w [itg A + c.u (4.5 rho itg c.u + 3 k drho c.grad phi)], odd part
+                // O = w [3 rho itg c.u + 3 k c.F], k = 1 - itg/2, A = 3p - 1.5 rho |u|^2;
+                // coefficients at w = 1/9, the diagonals take a quarter at the end
+                const double A = fma(-1.5, ruu, p3);
+                const double omg = 1.0 - itg;
+                const double it9 = (1.0 / 9.0) * itg, k9 = fma(-0.5, it9, 1.0 / 9.0);
+                gd[n] = fma(omg, gv[0], itg * fma(4.0 / 9.0, A, -p3));
+                const double e0 = it9 * A, ri = rho * it9, e1 = 4.5 * ri, o1 = 3.0 * ri;
+                const double e2 = (1.5 * P.drho) * k9, o2 = 3.0 * k9;
+                auto pair = [&](double cu, double cF, double cq, double &s, double &d) {
+                    const double E = fma(cu, fma(e2, cq, e1 * cu), e0);
+                    const double O = fma(o2, cF, o1 * cu);
+                    s = E + O;
+                    d = E - O;
+                };
+                double s, d;
+                pair(ux, Fx, qx, s, d);
+                gd[2 * N + n] = fma(omg, gv[2], s);
+                gd[4 * N + n] = fma(omg, gv[4], d);
+                pair(uy, Fy, qy, s, d);
+                gd[3 * N + n] = fma(omg, gv[3], s);
+                gd[1 * N + n] = fma(omg, gv[1], d);
+                pair(ux + uy, Fx + Fy, qx + qy, s, d);
+                gd[5 * N + n] = fma(0.25, s, omg * gv[5]);
+                gd[7 * N + n] = fma(0.25, d, omg * gv[7]);
+                pair(uy - ux, Fy - Fx, qy - qx, s, d);
+                gd[6 * N + n] = fma(0.25, s, omg * gv[6]);
+                gd[8 * N + n] = fma(0.25, d, omg * gv[8]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fcur[i] = fnext[i];
+        scur = snext;
+    }
+
+    if (PASS & PASS_DIAG) {
+        __syncthreads();  // every flag write of the march is done
+        double d_phi = dacc[0][lin], d_E = dacc[1][lin],
+               d_bud = 1.5 * dacc[2][lin] - 0.5 * dacc[3][lin];
+        double d_u2 = facc[0][lin], d_mumin = facc[1][lin], d_mumax = facc[2][lin],
+               d_bad = sm.bad ? 1.0 : 0.0;
+        write_partial<NW>(sm.red, lin, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
+                          a.partials + part);
+    }
+}

@@ -69,10 +69,6 @@ struct Arith<float> {
     // reciprocal to ~1 ulp (rho and tau_g are O(1); FP32 rounding elsewhere dominates)
     __device__ static float rcp(float x) { return __fdividef(1.0f, x); }
 };
-template <>
-struct Arith<double> {
-    __device__ static double rcp(double x) { return 1.0 / x; }
-};
 
 // row index wrap for rows in [-n, 2n) (n >= 4), any row otherwise
 __device__ __forceinline__ int wrap_row(int r, int n, bool small)
@@ -201,6 +197,49 @@ __device__ __forceinline__ void warp_reduce(double &sum0, double &sum1, T &mx, T
     }
 }
 
+// One CTA's diagnostics partial from its threads' sums and extrema (every
+// thread calls it; NW warps): a fixed xor butterfly per warp, then the warps
+// in order.
+template <int NW, typename T>
+__device__ __forceinline__ void write_partial(double (*red)[NW], int lin, double d_phi, double d_E,
+                                              T d_u2, T d_mumin, T d_mumax, double d_bud, T d_bad,
+                                              DiagPartial *out)
+{
+    warp_reduce(d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad);
+    const int lane = lin & 31, wid = lin >> 5;
+    if (lane == 0) {
+        red[0][wid] = d_phi;
+        red[1][wid] = d_E;
+        red[2][wid] = (double)d_u2;
+        red[3][wid] = (double)d_mumin;
+        red[4][wid] = (double)d_mumax;
+        red[5][wid] = d_bud;
+        red[6][wid] = (double)d_bad;
+    }
+    __syncthreads();
+    if (lin == 0) {
+        DiagPartial o;
+        o.sum_phi = 0.0;
+        o.E = 0.0;
+        o.u2max = 0.0;
+        o.mu_min = DBL_MAX;
+        o.mu_max = -DBL_MAX;
+        o.budget = 0.0;
+        o.nonfinite = 0.0;
+        o.pad = 0.0;
+        for (int w = 0; w < NW; ++w) {
+            o.sum_phi += red[0][w];
+            o.E += red[1][w];
+            o.u2max = fmax(o.u2max, red[2][w]);
+            o.mu_min = fmin(o.mu_min, red[3][w]);
+            o.mu_max = fmax(o.mu_max, red[4][w]);
+            o.budget += red[5][w];
+            o.nonfinite = fmax(o.nonfinite, red[6][w]);
+        }
+        *out = o;
+    }
+}
+
 // Resident CTAs per SM targeted by the register budget: every FP32 variant
 // fits 64 registers (1024 threads per SM; the diagnostics accumulate in
 // shared memory), with small register spills in the multi-step kernels
@@ -321,11 +360,11 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
 {
     using SM = TileSmem<T, TX>;
     using SL = SegLayout<TX>;
-    static_assert(!SEG || sizeof(T) == 4, "row-segment staging is FP32");
+    static_assert(sizeof(T) == 4, "FP64 storage runs d2q9_tile64");
     // staged diagnostics step (its own layout of the staging memory)
     constexpr bool DSEG = SEG && (PASS & PASS_DIAG);
     constexpr int R = SM::R, WP = SM::WP, WM = SM::WM;
-    constexpr bool REST_PAIR = sizeof(T) == 4;
+    constexpr bool REST_PAIR = true;
     constexpr int NT = SM::NT, NACC = DiagAcc<T>::NACC, NW = NT / 32;
     T *const phs = sm.phs;
     T *const mus = sm.mus;
@@ -627,7 +666,7 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
             T gpx, gpy, Fx, Fy, rho, inv_rho, itg, ux, uy, grx, gry, ugr, uu, S;
             // Eq. gradient: grad = 3 sum_{i!=0} w_i c_i Psi(x + c_i)
             //   = (1/3)(axis differences) + (1/12)(diagonal differences)
-            if constexpr (sizeof(T) == 4) {
+            {
                 // x and y components as the two lanes of paired instructions
                 const float2 gp = fma2(
                     f2(1.0f / 3.0f), sub2(make_float2(p0[j + 1], pp[j]), make_float2(p0[j - 1], pm[j])),
@@ -664,40 +703,13 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                 ugr = us.x;
                 S = us.y;
                 uu = fmaf(ux, ux, uy * uy);
-            } else {
-                gpx = T(1.0 / 3.0) * (p0[j + 1] - p0[j - 1]) +
-                      T(1.0 / 12.0) * ((pp[j + 1] - pp[j - 1]) + (pm[j + 1] - pm[j - 1]));
-                gpy = T(1.0 / 3.0) * (pp[j] - pm[j]) +
-                      T(1.0 / 12.0) * ((pp[j + 1] - pm[j + 1]) + (pp[j - 1] - pm[j - 1]));
-                const T gmx = T(1.0 / 3.0) * (m0[k + 1] - m0[k - 1]) +
-                              T(1.0 / 12.0) * ((mp[k + 1] - mp[k - 1]) + (mm[k + 1] - mm[k - 1]));
-                const T gmy = T(1.0 / 3.0) * (mp[k] - mm[k]) +
-                              T(1.0 / 12.0) * ((mp[k + 1] - mm[k + 1]) + (mp[k - 1] - mm[k - 1]));
-                // F = -phi grad(mu) + G; rho, nu linear in phi (Eq. vis)
-                Fx = -phi * gmx + P.G[0];
-                Fy = -phi * gmy + P.G[1];
-                const T dphi = phi - P.phiv;
-                rho = P.rhov + dphi * P.drho;
-                const T nu = P.nuv + dphi * P.dnu;
-                inv_rho = Arith<T>::rcp(rho);
-                itg = Arith<T>::rcp(T(0.5) + T(3) * nu);  // nu = cs2 (tau_g - 1/2)
-                // rho u = sum_i c_i g_i + F/2
-                const T jx = (gv[2] - gv[4]) + ((gv[5] - gv[6]) + (gv[8] - gv[7]));
-                const T jy = (gv[3] - gv[1]) + ((gv[5] + gv[6]) - (gv[7] + gv[8]));
-                ux = (jx + T(0.5) * Fx) * inv_rho;
-                uy = (jy + T(0.5) * Fy) * inv_rho;
-                grx = P.drho * gpx;  // grad rho (chain rule)
-                gry = P.drho * gpy;
-                ugr = ux * grx + uy * gry;
-                uu = ux * ux + uy * uy;
-                S = ux * gpx + uy * gpy;  // u.grad(phi)
             }
             // p = cs2/(1-w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0(u)],
             // rho s_0 = -(2/3) rho |u|^2 for D2Q9
             const T p = T(0.6) * (sum_moving(gv) + T(0.5) * ugr - T(2.0 / 3.0) * rho * uu);
 
             if (PASS & PASS_DIAG) {
-                if constexpr (sizeof(T) == 4) {
+                {
                     // (hi, lo) += x with an exact two-sum on the high word
                     auto acc2 = [&](int q, float x) {
                         const float hi = dacc[q][lin];
@@ -709,11 +721,6 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                     acc2(2, 0.5f * rho * uu);
                     acc2(4, S);
                     acc2(6, Sprev);
-                } else {
-                    dacc[0][lin] += phi;
-                    dacc[1][lin] += 0.5 * rho * uu;
-                    dacc[2][lin] += S;
-                    dacc[3][lin] += Sprev;
                 }
                 facc[0][lin] = fmax(facc[0][lin], uu);
                 facc[1][lin] = fmin(facc[1][lin], mu);
@@ -789,7 +796,7 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                 const T kg = T(1) - T(0.5) * itg;
                 const T A = T(3) * p - T(1.5) * rho * uu;
                 st_stream(gd + n, gv[0] + ((T(4.0 / 9.0) * A - T(3) * p) - gv[0]) * itg);  // G_0 = 0
-                if constexpr (sizeof(T) == 4) {
+                {
                     // two populations per paired instruction: f 1..4 and 5..8 in
                     // pairs; g the two axis and the two diagonal direction pairs
                     const float2 it2 = f2(itf);
@@ -825,27 +832,6 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                         st_stream(gd + (m0i * N + n), om.x);
                         st_stream(gd + (m1i * N + n), om.y);
                     }
-                } else {
-#pragma unroll
-                    for (int i = 1; i <= 4; ++i)
-                        st_stream(fd + (i * N + n), fcur[i] + ((ea - fcur[i]) * itf + sa));
-#pragma unroll
-                    for (int i = 5; i <= 8; ++i)
-                        st_stream(fd + (i * N + n), fcur[i] + ((ed - fcur[i]) * itf + sd));
-                    const T cu_[4] = {ux, uy, ux + uy, uy - ux};
-                    const T cF_[4] = {Fx, Fy, Fx + Fy, Fy - Fx};
-                    const T cg_[4] = {grx, gry, grx + gry, gry - grx};
-                    constexpr int ip[4] = {2, 3, 5, 6}, im[4] = {4, 1, 7, 8};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const T w = q < 2 ? T(1.0 / 9.0) : T(1.0 / 36.0);
-                        const T cu = cu_[q];
-                        const T eq_s = w * (A + T(4.5) * rho * cu * cu), eq_a = T(3) * w * rho * cu;
-                        const T G_s = T(3) * w * kg * cu * cg_[q], G_a = T(3) * w * kg * cF_[q];
-                        const T gp = gv[ip[q]], gm = gv[im[q]];
-                        st_stream(gd + (ip[q] * N + n), gp + ((eq_s + eq_a - gp) * itg + (G_s + G_a)));
-                        st_stream(gd + (im[q] * N + n), gm + ((eq_s - eq_a - gm) * itg + (G_s - G_a)));
-                    }
                 }
             }
         }
@@ -856,54 +842,36 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
 
     if (PASS & PASS_DIAG) {
         __syncthreads();  // every flag write of the march is done
-        double d_phi, d_E, d_bud;
-        if constexpr (sizeof(T) == 4) {
-            d_phi = (double)dacc[0][lin] + (double)dacc[1][lin];
-            d_E = (double)dacc[2][lin] + (double)dacc[3][lin];
-            d_bud = 1.5 * ((double)dacc[4][lin] + (double)dacc[5][lin]) -
-                    0.5 * ((double)dacc[6][lin] + (double)dacc[7][lin]);
-        } else {
-            d_phi = dacc[0][lin];
-            d_E = dacc[1][lin];
-            d_bud = 1.5 * dacc[2][lin] - 0.5 * dacc[3][lin];
-        }
-        T d_u2 = facc[0][lin], d_mumin = facc[1][lin], d_mumax = facc[2][lin],
-          d_bad = *dbad ? T(1) : T(0);
-        warp_reduce(d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad);
-        double(*red)[NW] = sm.red;
-        const int lane = lin & 31, wid = lin >> 5;
-        if (lane == 0) {
-            red[0][wid] = d_phi;
-            red[1][wid] = d_E;
-            red[2][wid] = (double)d_u2;
-            red[3][wid] = (double)d_mumin;
-            red[4][wid] = (double)d_mumax;
-            red[5][wid] = d_bud;
-            red[6][wid] = (double)d_bad;
-        }
-        __syncthreads();
-        if (wid == 0 && lane == 0) {
-            DiagPartial o;
-            o.sum_phi = 0.0;
-            o.E = 0.0;
-            o.u2max = 0.0;
-            o.mu_min = DBL_MAX;
-            o.mu_max = -DBL_MAX;
-            o.budget = 0.0;
-            o.nonfinite = 0.0;
-            o.pad = 0.0;
-            for (int w = 0; w < NW; ++w) {
-                o.sum_phi += red[0][w];
-                o.E += red[1][w];
-                o.u2max = fmax(o.u2max, red[2][w]);
-                o.mu_min = fmin(o.mu_min, red[3][w]);
-                o.mu_max = fmax(o.mu_max, red[4][w]);
-                o.budget += red[5][w];
-                o.nonfinite = fmax(o.nonfinite, red[6][w]);
-            }
-            a.partials[part] = o;
-        }
+        const double d_phi = (double)dacc[0][lin] + (double)dacc[1][lin];
+        const double d_E = (double)dacc[2][lin] + (double)dacc[3][lin];
+        const double d_bud = 1.5 * ((double)dacc[4][lin] + (double)dacc[5][lin]) -
+                             0.5 * ((double)dacc[6][lin] + (double)dacc[7][lin]);
+        write_partial<NW, T>(sm.red, lin, d_phi, d_E, facc[0][lin], facc[1][lin], facc[2][lin],
+                             d_bud, *dbad ? T(1) : T(0), a.partials + part);
     }
+}
+
+#include "d2q9_fp64.cuh"
+
+// One tile of either storage type (see d2q9_tile; FP64 has a march of its own,
+// and no row-segment staging).
+template <typename T, int TX>
+struct SmemOf {
+    using type = TileSmem<T, TX>;
+};
+template <int TX>
+struct SmemOf<double, TX> {
+    using type = TileSmem64<TX>;
+};
+template <typename T, int TX, int PASS, bool NC = true, bool SEG = false>
+__device__ __forceinline__ void run_tile(typename SmemOf<T, TX>::type &sm, T *dyn,
+                                         const StepParams<T> &P, const PassArgs &a, int x0, int y0,
+                                         int yend, int dir, int part, unsigned &bph)
+{
+    if constexpr (sizeof(T) == 8)
+        d2q9_tile64<TX, PASS, NC>(sm, dyn, P, a, x0, y0, yend, dir, part);
+    else
+        d2q9_tile<T, TX, PASS, NC, SEG>(sm, dyn, P, a, x0, y0, yend, dir, part, bph);
 }
 
 // The kernels' dynamic shared memory (tile_dyn_bytes of their tile width).
@@ -919,9 +887,9 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     // march direction: alternating between neighbouring row tiles, and
     // reversed on every other step
     const int dir = ((blockIdx.y & 1) ? -1 : 1) * (a.flip ? -1 : 1);
-    __shared__ TileSmem<T, TX> sm;
+    __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
-    d2q9_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, blockIdx.x * TX, y0,
+    run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, blockIdx.x * TX, y0,
                            min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + blockIdx.x, bph);
 }
 
@@ -949,9 +917,9 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     a.eqs_src = c.eqs + parity;
     a.eqs_dst = c.eqs + (parity ^ 1);
     a.eqs_target = c.eqs + 2;
-    __shared__ TileSmem<T, TX> sm;
+    __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
-    d2q9_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, t.x0, t.y0, t.yend,
+    run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, t.x0, t.y0, t.yend,
                            parity ? -t.dir : t.dir, blockIdx.x, bph);
 }
 
@@ -1152,10 +1120,10 @@ __global__ void __launch_bounds__((Occ<T, PASS_STATE, TX>::nth), (Occ<T, PASS_ST
                 f1[n] = T(NAN);
             }
     };
-    __shared__ TileSmem<T, TX> sm;
+    __shared__ typename SmemOf<T, TX>::type sm;
     // the stages' mbarriers (bulk-copy staging), their next parities
     unsigned bph = 0;
-    if (SEGK) {
+    if constexpr (SEGK) {
         if (lin == 0) {
             mbar_init(&sm.bar[0], 1);
             mbar_init(&sm.bar[1], 1);
@@ -1237,16 +1205,16 @@ __global__ void __launch_bounds__((Occ<T, PASS_STATE, TX>::nth), (Occ<T, PASS_ST
         const bool seg = SEGK && seg_ok<T, TX>(P.nx, a.f_src, a.g_src, a.S);
         if (k == pa.diag_k) {
             if (seg)
-                d2q9_tile<T, TX, PASS_STATE | PASS_DIAG, false, SEGK>(sm, dyn, P, a, t.x0, t.y0,
+                run_tile<T, TX, PASS_STATE | PASS_DIAG, false, SEGK>(sm, dyn, P, a, t.x0, t.y0,
                                                                        t.yend, dir, ti, bph);
             else
-                d2q9_tile<T, TX, PASS_STATE | PASS_DIAG, false>(sm, dyn, P, a, t.x0, t.y0, t.yend,
+                run_tile<T, TX, PASS_STATE | PASS_DIAG, false>(sm, dyn, P, a, t.x0, t.y0, t.yend,
                                                                  dir, ti, bph);
         } else if (seg) {
-            d2q9_tile<T, TX, PASS_STATE, false, SEGK>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti,
+            run_tile<T, TX, PASS_STATE, false, SEGK>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti,
                                                       bph);
         } else {
-            d2q9_tile<T, TX, PASS_STATE, false>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph);
+            run_tile<T, TX, PASS_STATE, false>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph);
         }
         // every thread read s_stepdone at this pair's top, before the tile's
         // barriers: thread 0 folds in what lane 31 saw, for the next pair, and
@@ -1257,7 +1225,9 @@ __global__ void __launch_bounds__((Occ<T, PASS_STATE, TX>::nth), (Occ<T, PASS_ST
             s_stop[it & 1] = err_seen;
         }
         __syncthreads();  // every output of the step (and its partial) is stored
-        if (SEGK && sm.stage_timeout) {
+        bool stage_late = false;
+        if constexpr (SEGK) stage_late = sm.stage_timeout != 0;
+        if (stage_late) {
             // a stage's copies did not land in time: the tile is invalid; the
             // error word stops the other CTAs
             if (lin == 0) {
