@@ -85,5 +85,20 @@ __device__ __forceinline__ Nb make_nb(int x, int y, int z, int nx, int ny, int n
     return b;
 }
 
+// mu = psi'(phi) - kappa lap(phi) of an FP64 field at a node (Eq. chemical_potencial)
+template <class P>
+__device__ __forceinline__ double mu_of_field(const P &prm, const double *__restrict__ phi,
+                                              const Nb &b, double c)
+{
+    double fa = 0.0, ed = 0.0;
+#pragma unroll
+    for (int i = 1; i < 19; ++i) {
+        const double d = __ldg(phi + b.at(c3x(i), c3y(i), c3z(i))) - c;
+        if (i <= 6) fa += d; else ed += d;
+    }
+    const double lap = (1.0 / 3.0) * fa + (1.0 / 6.0) * ed;
+    return 4.0 * prm.beta * (c - prm.phil) * (c - prm.phiv) * (c - prm.phibar) - prm.kappa * lap;
+}
+
 }  // namespace d3
 }  // namespace wblbm

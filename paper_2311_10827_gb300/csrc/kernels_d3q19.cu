@@ -335,44 +335,32 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
 
 // ------------------------------------------------------------ initial state
 
-// mu0 = psi'(phi0) - kappa lap(phi0) in FP64
-__global__ void d3q19_init_mu(const StepParams<double> P, const double *__restrict__ phi,
-                              double *__restrict__ mu)
-{
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (size_t)P.N) return;
-    const int nx = P.nx, ny = P.ny, nz = P.nz;
-    const int x = (int)(n % nx), y = (int)((n / nx) % ny), z = (int)(n / ((size_t)nx * ny));
-    const Nb b = make_nb(x, y, z, nx, ny, nz);
-    const double c = phi[n];
-    double fa = 0.0, ed = 0.0;
-    for (int i = 1; i < 19; ++i) {
-        const double d = phi[b.at(c3x(i), c3y(i), c3z(i))] - c;
-        if (i <= 6) fa += d; else ed += d;
-    }
-    const double lap = (1.0 / 3.0) * fa + (1.0 / 6.0) * ed;
-    mu[n] = 4.0 * P.beta * (c - P.phil) * (c - P.phiv) * (c - P.phibar) - P.kappa * lap;
-}
-
+// f_i(x, 0) = f_i^eq(phi0(x), mu0(x)) with mu0 in FP64, the value of node x
+// stored at x - c_i; g = 0, S = 0.  As in 2D each node forms its two distinct
+// values w_i alpha mu once and stores them 18 times, because the FP64 pipe
+// bounds the kernel (64^3 FP32: 60 -> 34 us against a second pass that formed
+// them where they are stored).
 template <typename T>
-__global__ void d3q19_init_pop(const StepParams<double> P, const double *__restrict__ phi,
-                               const double *__restrict__ mu, T *__restrict__ f, T *__restrict__ g,
-                               T *__restrict__ S)
+__global__ void __launch_bounds__(256)
+    d3q19_init_k(const StepParams<double> P, const double *__restrict__ phi, T *__restrict__ f,
+                 T *__restrict__ g, T *__restrict__ S)
 {
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (size_t)P.N) return;
-    const size_t N = (size_t)P.N;
-    const int nx = P.nx, ny = P.ny, nz = P.nz;
-    const int x = (int)(n % nx), y = (int)((n / nx) % ny), z = (int)(n / ((size_t)nx * ny));
-    const Nb b = make_nb(x, y, z, nx, ny, nz);
-    for (int i = 0; i < 19; ++i) {
-        const unsigned m = b.at(c3x(i), c3y(i), c3z(i));  // f_i(x,0) stored at x - c_i
-        const double am = P.alpha * mu[m];
-        const double fe = i == 0 ? phi[m] - (1.0 - w3(0)) * am : w3(i) * am;
-        f[i * N + n] = (T)fe;
-        g[i * N + n] = T(0);
-        if (sizeof(T) == 4 && i == 0) f[19 * N + n] = (T)(fe - (double)(T)fe);
-    }
+    const unsigned N = (unsigned)P.N, n = blockIdx.x * 256u + threadIdx.x;
+    if (n >= N) return;
+    const unsigned nx = P.nx, ny = P.ny;
+    const unsigned r = n / nx;
+    const Nb b = make_nb((int)(n - r * nx), (int)(r % ny), (int)(r / ny), P.nx, P.ny, P.nz);
+    const double c = __ldg(phi + n);
+    const double am = P.alpha * mu_of_field(P, phi, b, c);
+    const double f0 = c - (1.0 - w3(0)) * am;
+    f[n] = (T)f0;
+    if (sizeof(T) == 4) f[19u * N + n] = (T)(f0 - (double)(T)f0);
+    const T va = (T)(w3(1) * am), ve = (T)(w3(7) * am);
+#pragma unroll
+    for (int i = 1; i < 19; ++i)
+        f[i * N + b.at(-c3x(i), -c3y(i), -c3z(i))] = i <= 6 ? va : ve;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) g[i * N + n] = T(0);
     S[n] = T(0);
 }
 
@@ -494,24 +482,15 @@ cudaError_t d3q19_pass(int precision, int pass, const void *params, const PassAr
                           : pass3_t<float>(pass, params, a, s, phi_work, st);
 }
 
-cudaError_t d3q19_init_mu_fp64(const void *params, const double *phi0, double *mu, cudaStream_t st)
+cudaError_t d3q19_init(int precision, const void *params, const double *phi0, void *f, void *g,
+                       void *S, cudaStream_t st)
 {
     const StepParams<double> &P = *static_cast<const StepParams<double> *>(params);
     const unsigned nb = (unsigned)((P.N + 255) / 256);
-    d3q19_init_mu<<<nb, 256, 0, st>>>(P, phi0, mu);
-    return cudaGetLastError();
-}
-
-cudaError_t d3q19_init(int precision, const void *params, const double *phi0, double *mu_tmp,
-                       void *f, void *g, void *S, cudaStream_t st)
-{
-    const StepParams<double> &P = *static_cast<const StepParams<double> *>(params);
-    const unsigned nb = (unsigned)((P.N + 255) / 256);
-    d3q19_init_mu<<<nb, 256, 0, st>>>(P, phi0, mu_tmp);
     if (precision == 0)
-        d3q19_init_pop<double><<<nb, 256, 0, st>>>(P, phi0, mu_tmp, (double *)f, (double *)g, (double *)S);
+        d3q19_init_k<double><<<nb, 256, 0, st>>>(P, phi0, (double *)f, (double *)g, (double *)S);
     else
-        d3q19_init_pop<float><<<nb, 256, 0, st>>>(P, phi0, mu_tmp, (float *)f, (float *)g, (float *)S);
+        d3q19_init_k<float><<<nb, 256, 0, st>>>(P, phi0, (float *)f, (float *)g, (float *)S);
     return cudaGetLastError();
 }
 

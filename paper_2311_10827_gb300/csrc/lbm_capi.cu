@@ -48,7 +48,8 @@ struct lbm_ctx {
     int nsm;
     void *f[2], *g[2], *S;
     int cur;     // f[cur], g[cur] hold the current state
-    double *aux;         // N doubles (initial chemical potential)
+    double *aux;         // N doubles: scratch of the offset initial condition and, for D2Q9,
+                         // of the batch tuner (else null)
     void *phiw;          // D3Q19: phi field written by the first pass of a step
     double *stage;       // (3 + D) N doubles, host moment staging (lazy)
     DiagPartial *partials;
@@ -455,7 +456,7 @@ int create_impl(const lbm_grid *grid, int lattice, const lbm_params *params, voi
         dalloc(&ctx->g[1], ctx->gbytes);
         dalloc(&ctx->S, N * ssz);
     }
-    dalloc((void **)&ctx->aux, N * sizeof(double));
+    if (ctx->codec >= 0 || lattice == LBM_D2Q9) dalloc((void **)&ctx->aux, N * sizeof(double));
     if (lattice == LBM_D3Q19) dalloc(&ctx->phiw, N * ssz);
     if (ctx->codec >= 0) dalloc((void **)&ctx->scw, 4 * sizeof(float));
     dalloc((void **)&ctx->eqs, 4 * sizeof(float));
@@ -513,14 +514,16 @@ int lbm_init_phi(lbm_ctx *ctx, const double *phi, int on_device)
         e = cudaMemcpyAsync(ctx->scw, OFFSET_INITIAL_SCALES, sizeof OFFSET_INITIAL_SCALES,
                             cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess)
-            e = d3q19_off_init(ctx->codec, &ctx->pd, &ctx->pf, src, ctx->aux, ctx->f[0],
-                               ctx->g[0], ctx->S, OFFSET_INITIAL_SCALES, ctx->stream);
+            // (the other g buffer, 38 N bytes, is free here: scratch)
+            e = d3q19_off_init(ctx->codec, &ctx->pd, &ctx->pf, src, ctx->aux,
+                               static_cast<double *>(ctx->g[1]), ctx->f[0], ctx->g[0], ctx->S,
+                               OFFSET_INITIAL_SCALES, ctx->stream);
     } else if (ctx->lattice == LBM_D3Q19) {
-        e = d3q19_init(ctx->prm.precision, &ctx->pd, src, ctx->aux, ctx->f[0], ctx->g[0],
-                       ctx->S, ctx->stream);
+        e = d3q19_init(ctx->prm.precision, &ctx->pd, src, ctx->f[0], ctx->g[0], ctx->S,
+                       ctx->stream);
     } else {
-        e = d2q9_init(ctx->prm.precision, &ctx->pd, src, ctx->aux, ctx->f[0], ctx->g[0],
-                      ctx->S, ctx->stream);
+        e = d2q9_init(ctx->prm.precision, &ctx->pd, src, ctx->f[0], ctx->g[0], ctx->S,
+                      ctx->stream);
     }
     // a host array is read until the upload completes: return after it
     if (e == cudaSuccess && !on_device) e = cudaEventSynchronize(ctx->up_ev);

@@ -222,8 +222,8 @@ struct PersistArgs {
 cudaError_t d2q9_batch_persist(int precision, int width, bool seg, const PersistArgs &pa,
                                int nctas, cudaStream_t st);
 int d2q9_batch_persist_ctas_per_sm(int precision, int width, bool seg);
-cudaError_t d2q9_init(int precision, const void *params, const double *phi0, double *mu_tmp,
-                      void *f, void *g, void *S, cudaStream_t st);
+cudaError_t d2q9_init(int precision, const void *params, const double *phi0, void *f, void *g,
+                      void *S, cudaStream_t st);
 cudaError_t d2q9_get_state(int precision, int nx, int ny, const void *f, const void *g,
                            const void *S, const float *eqs, double *fo, double *go, double *So,
                            cudaStream_t st);
@@ -239,16 +239,13 @@ int d3q19_ctas_per_sm(int precision);
 int d3q19_off_ctas_per_sm(int codec);
 cudaError_t d3q19_pass(int precision, int pass, const void *params, const PassArgs &a,
                        const LaunchShape &s, void *phi_work, cudaStream_t st);
-cudaError_t d3q19_init(int precision, const void *params, const double *phi0, double *mu_tmp,
-                       void *f, void *g, void *S, cudaStream_t st);
+cudaError_t d3q19_init(int precision, const void *params, const double *phi0, void *f, void *g,
+                       void *S, cudaStream_t st);
 cudaError_t d3q19_get_state(int precision, const void *params, const void *f, const void *g,
                             const void *S, const float *eqs, double *fo, double *go, double *So,
                             cudaStream_t st);
 cudaError_t d3q19_set_state(int precision, const void *params, void *f, void *g, void *S,
                             const double *fi, const double *gi, const double *Si, cudaStream_t st);
-
-// FP64 chemical potential of an initial phi field (Eq. chemical_potencial)
-cudaError_t d3q19_init_mu_fp64(const void *params, const double *phi0, double *mu, cudaStream_t st);
 
 // Populations stored as 16-bit offsets from their equilibria
 // (kernels_d3q19_off.cu).  One parity of the state: the f buffer holds the
@@ -274,9 +271,10 @@ __host__ __device__ inline OffsetLayout offset_layout(long long N, int Q, int D)
 cudaError_t d3q19_off_pass(int codec, int pass, const void *params32, const PassArgs &a,
                            const LaunchShape &s, void *phi_work, const float *target,
                            cudaStream_t st);
+// tmp_a, tmp_e: scratch of N doubles each
 cudaError_t d3q19_off_init(int codec, const void *params64, const void *params32,
-                           const double *phi0, double *mu_tmp, void *f, void *g, void *S,
-                           const float *target_host, cudaStream_t st);
+                           const double *phi0, double *tmp_a, double *tmp_e, void *f, void *g,
+                           void *S, const float *target_host, cudaStream_t st);
 cudaError_t d3q19_off_get_state(int codec, const void *params32, const void *f, const void *g,
                                 const void *S, double *fo, double *go, double *So, cudaStream_t st);
 cudaError_t d3q19_off_set_state(int codec, const void *params32, void *f, void *g, void *S,
