@@ -28,6 +28,7 @@
 #include <float.h>
 #include <math.h>
 
+#include "launch.cuh"
 #include "lbm_internal.h"
 
 namespace wblbm {
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
                           R *__restrict__ lphi, R *__restrict__ lmu, R *__restrict__ lgphi,
                           R *__restrict__ lgmu, double *dpar)
 {
+    pdl_wait();
     const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned N = geo.N;
     constexpr R IC = R(1.0 / CS2A);
@@ -298,6 +300,7 @@ __global__ void __launch_bounds__(AMX *AMY)
                const R *__restrict__ lgmu, R *__restrict__ lpt_out, double *dpar)
 {
     __shared__ R smu[AHX * AHY];
+    pdl_wait();
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * AMX, y0 = blockIdx.y * AMY;
     for (int q = tid; q < AHX * AHY; q += AMX * AMY) {
@@ -373,11 +376,12 @@ void adj_step_t(const StepParams<R> &P, AdjGeom geo, const R *f, const R *g, con
     const unsigned N = geo.N;
     R *lphi = work, *lmu = work + N, *lgphi = work + 2 * (size_t)N, *lgmu = work + 4 * (size_t)N;
     const unsigned nb = (N + 255) / 256;
-    adj_local<R><<<nb, 256, 0, st>>>(P, geo, f, g, phi, mu, p, u, lf_in, lpt, lg_in, lS_in,
-                                     lf_out, lg_out, lS_out, lphi, lmu, lgphi, lgmu, dpar);
+    launch_pdl(adj_local<R>, nb, 256, 0, st, P, geo, f, g, phi, mu, p, u, lf_in, lpt, lg_in, lS_in,
+               lf_out, lg_out, lS_out, lphi, lmu, lgphi, lgmu, dpar);
     // lpt is read (gathered) by adj_local above and rewritten here
     const dim3 tiles((geo.nx + AMX - 1) / AMX, (geo.ny + AMY - 1) / AMY);
-    adj_mu_phi<R><<<tiles, AMX * AMY, 0, st>>>(P, geo, phi, lphi, lgphi, lmu, lgmu, lpt, dpar);
+    launch_pdl(adj_mu_phi<R>, tiles, AMX * AMY, 0, st, P, geo, phi, lphi, lgphi, lmu, lgmu, lpt,
+               dpar);
 }
 
 template <typename R>

@@ -36,6 +36,7 @@
 #include <float.h>
 #include <math.h>
 
+#include "launch.cuh"
 #include "lbm_internal.h"
 
 namespace wblbm {
@@ -883,6 +884,7 @@ template <typename T, int TX, int PASS>
 __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ctas))
     d2q9_pass_kernel(const StepParams<T> P, PassArgs a, int rows)
 {
+    pdl_wait();
     const int y0 = blockIdx.y * rows;
     // march direction: alternating between neighbouring row tiles, and
     // reversed on every other step
@@ -901,6 +903,7 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     d2q9_batch_kernel(const BatchCase *__restrict__ cases, const BatchTile *__restrict__ tiles,
                       int parity, DiagPartial *partials)
 {
+    pdl_wait();
     const BatchTile t = tiles[blockIdx.x];
     const BatchCase &c = cases[t.c];
     const StepParams<T> P = *reinterpret_cast<const StepParams<T> *>(
@@ -1417,8 +1420,7 @@ cudaError_t launch_pass(const void *params, const PassArgs &a, const LaunchShape
     const StepParams<T> &P = *static_cast<const StepParams<T> *>(params);
     constexpr int dyn = tile_dyn_bytes<T, TXW>();
     dim3 grid(s.grid_x, s.grid_y), block(TXW, TYB);
-    d2q9_pass_kernel<T, TXW, PASS><<<grid, block, dyn, st>>>(P, a, s.rows);
-    return cudaGetLastError();
+    return launch_pdl(d2q9_pass_kernel<T, TXW, PASS>, grid, block, dyn, st, P, a, s.rows);
 }
 
 template <typename T>
@@ -1445,11 +1447,10 @@ cudaError_t launch_batch_t(const BatchCase *cases, const BatchTile *tiles, int n
     dim3 block(TX, TYB);
     constexpr int dyn = tile_dyn_bytes<T, TX>();
     if (partials)
-        d2q9_batch_kernel<T, TX, PASS_STATE | PASS_DIAG>
-            <<<ntiles, block, dyn, st>>>(cases, tiles, parity, partials);
-    else
-        d2q9_batch_kernel<T, TX, PASS_STATE><<<ntiles, block, dyn, st>>>(cases, tiles, parity, nullptr);
-    return cudaGetLastError();
+        return launch_pdl(d2q9_batch_kernel<T, TX, PASS_STATE | PASS_DIAG>, ntiles, block, dyn, st,
+                          cases, tiles, parity, partials);
+    return launch_pdl(d2q9_batch_kernel<T, TX, PASS_STATE>, ntiles, block, dyn, st, cases, tiles,
+                      parity, (DiagPartial *)nullptr);
 }
 
 }  // namespace

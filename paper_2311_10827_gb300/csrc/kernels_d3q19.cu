@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include "d3q19_lattice.cuh"
+#include "launch.cuh"
 #include "lbm_internal.h"
 
 namespace wblbm {
@@ -31,6 +32,7 @@ template <typename T>
 __global__ void __launch_bounds__(PHI_TX)
     d3q19_phi_kernel(const StepParams<T> P, const T *__restrict__ f, T *__restrict__ phi)
 {
+    pdl_wait();
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const int x = blockIdx.x * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
     if (x >= nx) return;
@@ -56,6 +58,7 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
     __shared__ T phs[RP * PA];
     __shared__ T mus[RM * MA];
 
+    pdl_wait();
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
@@ -413,10 +416,12 @@ cudaError_t launch3(const void *params, const PassArgs &a, const LaunchShape &s,
 {
     const StepParams<T> &P = *static_cast<const StepParams<T> *>(params);
     const dim3 pg((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz);
-    d3q19_phi_kernel<T><<<pg, PHI_TX, 0, st>>>(P, static_cast<const T *>(a.f_src), static_cast<T *>(phi));
+    const cudaError_t e = launch_pdl(d3q19_phi_kernel<T>, pg, PHI_TX, 0, st, P,
+                                     static_cast<const T *>(a.f_src), static_cast<T *>(phi));
+    if (e != cudaSuccess) return e;
     dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TX3, TY3);
-    d3q19_pass_kernel<T, PASS><<<grid, block, 0, st>>>(P, a, static_cast<const T *>(phi), s.rows);
-    return cudaGetLastError();
+    return launch_pdl(d3q19_pass_kernel<T, PASS>, grid, block, 0, st, P, a,
+                      static_cast<const T *>(phi), s.rows);
 }
 
 template <typename T>

@@ -39,6 +39,7 @@
 #include <math.h>
 
 #include "d3q19_lattice.cuh"
+#include "launch.cuh"
 #include "lbm_internal.h"
 
 namespace wblbm {
@@ -88,6 +89,7 @@ template <class C>
 __global__ void __launch_bounds__(PHI_TX)
     d3q19_off_phi_kernel(const StepParams<float> P, const OffBuf src, float *__restrict__ phi)
 {
+    pdl_wait();
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const int x = blockIdx.x * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
     if (x >= nx) return;
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepPara
     __shared__ float4 qa[RQ * MA];
     __shared__ float2 qb[RQ * MA];
 
+    pdl_wait();
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
@@ -699,10 +702,11 @@ cudaError_t launch_off(const StepParams<float> &P, const PassArgs &a, const Laun
 {
     const OffBuf src = off_view(a.f_src, a.g_src, P.N), dst = off_view(a.f_dst, a.g_dst, P.N);
     const dim3 pg((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz);
-    d3q19_off_phi_kernel<C><<<pg, PHI_TX, 0, st>>>(P, src, phi);
+    const cudaError_t e = launch_pdl(d3q19_off_phi_kernel<C>, pg, PHI_TX, 0, st, P, src, phi);
+    if (e != cudaSuccess) return e;
     dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TX3, TY3);
-    d3q19_off_pass_kernel<C, PASS><<<grid, block, 0, st>>>(P, a, src, dst, target, phi, s.rows);
-    return cudaGetLastError();
+    return launch_pdl(d3q19_off_pass_kernel<C, PASS>, grid, block, 0, st, P, a, src, dst, target,
+                      phi, s.rows);
 }
 
 template <class C>
