@@ -51,6 +51,16 @@ struct CodecF16 {
     static constexpr unsigned short INF_BITS = 0x7c00;
     __device__ static float dec(unsigned short u) { return __half2float(__ushort_as_half(u)); }
     __device__ static unsigned short enc(float v) { return __half_as_ushort(__float2half_rn(v)); }
+    // two values in one word, the first in the low half
+    __device__ static float2 dec2(unsigned v)
+    {
+        return __half22float2(*reinterpret_cast<const __half2 *>(&v));
+    }
+    __device__ static unsigned enc2(float2 v)
+    {
+        const __half2 h = __float22half2_rn(v);
+        return *reinterpret_cast<const unsigned *>(&h);
+    }
 };
 struct CodecBF16 {
     static constexpr unsigned short INF_BITS = 0x7f80;
@@ -61,6 +71,15 @@ struct CodecBF16 {
     __device__ static unsigned short enc(float v)
     {
         return __bfloat16_as_ushort(__float2bfloat16_rn(v));
+    }
+    __device__ static float2 dec2(unsigned v)
+    {
+        return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+    }
+    __device__ static unsigned enc2(float2 v)
+    {
+        const __nv_bfloat162 h = __float22bfloat162_rn(v);
+        return *reinterpret_cast<const unsigned *>(&h);
     }
 };
 
@@ -125,34 +144,72 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 
 // ------------------------------------------------------------------ pass 2
 
-template <class C, int PASS>
-__global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepParams<float> P,
-                                                                  PassArgs a, const OffBuf src,
-                                                                  const OffBuf dst,
-                                                                  const float *__restrict__ target,
-                                                                  const float *__restrict__ phif,
-                                                                  int planes)
+// The paired FP32 datapath: two independent lanes per instruction, each
+// rounding as the scalar instruction does.  The lanes are the thread's two
+// nodes.
+__device__ __forceinline__ float2 f2(float s) { return make_float2(s, s); }
+__device__ __forceinline__ float2 add2(float2 x, float2 y) { return __fadd2_rn(x, y); }
+__device__ __forceinline__ float2 mul2(float2 x, float2 y) { return __fmul2_rn(x, y); }
+__device__ __forceinline__ float2 fma2(float2 x, float2 y, float2 z) { return __ffma2_rn(x, y, z); }
+// x - y as one multiply-add by -1 (the same single rounding)
+__device__ __forceinline__ float2 sub2(float2 x, float2 y) { return __ffma2_rn(y, f2(-1.0f), x); }
+__device__ __forceinline__ float2 neg2(float2 x) { return __fmul2_rn(x, f2(-1.0f)); }
+// sum_d c_d v_d of a velocity c (components 0, 1, -1; the first non-zero one may be -1)
+__device__ __forceinline__ float2 dot_c(int cx, int cy, int cz, float2 x, float2 y, float2 z)
+{
+    float2 s = cx ? (cx > 0 ? x : neg2(x)) : (cy ? (cy > 0 ? y : neg2(y)) : (cz > 0 ? z : neg2(z)));
+    if (cx && cy) s = cy > 0 ? add2(s, y) : sub2(s, y);
+    if ((cx || cy) && cz) s = cz > 0 ? add2(s, z) : sub2(s, z);
+    return s;
+}
+
+// What bounds this pass: instruction issue and the latency of the pulls.
+// Rebuilding 38 populations per node from their offsets took 1570 instructions
+// per node with one node per thread (256^3 FP16: 1.135 ms, issue slots 60% busy
+// at 16 warps per SM, DRAM 38%).  A thread owns two nodes adjacent in x
+// instead: their arithmetic runs on the paired FP32 datapath (the same
+// roundings in the same order), 16-bit values of a pair are loaded and stored
+// as one 32-bit word where their alignment allows (every store, and the pulls
+// without an x component), and the plane offsets of the asynchronous copies are
+// formed once per march: 1030 instructions per node, 160^3 279 -> 233 us, whole
+// 256^3 runs 1.40 -> 1.17 ms per step.  EVEN: rows of an even number of nodes,
+// which is what those words need; other grids load and store single values.
+// Three CTAs of 128 threads per SM at 168 registers; four spill (83 ms against
+// 47 ms per 40 steps at 256^3).  Measured and not kept, all bit-identical: the
+// pulls staged a plane ahead in shared memory by 4-byte asynchronous copies
+// (333 us: the load/store units take one word per thread at a time), the next
+// plane's pulls in registers during the collisions at two CTAs per SM (238 us),
+// or while its mu is formed (264 us: they spill).
+constexpr int TXP = 16;           // pairs per row of a tile: TX3 = 2 TXP nodes
+static_assert(TX3 == 2 * TXP, "tile width");
+constexpr int OFF_NT = TXP * TY3;  // threads per CTA
+template <class C, int PASS, bool EVEN>
+__global__ void __launch_bounds__(OFF_NT, 3)
+    d3q19_off_pass_kernel(const StepParams<float> P, PassArgs a, const OffBuf src, const OffBuf dst,
+                          const float *__restrict__ target, const float *__restrict__ phif,
+                          int planes)
 {
     constexpr int PX = TX3 + 4, PY = TY3 + 4, PA = PX * PY;  // phi plane (halo 2)
-    constexpr int MX = TX3 + 2, MY = TY3 + 2, MA = MX * MY;  // mu / macro plane (halo 1)
-    constexpr int RP = 5, RM = 3, RQ = 3;
-    __shared__ float phs[RP * PA];
-    __shared__ float mus[RM * MA];
+    constexpr int MX = TX3 + 4, MY = TY3 + 2, MA = MX * MY;  // mu / macro plane (halo 1 used in
+                                                             // x of the 2 stored: even pairs)
+    constexpr int RP = 5, RM = 3;
+    constexpr int MW = TX3 + 2, MN = MW * MY;  // nodes of a mu / macro plane
+    __shared__ __align__(16) float phs[RP * PA];
+    __shared__ __align__(16) float mus[RM * MA];
     // the source macros of the plane two ahead, copied while a plane is updated
-    __shared__ float mraw[6 * MA];
-    // per source node: {alpha mu, A = 3p - 3/2 rho |u|^2, rho ux, rho uy} and
-    // {rho uz, 9 / (2 rho)}: g^eq_i = w_i (A + 3 c.j + (9/2)(c.j)^2 / rho)
-    __shared__ float4 qa[RQ * MA];
-    __shared__ float2 qb[RQ * MA];
+    __shared__ float mraw[6 * MN];
+    // per source node {alpha mu, A = 3p - 3/2 rho |u|^2, rho u_x, rho u_y, rho u_z, 9 / (2 rho)}:
+    // g^eq_i = w_i (A + 3 c.j + (9/2)(c.j)^2 / rho); ring of three planes per quantity
+    __shared__ __align__(16) float qs[6][RM * MA];
 
     pdl_wait();
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TXP + tx;
     const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
-    const int x = x0 + tx, y = y0 + ty;
-    const bool col_ok = x < nx && y < ny;
+    const int x = x0 + 2 * tx, y = y0 + ty;
+    const bool okA = x < nx && y < ny, okB = EVEN ? okA : (x + 1 < nx && y < ny);
     const unsigned plane = (unsigned)nx * ny;
     const float s_f = __ldg(src.sc), s_g = __ldg(src.sc + 1);
     const float t_f = __ldg(target), t_g = __ldg(target + 1);
@@ -162,29 +219,35 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepPara
         dst.sc[1] = t_g;
     }
 
-    auto pslot = [&](int zz) { return (zz - z0 + 2) % RP; };
-    auto mslot = [&](int zz) { return (zz - z0 + 1) % RM; };
-    auto qslot = [&](int zz) { return (zz - z0 + 1) % RQ; };
-
     // grids narrower than a tile plus halo wrap by division (uniform flags)
     const bool smx = nx < PX + 2, smy = ny < PY + 2, smz = nz < 8;
-    auto load_phi_plane = [&](int zz) {
-        float *d = phs + pslot(zz) * PA;
-        const unsigned zo = (unsigned)wrapc(zz, nz, smz) * plane;
-        for (int q = tid; q < PA; q += TX3 * TY3) {
-            const int lx = q % PX, ly = q / PX;
-            const unsigned xx = wrapc(x0 - 2 + lx, nx, smx), yy = wrapc(y0 - 2 + ly, ny, smy);
-            d[q] = phif[zo + yy * nx + xx];
-        }
-    };
-    // Eq. chemical_potencial with Eq. Laplace on D3Q19
-    auto mu_plane = [&](int zz) {
-        const float *pm = phs + pslot(zz - 1) * PA, *p0 = phs + pslot(zz) * PA,
-                    *pp = phs + pslot(zz + 1) * PA;
-        float *d = mus + mslot(zz) * MA;
-        for (int q = tid; q < MA; q += TX3 * TY3) {
-            const int lx = q % MX + 1, ly = q / MX + 1;
-            const int c = ly * PX + lx;
+    // this thread's elements of a phi plane and nodes of a mu / macro plane:
+    // ring index and in-plane offset in the grid (nodes past the halo repeat)
+    constexpr int KP = (PA + OFF_NT - 1) / OFF_NT, KM = (MN + OFF_NT - 1) / OFF_NT;
+    unsigned poff[KP], moff[KM];
+    int mring[KM];  // index in a stored plane (row stride MX, x halo 2)
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+        const int q = tid + k * OFF_NT;
+        poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
+    }
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+        const int q = tid + k * OFF_NT;
+        moff[k] = (unsigned)wrapc(y0 - 1 + q / MW, ny, smy) * nx + wrapc(x0 - 1 + q % MW, nx, smx);
+        mring[k] = q / MW * MX + q % MW + 1;
+    }
+    // ring slots of plane z0 + d: phi (d + 2) mod 5, mu and macros (d + 1) mod 3
+    auto wrapr = [](int v, int n) { return v >= n ? v - n : v; };
+    // Eq. chemical_potencial with Eq. Laplace on D3Q19, from the phi slots of the
+    // planes below, at and above into mu slot sm
+    auto mu_plane = [&](int s_m, int s_0, int s_p, int sm) {
+        const float *pm = phs + s_m * PA, *p0 = phs + s_0 * PA, *pp = phs + s_p * PA;
+        float *d = mus + sm * MA;
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+            if (tid + k * OFF_NT >= MN) break;
+            const int c = mring[k] + PX;  // one phi row further (halo 2 against 1)
             const float v = p0[c];
             const float fa = (p0[c + 1] - v) + (p0[c - 1] - v) + (p0[c + PX] - v) +
                              (p0[c - PX] - v) + (pp[c] - v) + (pm[c] - v);
@@ -194,55 +257,43 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepPara
                              ((pp[c + PX] - v) + (pp[c - PX] - v) + (pm[c + PX] - v) +
                               (pm[c - PX] - v));
             const float lap = (1.0f / 3.0f) * fa + (1.0f / 6.0f) * ed;
-            d[q] = 4.0f * P.beta * (v - P.phil) * (v - P.phiv) * (v - P.phibar) - P.kappa * lap;
+            d[mring[k]] = 4.0f * P.beta * (v - P.phil) * (v - P.phiv) * (v - P.phibar) - P.kappa * lap;
         }
     };
-    // equilibrium data of the source state's macros (ph, mu, p, u) at item q
-    // of a macro plane (tile + 1 halo)
-    auto put_macros = [&](int slot, int q, const float m6[6]) {
+    // equilibrium data of the source state's macros (phi, mu, p, u) at ring index r of slot sm
+    auto put_macros = [&](int sm, int r, const float m6[6]) {
         const float rho = P.rhov + (m6[0] - P.phiv) * P.drho;
-        qa[slot * MA + q] = make_float4(P.alpha * m6[1],
-                                        3.0f * m6[2] - 1.5f * rho * (m6[3] * m6[3] + m6[4] * m6[4] + m6[5] * m6[5]),
-                                        rho * m6[3], rho * m6[4]);
-        qb[slot * MA + q] = make_float2(rho * m6[5], 4.5f / rho);
-    };
-    auto macro_node = [&](int zz, int q) {
-        const unsigned m = (unsigned)wrapc(zz, nz, smz) * plane +
-                           (unsigned)wrapc(y0 - 1 + q / MX, ny, smy) * nx + wrapc(x0 - 1 + q % MX, nx, smx);
-        return m;
-    };
-    auto macro_plane = [&](int zz) {
-        for (int q = tid; q < MA; q += TX3 * TY3) {
-            const unsigned m = macro_node(zz, q);
-            float m6[6];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) m6[k] = __ldg(src.M + k * N + m);
-            put_macros(qslot(zz), q, m6);
-        }
-    };
-    auto grad3 = [&](const float *m, const float *c0, const float *p, int c, int SX, float out[3]) {
-        out[0] = (1.0f / 6.0f) * (c0[c + 1] - c0[c - 1]) +
-                 (1.0f / 12.0f) * ((c0[c + SX + 1] - c0[c + SX - 1]) + (c0[c - SX + 1] - c0[c - SX - 1]) +
-                                   (p[c + 1] - p[c - 1]) + (m[c + 1] - m[c - 1]));
-        out[1] = (1.0f / 6.0f) * (c0[c + SX] - c0[c - SX]) +
-                 (1.0f / 12.0f) * ((c0[c + SX + 1] - c0[c - SX + 1]) + (c0[c + SX - 1] - c0[c - SX - 1]) +
-                                   (p[c + SX] - p[c - SX]) + (m[c + SX] - m[c - SX]));
-        out[2] = (1.0f / 6.0f) * (p[c] - m[c]) +
-                 (1.0f / 12.0f) * ((p[c + 1] - m[c + 1]) + (p[c - 1] - m[c - 1]) +
-                                   (p[c + SX] - m[c + SX]) + (p[c - SX] - m[c - SX]));
+        const int q = sm * MA + r;
+        qs[0][q] = P.alpha * m6[1];
+        qs[1][q] = 3.0f * m6[2] - 1.5f * rho * (m6[3] * m6[3] + m6[4] * m6[4] + m6[5] * m6[5]);
+        qs[2][q] = rho * m6[3];
+        qs[3][q] = rho * m6[4];
+        qs[4][q] = rho * m6[5];
+        qs[5][q] = 4.5f / rho;
     };
 
     double d_phi = 0.0, d_E = 0.0, d_u2 = 0.0, d_mumin = DBL_MAX, d_mumax = -DBL_MAX,
            d_bud = 0.0, d_bad = 0.0;
 
-    for (int q = 0; q < 5; ++q) load_phi_plane(z0 - 2 + q);
-    macro_plane(z0 - 1);
-    macro_plane(z0);
-    macro_plane(z0 + 1);
+    for (int d = 0; d < 5; ++d) {
+        const unsigned zo = (unsigned)wrapc(z0 - 2 + d, nz, smz) * plane;
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+            if (tid + k * OFF_NT < PA) phs[d * PA + tid + k * OFF_NT] = phif[zo + poff[k]];
+    }
+    for (int d = 0; d < 3; ++d) {
+        const unsigned zo = (unsigned)wrapc(z0 - 1 + d, nz, smz) * plane;
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+            if (tid + k * OFF_NT >= MN) break;
+            float m6[6];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) m6[c] = __ldg(src.M + (c * N + zo + moff[k]));
+            put_macros(d, mring[k], m6);
+        }
+    }
     __syncthreads();
-    mu_plane(z0 - 1);
-    mu_plane(z0);
-    mu_plane(z0 + 1);
+    for (int d = 0; d < 3; ++d) mu_plane(d, d + 1, d + 2, d);
     __syncthreads();
 
     // Plane zz + 3 of phi (into its ring slot) and the raw source macros of
@@ -252,191 +303,307 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepPara
     // (read) and zz+3 (being written); mu and macros zz-1..zz+1; once every
     // thread is past the update, macro plane zz+2 and mu plane zz+2 take the
     // slots of zz-1.
-    const unsigned xw = col_ok ? (unsigned)x : 0, yw = col_ok ? (unsigned)y : 0;
-    Nb b = make_nb(xw, yw, z0, nx, ny, nz);
+    const unsigned xw = okA ? (unsigned)x : 0, yw = okA ? (unsigned)y : 0;
+    Nb b = make_nb((int)xw, (int)yw, z0, nx, ny, nz);
+    const unsigned xB = okB ? xw + 1 : 0;                   // the second node's column
+    const unsigned xp2 = (unsigned)wrap1((int)xw + 2, nx);  // and its +x neighbour (nx >= 2)
+    const unsigned xpp = nx == 1 ? 0u : xp2;
+    int sp = 1, sq = 0;  // phi slot of plane zz - 1, mu / macro slot of plane zz - 1
     for (int zz = z0; zz < zend; ++zz) {
+        const int sp0 = wrapr(sp + 1, RP), spp = wrapr(sp + 2, RP);
+        const int sq0 = wrapr(sq + 1, RM), sqp = wrapr(sq + 2, RM);
         {
             const unsigned zo = (unsigned)wrapc(zz + 3, nz, smz) * plane;
-            float *d = phs + pslot(zz + 3) * PA;
-            for (int q = tid; q < PA; q += TX3 * TY3) {
-                const unsigned xx = wrapc(x0 - 2 + q % PX, nx, smx), yy = wrapc(y0 - 2 + q / PX, ny, smy);
-                cp_async4(d + q, phif + (zo + yy * nx + xx));
-            }
-            for (int q = tid; q < MA; q += TX3 * TY3) {
-                const unsigned m = macro_node(zz + 2, q);
+            float *d = phs + wrapr(sp + 4, RP) * PA + tid;
 #pragma unroll
-                for (int c = 0; c < 6; ++c) cp_async4(mraw + c * MA + q, src.M + ((size_t)c * N + m));
+            for (int k = 0; k < KP; ++k)
+                if (tid + k * OFF_NT < PA) cp_async4(d + k * OFF_NT, phif + (zo + poff[k]));
+            const unsigned zm = (unsigned)wrapc(zz + 2, nz, smz) * plane;
+#pragma unroll
+            for (int k = 0; k < KM; ++k) {
+                if (tid + k * OFF_NT >= MN) break;
+                const float *m = src.M + (zm + moff[k]);
+#pragma unroll
+                for (int c = 0; c < 6; ++c)
+                    cp_async4(mraw + c * MN + tid + k * OFF_NT, m + (size_t)c * N);
             }
             cp_commit();
         }
-        if (col_ok) {
+        if (okA) {
         nb_plane(b, zz, nx, ny, nz);
-        const unsigned n = b.at(0, 0, 0);
-        // the two 16-bit offsets of direction i share one register
-        unsigned hk[19];
+        const unsigned row = b.zs[1] + b.ys[1], n = row + xw;
+        // the offsets of the two nodes share one register (the first in the low half)
+        unsigned hp[19], kp[19];
+        auto pull = [&](const unsigned short *v, int i) -> unsigned {
+            const unsigned r = i * N + b.zs[1 - c3z(i)] + b.ys[1 - c3y(i)];
+            if (c3x(i) == 0 && EVEN) return __ldg(reinterpret_cast<const unsigned *>(v + (r + xw)));
+            const unsigned ca = c3x(i) > 0 ? b.xs[0] : (c3x(i) < 0 ? b.xs[2] : xw);
+            const unsigned cb = c3x(i) > 0 ? xw : (c3x(i) < 0 ? xpp : xB);
+            return (unsigned)__ldg(v + (r + ca)) | ((unsigned)__ldg(v + (r + cb)) << 16);
+        };
 #pragma unroll
         for (int i = 0; i < 19; ++i) {
-            const unsigned s = b.at(-c3x(i), -c3y(i), -c3z(i));
-            hk[i] = (unsigned)__ldg(src.h + (i * N + s)) | ((unsigned)__ldg(src.k + (i * N + s)) << 16);
+            hp[i] = pull(src.h, i);
+            kp[i] = pull(src.k, i);
         }
-        auto hr = [&](int i) { return (unsigned short)(hk[i] & 0xffffu); };
-        auto kr = [&](int i) { return (unsigned short)(hk[i] >> 16); };
-        float Sprev = 0.0f;
-        if (PASS & (PASS_STATE | PASS_DIAG)) Sprev = __ldcs(static_cast<const float *>(a.S) + n);
-        const float phi_hi = __ldg(src.M + n), p_own = __ldg(src.M + 2 * N + n);
+        // an FP32 value of each of the two nodes
+        auto own = [&](const float *v) -> float2 {
+            if (EVEN) return __ldg(reinterpret_cast<const float2 *>(v + n));
+            return make_float2(__ldg(v + n), __ldg(v + (row + xB)));
+        };
+        float2 Sprev = f2(0.0f);
+        if (PASS & (PASS_STATE | PASS_DIAG)) {
+            const float *S = static_cast<const float *>(a.S);
+            if (EVEN)
+                Sprev = __ldcs(reinterpret_cast<const float2 *>(S + n));
+            else
+                Sprev = make_float2(__ldcs(S + n), __ldcs(S + (row + xB)));
+        }
+        const float2 phi_hi = own(src.M), p_own = own(src.M + 2 * N);
 
         // populations after streaming, rebuilt from offsets and source macros
-        const int cq = (ty + 1) * MX + (tx + 1);
-        float fv[19], gv[19];
-        float flo;  // rest population minus its high word phi_hi
+        const int c0 = (ty + 1) * MX + 2 * tx + 2;  // ring index of the first node (even)
+        // the pair at ring index c, c + 1 of a plane (one 64-bit read where c is even)
+        auto pair_at = [&](const float *pl, int c, bool even) -> float2 {
+            if (even) return *reinterpret_cast<const float2 *>(pl + c);
+            return make_float2(pl[c], pl[c + 1]);
+        };
+        const float2 sf2 = f2(s_f), sg2 = f2(s_g);
+        float2 fv[19], gv[19];
+        float2 flo;  // rest population minus its high word phi_hi
         {
-            const float4 A0 = qa[qslot(zz) * MA + cq];
-            flo = -(2.0f / 3.0f) * A0.x + s_f * C::dec(hr(0));
-            gv[0] = (1.0f / 3.0f) * A0.y - 3.0f * p_own + s_g * C::dec(kr(0));
-            fv[0] = 0.0f;
+            const float2 ax = pair_at(qs[0] + sq0 * MA, c0, true);
+            const float2 ay = pair_at(qs[1] + sq0 * MA, c0, true);
+            flo = fma2(sf2, C::dec2(hp[0]), mul2(f2(-(2.0f / 3.0f)), ax));
+            gv[0] = fma2(sg2, C::dec2(kp[0]),
+                         fma2(f2(1.0f / 3.0f), ay, mul2(f2(-3.0f), p_own)));
         }
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
-            const int c = qslot(zz - c3z(i)) * MA + cq - c3y(i) * MX - c3x(i);
-            const float4 A = qa[c];
-            const float2 B = qb[c];
-            const float w = (float)w3(i);
-            fv[i] = w * A.x + s_f * C::dec(hr(i));
-            float cj = 0.0f;
-            if (c3x(i)) cj += (float)c3x(i) * A.z;
-            if (c3y(i)) cj += (float)c3y(i) * A.w;
-            if (c3z(i)) cj += (float)c3z(i) * B.x;
-            gv[i] = w * (A.y + cj * (3.0f + B.y * cj)) + s_g * C::dec(kr(i));
+            const int sl = c3z(i) > 0 ? sq : (c3z(i) < 0 ? sqp : sq0);
+            const int c = sl * MA + c0 - c3y(i) * MX - c3x(i);
+            constexpr float w1 = (float)w3(1), w7 = (float)w3(7);
+            const float2 w = f2(i <= 6 ? w1 : w7);
+            const bool ev = c3x(i) == 0;
+            fv[i] = fma2(w, pair_at(qs[0], c, ev), mul2(sf2, C::dec2(hp[i])));
+            float2 jx = f2(0.0f), jy = f2(0.0f), jz = f2(0.0f);
+            if (c3x(i)) jx = pair_at(qs[2], c, ev);
+            if (c3y(i)) jy = pair_at(qs[3], c, ev);
+            if (c3z(i)) jz = pair_at(qs[4], c, ev);
+            const float2 cj = dot_c(c3x(i), c3y(i), c3z(i), jx, jy, jz);
+            const float2 e = fma2(cj, fma2(pair_at(qs[5], c, ev), cj, f2(3.0f)),
+                                  pair_at(qs[1], c, ev));
+            gv[i] = fma2(sg2, C::dec2(kp[i]), mul2(w, e));
         }
 
-        float snz = 0.0f, sg = 0.0f;
+        float2 snz = add2(fv[1], fv[2]), sg = add2(gv[1], gv[2]);
 #pragma unroll
-        for (int i = 1; i < 19; i += 2) {
-            snz += fv[i] + fv[i + 1];
-            sg += gv[i] + gv[i + 1];
+        for (int i = 3; i < 19; i += 2) {
+            snz = add2(snz, add2(fv[i], fv[i + 1]));
+            sg = add2(sg, add2(gv[i], gv[i + 1]));
         }
         // phi = phi_hi + (flo + snz) as an exact two-sum: phi (FP32) + r
-        const float lo_sum = flo + snz;
-        const float phi = phi_hi + lo_sum;
-        const float bp = phi - phi_hi;
-        const float r = (phi_hi - (phi - bp)) + (lo_sum - bp);
+        const float2 lo_sum = add2(flo, snz);
+        const float2 phi = add2(phi_hi, lo_sum);
+        const float2 bp = sub2(phi, phi_hi);
+        const float2 r = add2(sub2(phi_hi, sub2(phi, bp)), sub2(lo_sum, bp));
 
-        const int cp = (ty + 2) * PX + (tx + 2), cm = cq;
-        const float *mz = mus + mslot(zz) * MA;
-        const float mu = mz[cm];
-        float gp[3], gm[3];
-        grad3(phs + pslot(zz - 1) * PA, phs + pslot(zz) * PA, phs + pslot(zz + 1) * PA, cp, PX, gp);
-        grad3(mus + mslot(zz - 1) * MA, mz, mus + mslot(zz + 1) * MA, cm, MX, gm);
+        // Eq. gradient on D3Q19: (1/6) face differences + (1/12) edge differences
+        auto grad3 = [&](const float *m, const float *z, const float *p, int c, float2 out[3]) {
+            const int SX = PX;  // both rings have the same row stride
+            const float2 xe = pair_at(z, c + 1, false), xw_ = pair_at(z, c - 1, false);
+            const float2 yn = pair_at(z, c + SX, true), ys = pair_at(z, c - SX, true);
+            const float2 pc = pair_at(p, c, true), mc = pair_at(m, c, true);
+            const float2 ne = pair_at(z, c + SX + 1, false), nw = pair_at(z, c + SX - 1, false);
+            const float2 se = pair_at(z, c - SX + 1, false), sw = pair_at(z, c - SX - 1, false);
+            const float2 pe = pair_at(p, c + 1, false), pw = pair_at(p, c - 1, false);
+            const float2 me = pair_at(m, c + 1, false), mw = pair_at(m, c - 1, false);
+            const float2 pn = pair_at(p, c + SX, true), ps = pair_at(p, c - SX, true);
+            const float2 mn = pair_at(m, c + SX, true), ms = pair_at(m, c - SX, true);
+            const float2 k6 = f2(1.0f / 6.0f), k12 = f2(1.0f / 12.0f);
+            out[0] = fma2(k6, sub2(xe, xw_),
+                          mul2(k12, add2(add2(add2(sub2(ne, nw), sub2(se, sw)), sub2(pe, pw)),
+                                         sub2(me, mw))));
+            out[1] = fma2(k6, sub2(yn, ys),
+                          mul2(k12, add2(add2(add2(sub2(ne, se), sub2(nw, sw)), sub2(pn, ps)),
+                                         sub2(mn, ms))));
+            out[2] = fma2(k6, sub2(pc, mc),
+                          mul2(k12, add2(add2(add2(sub2(pe, me), sub2(pw, mw)), sub2(pn, mn)),
+                                         sub2(ps, ms))));
+        };
+        const int cp = (ty + 2) * PX + 2 * tx + 2;
+        const float *m0 = mus + sq0 * MA, *mm = mus + sq * MA, *mp = mus + sqp * MA;
+        const float2 mu = pair_at(m0, c0, true);
+        float2 gp[3], gm[3];
+        grad3(phs + sp * PA, phs + sp0 * PA, phs + spp * PA, cp, gp);
+        grad3(mm, m0, mp, c0, gm);
 
-        float F[3], gr[3], u[3];
-        const float dphi = phi - P.phiv;
-        const float rho = P.rhov + dphi * P.drho;
-        const float nu = P.nuv + dphi * P.dnu;
-        const float inv_rho = __fdividef(1.0f, rho);
-        const float itg = __fdividef(1.0f, 0.5f + 3.0f * nu);
-        float j3[3] = {0.0f, 0.0f, 0.0f};
+        float2 F[3], gr[3], u[3];
+        const float2 dphi = sub2(phi, f2(P.phiv));
+        const float2 rho = fma2(dphi, f2(P.drho), f2(P.rhov));
+        const float2 nu = fma2(dphi, f2(P.dnu), f2(P.nuv));
+        const float2 inv_rho = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+        const float2 tg = fma2(f2(3.0f), nu, f2(0.5f));
+        const float2 itg = make_float2(__fdividef(1.0f, tg.x), __fdividef(1.0f, tg.y));
+        float2 j3[3] = {f2(0.0f), f2(0.0f), f2(0.0f)};
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
-            if (c3x(i)) j3[0] += (float)c3x(i) * gv[i];
-            if (c3y(i)) j3[1] += (float)c3y(i) * gv[i];
-            if (c3z(i)) j3[2] += (float)c3z(i) * gv[i];
+            if (c3x(i)) j3[0] = c3x(i) > 0 ? add2(j3[0], gv[i]) : sub2(j3[0], gv[i]);
+            if (c3y(i)) j3[1] = c3y(i) > 0 ? add2(j3[1], gv[i]) : sub2(j3[1], gv[i]);
+            if (c3z(i)) j3[2] = c3z(i) > 0 ? add2(j3[2], gv[i]) : sub2(j3[2], gv[i]);
         }
-        float ugr = 0.0f, uu = 0.0f, S = 0.0f;
+        float2 ugr = f2(0.0f), uu = f2(0.0f), S = f2(0.0f);
+        const float2 mphi = neg2(phi);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            F[d] = -phi * gm[d] + P.G[d];
-            gr[d] = P.drho * gp[d];
-            u[d] = (j3[d] + 0.5f * F[d]) * inv_rho;
-            ugr += u[d] * gr[d];
-            uu += u[d] * u[d];
-            S += u[d] * gp[d];
+            F[d] = fma2(mphi, gm[d], f2(P.G[d]));
+            gr[d] = mul2(f2(P.drho), gp[d]);
+            u[d] = mul2(fma2(f2(0.5f), F[d], j3[d]), inv_rho);
+            ugr = fma2(u[d], gr[d], ugr);
+            uu = fma2(u[d], u[d], uu);
+            S = fma2(u[d], gp[d], S);
         }
-        const float p = 0.5f * (sg + 0.5f * ugr - 0.5f * rho * uu);
+        const float2 p =
+            mul2(f2(0.5f), fma2(mul2(f2(-0.5f), rho), uu, fma2(f2(0.5f), ugr, sg)));
 
         if (PASS & PASS_DIAG) {
-            const double u2 = (double)uu;
-            d_phi += (double)phi + (double)r;
-            d_E += 0.5 * (double)rho * u2;
-            d_u2 = fmax(d_u2, u2);
-            d_mumin = fmin(d_mumin, (double)mu);
-            d_mumax = fmax(d_mumax, (double)mu);
-            d_bud += 1.5 * (double)S - 0.5 * (double)Sprev;
-            if (!isfinite(phi) || !isfinite(p) || !isfinite(uu) || !isfinite(mu)) d_bad = 1.0;
+            auto acc = [&](float ph, float rr, float rh, float u2f, float m, float Sn, float So,
+                           float pp) {
+                const double u2 = (double)u2f;
+                d_phi += (double)ph + (double)rr;
+                d_E += 0.5 * (double)rh * u2;
+                d_u2 = fmax(d_u2, u2);
+                d_mumin = fmin(d_mumin, (double)m);
+                d_mumax = fmax(d_mumax, (double)m);
+                d_bud += 1.5 * (double)Sn - 0.5 * (double)So;
+                if (!isfinite(ph) || !isfinite(pp) || !isfinite(u2f) || !isfinite(m)) d_bad = 1.0;
+            };
+            acc(phi.x, r.x, rho.x, uu.x, mu.x, S.x, Sprev.x, p.x);
+            if (okB) acc(phi.y, r.y, rho.y, uu.y, mu.y, S.y, Sprev.y, p.y);
         }
         if (PASS & PASS_MACROS) {
-            if (a.out_phi) a.out_phi[n] = (double)phi + (double)r;
-            if (a.out_p) a.out_p[n] = (double)p;
-            if (a.out_mu) a.out_mu[n] = (double)mu;
+            auto put = [&](double *o, double va, double vb) {
+                o[n] = va;
+                if (okB) o[n + 1] = vb;
+            };
+            if (a.out_phi)
+                put(a.out_phi, (double)phi.x + (double)r.x, (double)phi.y + (double)r.y);
+            if (a.out_p) put(a.out_p, (double)p.x, (double)p.y);
+            if (a.out_mu) put(a.out_mu, (double)mu.x, (double)mu.y);
             if (a.out_u) {
-                a.out_u[n] = (double)u[0];
-                a.out_u[(size_t)N + n] = (double)u[1];
-                a.out_u[2 * (size_t)N + n] = (double)u[2];
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    put(a.out_u + d * (size_t)N, (double)u[d].x, (double)u[d].y);
             }
         }
         if (PASS & PASS_STATE) {
-            __stcs(static_cast<float *>(a.S) + n, S);
-            __stcs(dst.M + n, phi);
-            __stcs(dst.M + N + n, mu);
-            __stcs(dst.M + 2 * N + n, p);
-            __stcs(dst.M + 3 * N + n, u[0]);
-            __stcs(dst.M + 4 * N + n, u[1]);
-            __stcs(dst.M + 5 * N + n, u[2]);
+            auto put = [&](float *o, float2 v) {
+                if (EVEN) {
+                    __stcs(reinterpret_cast<float2 *>(o + n), v);
+                } else {
+                    __stcs(o + n, v.x);
+                    if (okB) __stcs(o + n + 1, v.y);
+                }
+            };
+            auto put16 = [&](unsigned short *o, float2 v) {
+                const unsigned e = C::enc2(v);
+                if (EVEN) {
+                    __stcs(reinterpret_cast<unsigned *>(o + n), e);
+                } else {
+                    __stcs(o + n, (unsigned short)(e & 0xffffu));
+                    if (okB) __stcs(o + n + 1, (unsigned short)(e >> 16));
+                }
+            };
+            put(static_cast<float *>(a.S), S);
+            put(dst.M, phi);
+            put(dst.M + N, mu);
+            put(dst.M + 2 * N, p);
+            put(dst.M + 3 * N, u[0]);
+            put(dst.M + 4 * N, u[1]);
+            put(dst.M + 5 * N, u[2]);
             {
                 // B = phi + alpha sum_{i != 0} w_i (mu(x + c_i) - mu(x)) from the mu ring
-                const float *m0 = mz, *mm = mus + mslot(zz - 1) * MA, *mp = mus + mslot(zz + 1) * MA;
-                const float fa = (m0[cm + 1] - mu) + (m0[cm - 1] - mu) + (m0[cm + MX] - mu) +
-                                 (m0[cm - MX] - mu) + (mp[cm] - mu) + (mm[cm] - mu);
-                const float ed = ((m0[cm + MX + 1] - mu) + (m0[cm + MX - 1] - mu) +
-                                  (m0[cm - MX + 1] - mu) + (m0[cm - MX - 1] - mu)) +
-                                 ((mp[cm + 1] - mu) + (mp[cm - 1] - mu) + (mm[cm + 1] - mu) +
-                                  (mm[cm - 1] - mu)) +
-                                 ((mp[cm + MX] - mu) + (mp[cm - MX] - mu) + (mm[cm + MX] - mu) +
-                                  (mm[cm - MX] - mu));
-                __stcs(dst.M + 6 * N + n, phi + P.alpha * ((1.0f / 18.0f) * fa + (1.0f / 36.0f) * ed));
+                auto dm = [&](const float *pl, int o, bool ev) {
+                    return sub2(pair_at(pl, c0 + o, ev), mu);
+                };
+                const float2 fa = add2(
+                    add2(add2(add2(add2(dm(m0, 1, false), dm(m0, -1, false)), dm(m0, MX, true)),
+                              dm(m0, -MX, true)),
+                         dm(mp, 0, true)),
+                    dm(mm, 0, true));
+                const float2 e1 =
+                    add2(add2(add2(dm(m0, MX + 1, false), dm(m0, MX - 1, false)),
+                              dm(m0, -MX + 1, false)),
+                         dm(m0, -MX - 1, false));
+                const float2 e2 = add2(
+                    add2(add2(dm(mp, 1, false), dm(mp, -1, false)), dm(mm, 1, false)),
+                    dm(mm, -1, false));
+                const float2 e3 = add2(
+                    add2(add2(dm(mp, MX, true), dm(mp, -MX, true)), dm(mm, MX, true)),
+                    dm(mm, -MX, true));
+                const float2 ed = add2(add2(e1, e2), e3);
+                put(dst.M + 6 * N,
+                    fma2(f2(P.alpha), fma2(f2(1.0f / 18.0f), fa, mul2(f2(1.0f / 36.0f), ed)), phi));
             }
             // CH population (Eqs. BGK, F_i): offset = (f - f^eq)(1 - 1/tau_f) + F_i,
             // b = -5/2, -1, 1/2; the rest offset also carries the residual r of phi
-            const float Sh = 1.5f * S - 0.5f * Sprev;
-            const float am = P.alpha * mu;
-            const float omf = 1.0f - P.inv_tauf;
-            const float d0 = ((2.0f / 3.0f) * am - snz) * omf + r - (5.0f / 6.0f) * Sh;
-            __stcs(dst.h + n, C::enc(d0 * it_f));
-            const float fa = -(1.0f / 18.0f) * Sh, fe = (1.0f / 72.0f) * Sh;
+            const float2 Sh = fma2(f2(1.5f), S, mul2(f2(-0.5f), Sprev));
+            const float2 am = mul2(f2(P.alpha), mu);
+            const float2 omf = f2(1.0f - P.inv_tauf), itf2 = f2(it_f), itg2 = f2(it_g);
+            const float2 msnz = neg2(snz);
+            const float2 d0 = fma2(f2(-(5.0f / 6.0f)), Sh,
+                                   fma2(fma2(f2(2.0f / 3.0f), am, msnz), omf, r));
+            put16(dst.h, mul2(d0, itf2));
+            const float2 fa = mul2(f2(-(1.0f / 18.0f)), Sh), fe = mul2(f2(1.0f / 72.0f), Sh);
 #pragma unroll
             for (int i = 1; i < 19; ++i) {
-                const float w = (float)w3(i);
-                __stcs(dst.h + (i * N + n), C::enc(((fv[i] - w * am) * omf + (i <= 6 ? fa : fe)) * it_f));
+                const float2 w = f2(-(float)w3(i));
+                put16(dst.h + i * N,
+                      mul2(fma2(fma2(w, am, fv[i]), omf, i <= 6 ? fa : fe), itf2));
             }
             // hydrodynamic population (Eqs. g_i, G_i): offset = (g - g^eq)(1 - 1/tau_g) + G_i
-            const float kg = 1.0f - 0.5f * itg, omg = 1.0f - itg;
-            const float A = 3.0f * p - 1.5f * rho * uu;
-            __stcs(dst.k + n, C::enc((gv[0] - ((1.0f / 3.0f) * A - 3.0f * p)) * omg * it_g));
+            const float2 kg = fma2(f2(-0.5f), itg, f2(1.0f)), omg = sub2(f2(1.0f), itg);
+            const float2 p3 = mul2(f2(3.0f), p), mp3 = mul2(f2(-3.0f), p);
+            const float2 A = fma2(mul2(f2(-1.5f), rho), uu, p3);
+            put16(dst.k, mul2(mul2(sub2(gv[0], fma2(f2(1.0f / 3.0f), A, mp3)), omg), itg2));
+            const float2 r45 = mul2(f2(4.5f), rho);
 #pragma unroll
             for (int i = 1; i < 19; ++i) {
                 const int o = (i <= 6) ? (i % 2 ? i + 1 : i - 1)
                                        : (i <= 10 ? 17 - i : (i <= 14 ? 25 - i : 33 - i));
                 if (o < i) continue;  // each pair once, from its first member
-                const float w = (float)w3(i);
-                const float cu = (float)c3x(i) * u[0] + (float)c3y(i) * u[1] + (float)c3z(i) * u[2];
-                const float cF = (float)c3x(i) * F[0] + (float)c3y(i) * F[1] + (float)c3z(i) * F[2];
-                const float cg = (float)c3x(i) * gr[0] + (float)c3y(i) * gr[1] + (float)c3z(i) * gr[2];
-                const float eq_s = w * (A + 4.5f * rho * cu * cu), eq_a = 3.0f * w * rho * cu;
-                const float G_s = 3.0f * w * kg * cu * cg, G_a = 3.0f * w * kg * cF;
-                __stcs(dst.k + (i * N + n), C::enc(((gv[i] - eq_s - eq_a) * omg + G_s + G_a) * it_g));
-                __stcs(dst.k + (o * N + n), C::enc(((gv[o] - eq_s + eq_a) * omg + G_s - G_a) * it_g));
+                const float wf = (float)w3(i);
+                const float2 cu = dot_c(c3x(i), c3y(i), c3z(i), u[0], u[1], u[2]);
+                const float2 cF = dot_c(c3x(i), c3y(i), c3z(i), F[0], F[1], F[2]);
+                const float2 cg = dot_c(c3x(i), c3y(i), c3z(i), gr[0], gr[1], gr[2]);
+                const float2 X = fma2(mul2(r45, cu), cu, A);           // eq_s = w X
+                const float2 ra = mul2(f2(3.0f * wf), rho);            // eq_a = ra cu
+                const float2 mra = mul2(f2(-3.0f * wf), rho);
+                const float2 wk = mul2(f2(3.0f * wf), kg);             // G_a = wk cF
+                const float2 mwk = mul2(f2(-3.0f * wf), kg);
+                const float2 wkcu = mul2(wk, cu);                      // G_s = wk cu cg
+                const float2 ti = fma2(mra, cu, fma2(f2(-wf), X, gv[i]));
+                const float2 to = fma2(ra, cu, fma2(f2(-wf), X, gv[o]));
+                put16(dst.k + i * N, mul2(fma2(wk, cF, fma2(wkcu, cg, mul2(ti, omg))), itg2));
+                put16(dst.k + o * N, mul2(fma2(mwk, cF, fma2(wkcu, cg, mul2(to, omg))), itg2));
             }
         }
-        }  // col_ok
+        }  // okA
         cp_wait_all();
         __syncthreads();
-        for (int q = tid; q < MA; q += TX3 * TY3) {  // own copies: no barrier needed
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {  // own copies: no barrier needed
+            if (tid + k * OFF_NT >= MN) break;
             float m6[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MA + q];
-            put_macros(qslot(zz + 2), q, m6);
+            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MN + tid + k * OFF_NT];
+            put_macros(sq, mring[k], m6);
         }
-        mu_plane(zz + 2);
+        // phi planes zz + 1 .. zz + 3 -> mu plane zz + 2 in the slot of zz - 1
+        mu_plane(spp, wrapr(sp + 3, RP), wrapr(sp + 4, RP), sq);
         __syncthreads();
+        sp = sp0;
+        sq = sq0;
     }
 
     if (PASS & PASS_DIAG) {
@@ -449,7 +616,7 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_off_pass_kernel(const StepPara
             d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
             d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
         }
-        constexpr int NW = TX3 * TY3 / 32;
+        constexpr int NW = OFF_NT / 32;
         __shared__ double red[7][NW];
         const int lane = tid & 31, wid = tid >> 5;
         if (lane == 0) {
@@ -692,7 +859,7 @@ int off_ctas_per_sm_t()
 {
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, d3q19_off_pass_kernel<C, PASS_STATE>, TX3 * TY3, 0);
+        &n, d3q19_off_pass_kernel<C, PASS_STATE, true>, OFF_NT, 0);
     return e == cudaSuccess && n > 0 ? n : 2;
 }
 
@@ -704,9 +871,12 @@ cudaError_t launch_off(const StepParams<float> &P, const PassArgs &a, const Laun
     const dim3 pg((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz);
     const cudaError_t e = launch_pdl(d3q19_off_phi_kernel<C>, pg, PHI_TX, 0, st, P, src, phi);
     if (e != cudaSuccess) return e;
-    dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TX3, TY3);
-    return launch_pdl(d3q19_off_pass_kernel<C, PASS>, grid, block, 0, st, P, a, src, dst, target,
-                      phi, s.rows);
+    const dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TXP, TY3);
+    if (P.nx % 2 == 0)
+        return launch_pdl(d3q19_off_pass_kernel<C, PASS, true>, grid, block, 0, st, P, a, src, dst,
+                          target, phi, s.rows);
+    return launch_pdl(d3q19_off_pass_kernel<C, PASS, false>, grid, block, 0, st, P, a, src, dst,
+                      target, phi, s.rows);
 }
 
 template <class C>
