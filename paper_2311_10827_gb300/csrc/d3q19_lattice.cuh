@@ -9,6 +9,8 @@ namespace d3 {
 
 // column tile of the z-marching pass kernels (threads x, y)
 constexpr int TX3 = 32, TY3 = 8;
+// threads of the passes that update two x-neighbours per thread
+constexpr int TXP = TX3 / 2, PAIR_NT = TXP * TY3;
 
 // velocity order: rest; +x, -x, +y, -y, +z, -z; then the 12 edges
 // (+x+y, +x-y, -x+y, -x-y), (+x+z, +x-z, -x+z, -x-z), (+y+z, +y-z, -y+z, -y-z)
@@ -40,17 +42,6 @@ __device__ __forceinline__ int wrapi(int c, int n)
 __device__ __forceinline__ int wrap1(int c, int n) { return c < 0 ? c + n : (c >= n ? c - n : c); }
 // wrap of any c; `small` (a uniform flag) when c may leave [-n, 2n)
 __device__ __forceinline__ int wrapc(int c, int n, bool small) { return small ? wrapi(c, n) : wrap1(c, n); }
-
-template <typename T>
-struct Arith3;
-template <>
-struct Arith3<float> {
-    __device__ static float rcp(float x) { return __fdividef(1.0f, x); }
-};
-template <>
-struct Arith3<double> {
-    __device__ static double rcp(double x) { return 1.0 / x; }
-};
 
 // offsets of the 27 neighbours (dx, dy, dz in -1..1) of a node from wrapped
 // coordinates

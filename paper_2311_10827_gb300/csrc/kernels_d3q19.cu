@@ -19,6 +19,7 @@
 #include "d3q19_lattice.cuh"
 #include "launch.cuh"
 #include "lbm_internal.h"
+#include "pair32.cuh"
 
 namespace wblbm {
 namespace {
@@ -48,10 +49,58 @@ __global__ void __launch_bounds__(PHI_TX)
     phi[n] = v[0] + s;
 }
 
-template <typename T, int PASS>
-__global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T> P, PassArgs a,
-                                                              const T *__restrict__ phif, int planes)
+// One CTA's diagnostics partial from its NT threads' values (all of them call it)
+template <int NT>
+__device__ __forceinline__ void write_partial3(int tid, double d_phi, double d_E, double d_u2,
+                                               double d_mumin, double d_mumax, double d_bud,
+                                               double d_bad, DiagPartial *out)
 {
+    for (int o = 16; o > 0; o >>= 1) {
+        d_phi += __shfl_xor_sync(0xffffffffu, d_phi, o);
+        d_E += __shfl_xor_sync(0xffffffffu, d_E, o);
+        d_bud += __shfl_xor_sync(0xffffffffu, d_bud, o);
+        d_u2 = fmax(d_u2, __shfl_xor_sync(0xffffffffu, d_u2, o));
+        d_mumin = fmin(d_mumin, __shfl_xor_sync(0xffffffffu, d_mumin, o));
+        d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
+        d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
+    }
+    constexpr int NW = NT / 32;
+    __shared__ double red[7][NW];
+    const int lane = tid & 31, wid = tid >> 5;
+    if (lane == 0) {
+        red[0][wid] = d_phi;
+        red[1][wid] = d_E;
+        red[2][wid] = d_u2;
+        red[3][wid] = d_mumin;
+        red[4][wid] = d_mumax;
+        red[5][wid] = d_bud;
+        red[6][wid] = d_bad;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        DiagPartial o;
+        o.sum_phi = 0.0, o.E = 0.0, o.u2max = 0.0, o.mu_min = DBL_MAX, o.mu_max = -DBL_MAX;
+        o.budget = 0.0, o.nonfinite = 0.0, o.pad = 0.0;
+        for (int w = 0; w < NW; ++w) {
+            o.sum_phi += red[0][w];
+            o.E += red[1][w];
+            o.u2max = fmax(o.u2max, red[2][w]);
+            o.mu_min = fmin(o.mu_min, red[3][w]);
+            o.mu_max = fmax(o.mu_max, red[4][w]);
+            o.budget += red[5][w];
+            o.nonfinite = fmax(o.nonfinite, red[6][w]);
+        }
+        *out = o;
+    }
+}
+
+// The FP64 pass: one node per thread.
+template <int PASS>
+__global__ void __launch_bounds__(TX3 *TY3)
+    d3q19_pass_kernel(const StepParams<double> P, PassArgs a, const double *__restrict__ phif,
+                      int planes)
+{
+    using T = double;
     constexpr int PX = TX3 + 4, PY = TY3 + 4, PA = PX * PY;  // phi plane (halo 2)
     constexpr int MX = TX3 + 2, MY = TY3 + 2, MA = MX * MY;  // mu plane (halo 1)
     constexpr int RP = 5, RM = 3;
@@ -120,15 +169,6 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
     double d_phi = 0.0, d_E = 0.0, d_u2 = 0.0, d_mumin = DBL_MAX, d_mumax = -DBL_MAX,
            d_bud = 0.0, d_bad = 0.0;
 
-    // FP32: equilibrium shift of the source buffer and of the writes (only a
-    // time step reads it)
-    T a_src = T(0), a_dst = T(0);
-    if (sizeof(T) == 4 && (PASS & PASS_STATE)) {
-        a_src = *a.eqs_src;
-        a_dst = *a.eqs_target;
-        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) *a.eqs_dst = a_dst;
-    }
-
     for (int q = 0; q < 5; ++q) load_phi_plane(z0 - 2 + q);
     __syncthreads();
     mu_plane(z0 - 1);
@@ -170,14 +210,13 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
         T Sprev = T(0);
         if (PASS & (PASS_STATE | PASS_DIAG)) Sprev = __ldcs(static_cast<const T *>(a.S) + n);
 
-        const T lo0 = sizeof(T) == 4 ? __ldg(fsrc + (19u * N + n)) : T(0);
         T snz = T(0), sg = T(0);
 #pragma unroll
         for (int i = 1; i < 19; i += 2) {
             snz += fv[i] + fv[i + 1];
             sg += gv[i] + gv[i + 1];
         }
-        const T phi = fv[0] + (lo0 + snz);
+        const T phi = fv[0] + snz;
         const int cp = (ty + 2) * PX + (tx + 2), cm = (ty + 1) * MX + (tx + 1);
         const T *mz = mus + mslot(zz) * MA;
         const T mu = mz[cm];
@@ -189,8 +228,8 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
         const T dphi = phi - P.phiv;
         const T rho = P.rhov + dphi * P.drho;
         const T nu = P.nuv + dphi * P.dnu;
-        const T inv_rho = Arith3<T>::rcp(rho);
-        const T itg = Arith3<T>::rcp(T(0.5) + T(3) * nu);
+        const T inv_rho = T(1) / (rho);
+        const T itg = T(1) / (T(0.5) + T(3) * nu);
         T j3[3] = {T(0), T(0), T(0)};
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
@@ -240,26 +279,13 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
             __stcs(static_cast<T *>(a.S) + n, S);
             // CH population: b = -5/2, -1, 1/2 (rest, face, edge) for D = 3
             const T Sh = T(1.5) * S - T(0.5) * Sprev;
-            const T am = P.alpha * mu - a_src;  // in the source buffer's shifted variables
-            const T dsh = a_src - a_dst;         // move the writes to the target shift
+            const T am = P.alpha * mu;
             const T itf = P.inv_tauf;
-            {
-                const T d0 = -(T(2.0 / 3.0) * am - snz) * itf - T(5.0 / 6.0) * Sh - T(2.0 / 3.0) * dsh;
-                if (sizeof(T) == 4) {
-                    const T sl = lo0 + d0;  // exact two-sum on the high word
-                    const T hi = fv[0] + sl;
-                    const T bp = hi - fv[0];
-                    __stcs(fd + n, hi);
-                    __stcs(fd + (19u * N + n), (fv[0] - (hi - bp)) + (sl - bp));
-                } else {
-                    __stcs(fd + n, fv[0] + d0);
-                }
-            }
+            __stcs(fd + n, fv[0] + (-(T(2.0 / 3.0) * am - snz) * itf - T(5.0 / 6.0) * Sh));
             // each population moves by its own small increment (as in 2D: the
             // increments sum to sum_i F_i up to unbiased rounding)
             const T ea = T(1.0 / 18.0) * am, ee = T(1.0 / 36.0) * am;
-            const T sa = T(-1.0 / 18.0) * Sh + T(1.0 / 18.0) * dsh;
-            const T se = T(1.0 / 72.0) * Sh + T(1.0 / 36.0) * dsh;
+            const T sa = T(-1.0 / 18.0) * Sh, se = T(1.0 / 72.0) * Sh;
 #pragma unroll
             for (int i = 1; i < 19; ++i)
                 __stcs(fd + (i * N + n), fv[i] + (((i <= 6 ? ea : ee) - fv[i]) * itf + (i <= 6 ? sa : se)));
@@ -295,45 +321,301 @@ __global__ void __launch_bounds__(TX3 *TY3) d3q19_pass_kernel(const StepParams<T
         __syncthreads();
     }
 
-    if (PASS & PASS_DIAG) {
-        for (int o = 16; o > 0; o >>= 1) {
-            d_phi += __shfl_xor_sync(0xffffffffu, d_phi, o);
-            d_E += __shfl_xor_sync(0xffffffffu, d_E, o);
-            d_bud += __shfl_xor_sync(0xffffffffu, d_bud, o);
-            d_u2 = fmax(d_u2, __shfl_xor_sync(0xffffffffu, d_u2, o));
-            d_mumin = fmin(d_mumin, __shfl_xor_sync(0xffffffffu, d_mumin, o));
-            d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
-            d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
-        }
-        constexpr int NW = TX3 * TY3 / 32;
-        __shared__ double red[7][NW];
-        const int lane = tid & 31, wid = tid >> 5;
-        if (lane == 0) {
-            red[0][wid] = d_phi;
-            red[1][wid] = d_E;
-            red[2][wid] = d_u2;
-            red[3][wid] = d_mumin;
-            red[4][wid] = d_mumax;
-            red[5][wid] = d_bud;
-            red[6][wid] = d_bad;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            DiagPartial o;
-            o.sum_phi = 0.0, o.E = 0.0, o.u2max = 0.0, o.mu_min = DBL_MAX, o.mu_max = -DBL_MAX;
-            o.budget = 0.0, o.nonfinite = 0.0, o.pad = 0.0;
-            for (int w = 0; w < NW; ++w) {
-                o.sum_phi += red[0][w];
-                o.E += red[1][w];
-                o.u2max = fmax(o.u2max, red[2][w]);
-                o.mu_min = fmin(o.mu_min, red[3][w]);
-                o.mu_max = fmax(o.mu_max, red[4][w]);
-                o.budget += red[5][w];
-                o.nonfinite = fmax(o.nonfinite, red[6][w]);
-            }
-            a.partials[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = o;
-        }
+    if (PASS & PASS_DIAG)
+        write_partial3<TX3 * TY3>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
+                                  a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+}
+
+// The FP32 pass: two nodes adjacent in x per thread (TXP x TY3 threads), their
+// arithmetic on the paired FP32 datapath, 64-bit loads and stores of both
+// where rows are even (EVEN) and the pull has no x component.
+// What bounds it: HBM on large grids (408 B per node with the phi pass, at 90%
+// of the copy bandwidth), the latency of a plane on small ones.  719
+// instructions per node against 1192 with one node per thread, three CTAs of
+// 128 threads per SM (four, at 128 registers: 2% slower at 512^3).  Measured:
+// 64^3 24.0 -> 20.2 us per step, 512^3 runs 10.6 -> 9.7 ms per step.  Not kept:
+// phi summed inside this kernel for the plane three ahead (no phi pass): the
+// populations it read came back from HBM again for half of the update's pulls
+// (205 against 168 B read per node), 512^3 9.58 against 8.92 ms per step, 64^3
+// 27.1 against 19.6 us.
+template <int PASS, bool EVEN>
+__global__ void __launch_bounds__(PAIR_NT, 3)
+    d3q19_pass32_kernel(const StepParams<float> P, PassArgs a, const float *__restrict__ phif,
+                        int planes)
+{
+    constexpr int PX = TX3 + 4, PY = TY3 + 4, PA = PX * PY;  // phi plane (halo 2)
+    constexpr int MX = TX3 + 4, MY = TY3 + 2, MA = MX * MY;  // mu plane (halo 1; 2 stored in x)
+    constexpr int MW = TX3 + 2, MN = MW * MY;                // nodes of a mu plane
+    constexpr int RP = 5, RM = 3;
+    __shared__ __align__(16) float phs[RP * PA];
+    __shared__ __align__(16) float mus[RM * MA];
+
+    pdl_wait();
+    const int nx = P.nx, ny = P.ny, nz = P.nz;
+    const unsigned N = (unsigned)P.N;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TXP + tx;
+    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
+    const int x = x0 + 2 * tx, y = y0 + ty;
+    const bool okA = x < nx && y < ny, okB = EVEN ? okA : (x + 1 < nx && y < ny);
+    const unsigned plane = (unsigned)nx * ny;
+    const float *__restrict__ fsrc = static_cast<const float *>(a.f_src);
+    const float *__restrict__ gsrc = static_cast<const float *>(a.g_src);
+
+    // grids narrower than a tile plus halo wrap by division (uniform flags)
+    const bool smx = nx < PX + 2, smy = ny < PY + 2, smz = nz < 8;
+    // this thread's elements of a phi plane and nodes of a mu plane
+    constexpr int KP = (PA + PAIR_NT - 1) / PAIR_NT, KM = (MN + PAIR_NT - 1) / PAIR_NT;
+    unsigned poff[KP];
+    int mring[KM];
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+        const int q = tid + k * PAIR_NT;
+        poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
     }
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+        const int q = tid + k * PAIR_NT;
+        mring[k] = q / MW * MX + q % MW + 1;
+    }
+    auto wrapr = [](int v, int n) { return v >= n ? v - n : v; };
+    // Eq. chemical_potencial with Eq. Laplace on D3Q19, from the phi slots of the
+    // planes below, at and above into mu slot sm:
+    // lap = (1/3) sum_faces (phi_n - phi) + (1/6) sum_edges (phi_n - phi)
+    auto mu_plane = [&](int s_m, int s_0, int s_p, int sm) {
+        const float *pm = phs + s_m * PA, *p0 = phs + s_0 * PA, *pp = phs + s_p * PA;
+        float *d = mus + sm * MA;
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+            if (tid + k * PAIR_NT >= MN) break;
+            const int c = mring[k] + PX;  // one phi row further (halo 2 against 1)
+            const float v = p0[c];
+            const float fa = (p0[c + 1] - v) + (p0[c - 1] - v) + (p0[c + PX] - v) +
+                             (p0[c - PX] - v) + (pp[c] - v) + (pm[c] - v);
+            const float ed = ((p0[c + PX + 1] - v) + (p0[c + PX - 1] - v) + (p0[c - PX + 1] - v) +
+                              (p0[c - PX - 1] - v)) +
+                             ((pp[c + 1] - v) + (pp[c - 1] - v) + (pm[c + 1] - v) + (pm[c - 1] - v)) +
+                             ((pp[c + PX] - v) + (pp[c - PX] - v) + (pm[c + PX] - v) +
+                              (pm[c - PX] - v));
+            const float lap = (1.0f / 3.0f) * fa + (1.0f / 6.0f) * ed;
+            d[mring[k]] = 4.0f * P.beta * (v - P.phil) * (v - P.phiv) * (v - P.phibar) - P.kappa * lap;
+        }
+    };
+
+    double d_phi = 0.0, d_E = 0.0, d_u2 = 0.0, d_mumin = DBL_MAX, d_mumax = -DBL_MAX,
+           d_bud = 0.0, d_bad = 0.0;
+
+    // equilibrium shift of the source buffer and of the writes (only a time step reads it)
+    float a_src = 0.0f, a_dst = 0.0f;
+    if (PASS & PASS_STATE) {
+        a_src = *a.eqs_src;
+        a_dst = *a.eqs_target;
+        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) *a.eqs_dst = a_dst;
+    }
+
+    for (int d = 0; d < 5; ++d) {
+        const unsigned zo = (unsigned)wrapc(z0 - 2 + d, nz, smz) * plane;
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+            if (tid + k * PAIR_NT < PA) cp_async4(phs + d * PA + tid + k * PAIR_NT, phif + zo + poff[k]);
+    }
+    cp_commit();
+    cp_wait_all();
+    __syncthreads();
+    for (int d = 0; d < 3; ++d) mu_plane(d, d + 1, d + 2, d);
+    __syncthreads();
+
+    // Plane zz + 3 of phi is copied asynchronously while plane zz is updated.
+    // Ring use during the update of plane zz: phi planes zz-1..zz+1 (read),
+    // zz+3 (written: a fifth slot); mu planes zz-1..zz+1.
+    const unsigned xw = okA ? (unsigned)x : 0, yw = okA ? (unsigned)y : 0;
+    Nb b = make_nb((int)xw, (int)yw, z0, nx, ny, nz);
+    const unsigned xB = okB ? xw + 1 : 0;  // the second node's column and its +x neighbour
+    const unsigned xpp = nx == 1 ? 0u : (unsigned)wrap1((int)xw + 2, nx);
+    int sp = 1, sq = 0;  // phi slot of plane zz - 1, mu slot of plane zz - 1
+    for (int zz = z0; zz < zend; ++zz) {
+        const int sp0 = wrapr(sp + 1, RP), spp = wrapr(sp + 2, RP);
+        const int sq0 = wrapr(sq + 1, RM), sqp = wrapr(sq + 2, RM);
+        {
+            const unsigned zo = (unsigned)wrapc(zz + 3, nz, smz) * plane;
+            float *d = phs + wrapr(sp + 4, RP) * PA + tid;
+#pragma unroll
+            for (int k = 0; k < KP; ++k)
+                if (tid + k * PAIR_NT < PA) cp_async4(d + k * PAIR_NT, phif + (zo + poff[k]));
+            cp_commit();
+        }
+        if (okA) {
+        nb_plane(b, zz, nx, ny, nz);
+        const unsigned row = b.zs[1] + b.ys[1], n = row + xw;
+        auto pull = [&](const float *v, int i) -> float2 {
+            const unsigned r = i * N + b.zs[1 - c3z(i)] + b.ys[1 - c3y(i)];
+            if (c3x(i) == 0 && EVEN) return __ldg(reinterpret_cast<const float2 *>(v + (r + xw)));
+            const unsigned ca = c3x(i) > 0 ? b.xs[0] : (c3x(i) < 0 ? b.xs[2] : xw);
+            const unsigned cb = c3x(i) > 0 ? xw : (c3x(i) < 0 ? xpp : xB);
+            return make_float2(__ldg(v + (r + ca)), __ldg(v + (r + cb)));
+        };
+        float2 fv[19], gv[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            fv[i] = pull(fsrc, i);
+            gv[i] = pull(gsrc, i);
+        }
+        float2 Sprev = f2(0.0f), lo0;
+        if (EVEN)
+            lo0 = __ldg(reinterpret_cast<const float2 *>(fsrc + (19u * N + n)));
+        else
+            lo0 = make_float2(__ldg(fsrc + (19u * N + n)), __ldg(fsrc + (19u * N + row + xB)));
+        if (PASS & (PASS_STATE | PASS_DIAG)) {
+            const float *S = static_cast<const float *>(a.S);
+            if (EVEN)
+                Sprev = __ldcs(reinterpret_cast<const float2 *>(S + n));
+            else
+                Sprev = make_float2(__ldcs(S + n), __ldcs(S + (row + xB)));
+        }
+
+        float2 snz = add2(fv[1], fv[2]), sg = add2(gv[1], gv[2]);
+#pragma unroll
+        for (int i = 3; i < 19; i += 2) {
+            snz = add2(snz, add2(fv[i], fv[i + 1]));
+            sg = add2(sg, add2(gv[i], gv[i + 1]));
+        }
+        const float2 phi = add2(fv[0], add2(lo0, snz));
+        const int cp = (ty + 2) * PX + 2 * tx + 2, c0 = (ty + 1) * MX + 2 * tx + 2;
+        const float *m0 = mus + sq0 * MA;
+        const float2 mu = pair_at(m0, c0, true);
+        float2 gp[3], gm[3];
+        grad3_pair(phs + sp * PA, phs + sp0 * PA, phs + spp * PA, cp, PX, gp);
+        grad3_pair(mus + sq * MA, m0, mus + sqp * MA, c0, MX, gm);
+
+        float2 F[3], gr[3], u[3];
+        const float2 dphi = sub2(phi, f2(P.phiv));
+        const float2 rho = fma2(dphi, f2(P.drho), f2(P.rhov));
+        const float2 nu = fma2(dphi, f2(P.dnu), f2(P.nuv));
+        const float2 inv_rho = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+        const float2 tg = fma2(f2(3.0f), nu, f2(0.5f));
+        const float2 itg = make_float2(__fdividef(1.0f, tg.x), __fdividef(1.0f, tg.y));
+        float2 j3[3] = {f2(0.0f), f2(0.0f), f2(0.0f)};
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            if (c3x(i)) j3[0] = c3x(i) > 0 ? add2(j3[0], gv[i]) : sub2(j3[0], gv[i]);
+            if (c3y(i)) j3[1] = c3y(i) > 0 ? add2(j3[1], gv[i]) : sub2(j3[1], gv[i]);
+            if (c3z(i)) j3[2] = c3z(i) > 0 ? add2(j3[2], gv[i]) : sub2(j3[2], gv[i]);
+        }
+        float2 ugr = f2(0.0f), uu = f2(0.0f), S = f2(0.0f);
+        const float2 mphi = neg2(phi);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            F[d] = fma2(mphi, gm[d], f2(P.G[d]));
+            gr[d] = mul2(f2(P.drho), gp[d]);
+            u[d] = mul2(fma2(f2(0.5f), F[d], j3[d]), inv_rho);
+            ugr = fma2(u[d], gr[d], ugr);
+            uu = fma2(u[d], u[d], uu);
+            S = fma2(u[d], gp[d], S);
+        }
+        // p = cs2/(1 - w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0], cs2/(1-w0) = 1/2,
+        // rho s_0 = -(1/2) rho |u|^2
+        const float2 p =
+            mul2(f2(0.5f), fma2(mul2(f2(-0.5f), rho), uu, fma2(f2(0.5f), ugr, sg)));
+
+        if (PASS & PASS_DIAG) {
+            auto acc = [&](float ph, float rh, float u2f, float m, float Sn, float So, float pp) {
+                const double u2 = (double)u2f;
+                d_phi += (double)ph;
+                d_E += 0.5 * (double)rh * u2;
+                d_u2 = fmax(d_u2, u2);
+                d_mumin = fmin(d_mumin, (double)m);
+                d_mumax = fmax(d_mumax, (double)m);
+                d_bud += 1.5 * (double)Sn - 0.5 * (double)So;
+                if (!isfinite(ph) || !isfinite(pp) || !isfinite(u2f) || !isfinite(m)) d_bad = 1.0;
+            };
+            acc(phi.x, rho.x, uu.x, mu.x, S.x, Sprev.x, p.x);
+            if (okB) acc(phi.y, rho.y, uu.y, mu.y, S.y, Sprev.y, p.y);
+        }
+        if (PASS & PASS_MACROS) {
+            auto put = [&](double *o, float2 v) {
+                o[n] = (double)v.x;
+                if (okB) o[n + 1] = (double)v.y;
+            };
+            if (a.out_phi) put(a.out_phi, phi);
+            if (a.out_p) put(a.out_p, p);
+            if (a.out_mu) put(a.out_mu, mu);
+            if (a.out_u) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) put(a.out_u + d * (size_t)N, u[d]);
+            }
+        }
+        if (PASS & PASS_STATE) {
+            float *__restrict__ fd = static_cast<float *>(a.f_dst);
+            float *__restrict__ gd = static_cast<float *>(a.g_dst);
+            auto put = [&](float *o, float2 v) {
+                if (EVEN) {
+                    __stcs(reinterpret_cast<float2 *>(o + n), v);
+                } else {
+                    __stcs(o + n, v.x);
+                    if (okB) __stcs(o + n + 1, v.y);
+                }
+            };
+            put(static_cast<float *>(a.S), S);
+            // CH population: b = -5/2, -1, 1/2 (rest, face, edge) for D = 3
+            const float2 Sh = fma2(f2(1.5f), S, mul2(f2(-0.5f), Sprev));
+            const float2 am = fma2(f2(P.alpha), mu, f2(-a_src));  // in the source's shifted variables
+            const float dsh = a_src - a_dst;                      // move the writes to the target shift
+            const float2 itf = f2(P.inv_tauf);
+            {
+                const float2 q = fma2(f2(-(2.0f / 3.0f)), am, snz);
+                const float2 d0 = fma2(f2(-(5.0f / 6.0f)), Sh,
+                                       fma2(q, itf, f2(-(2.0f / 3.0f) * dsh)));
+                const float2 sl = add2(lo0, d0);  // exact two-sum on the high word
+                const float2 hi = add2(fv[0], sl);
+                const float2 bp = sub2(hi, fv[0]);
+                put(fd, hi);
+                put(fd + 19u * N, add2(sub2(fv[0], sub2(hi, bp)), sub2(sl, bp)));
+            }
+            // each population moves by its own small increment (as in 2D: the
+            // increments sum to sum_i F_i up to unbiased rounding)
+            const float2 ea = mul2(f2(1.0f / 18.0f), am), ee = mul2(f2(1.0f / 36.0f), am);
+            const float2 sa = fma2(f2(-1.0f / 18.0f), Sh, f2((1.0f / 18.0f) * dsh));
+            const float2 se = fma2(f2(1.0f / 72.0f), Sh, f2((1.0f / 36.0f) * dsh));
+#pragma unroll
+            for (int i = 1; i < 19; ++i)
+                put(fd + i * N,
+                    add2(fv[i], fma2(sub2(i <= 6 ? ea : ee, fv[i]), itf, i <= 6 ? sa : se)));
+            // hydrodynamic population, pairs of opposite directions (as in 2D)
+            const float2 kg = fma2(f2(-0.5f), itg, f2(1.0f));
+            const float2 p3 = mul2(f2(3.0f), p);
+            const float2 A = fma2(mul2(f2(-1.5f), rho), uu, p3);
+            put(gd, fma2(sub2(sub2(mul2(f2(1.0f / 3.0f), A), p3), gv[0]), itg, gv[0]));
+            const float2 r45 = mul2(f2(4.5f), rho);
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                const int o = (i <= 6) ? (i % 2 ? i + 1 : i - 1)
+                                       : (i <= 10 ? 17 - i : (i <= 14 ? 25 - i : 33 - i));
+                if (o < i) continue;  // each pair once, from its first member
+                const float w = (float)w3(i);
+                const float2 cu = dot_c(c3x(i), c3y(i), c3z(i), u[0], u[1], u[2]);
+                const float2 cF = dot_c(c3x(i), c3y(i), c3z(i), F[0], F[1], F[2]);
+                const float2 cg = dot_c(c3x(i), c3y(i), c3z(i), gr[0], gr[1], gr[2]);
+                const float2 es = mul2(f2(w), fma2(mul2(r45, cu), cu, A));
+                const float2 ea_ = mul2(mul2(f2(3.0f * w), rho), cu);
+                const float2 wk = mul2(f2(3.0f * w), kg);
+                const float2 Gs = mul2(mul2(wk, cu), cg), Ga = mul2(wk, cF);
+                put(gd + i * N, add2(gv[i], fma2(sub2(add2(es, ea_), gv[i]), itg, add2(Gs, Ga))));
+                put(gd + o * N, add2(gv[o], fma2(sub2(sub2(es, ea_), gv[o]), itg, sub2(Gs, Ga))));
+            }
+        }
+        }  // okA
+        cp_wait_all();
+        __syncthreads();
+        // phi planes zz + 1 .. zz + 3 -> mu plane zz + 2 in the slot of zz - 1
+        mu_plane(spp, wrapr(sp + 3, RP), wrapr(sp + 4, RP), sq);
+        __syncthreads();
+        sp = sp0;
+        sq = sq0;
+    }
+
+    if (PASS & PASS_DIAG)
+        write_partial3<PAIR_NT>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
+                                a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
 // ------------------------------------------------------------ initial state
@@ -415,13 +697,22 @@ cudaError_t launch3(const void *params, const PassArgs &a, const LaunchShape &s,
                     cudaStream_t st)
 {
     const StepParams<T> &P = *static_cast<const StepParams<T> *>(params);
+    const dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y));
     const dim3 pg((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz);
     const cudaError_t e = launch_pdl(d3q19_phi_kernel<T>, pg, PHI_TX, 0, st, P,
                                      static_cast<const T *>(a.f_src), static_cast<T *>(phi));
     if (e != cudaSuccess) return e;
-    dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TX3, TY3);
-    return launch_pdl(d3q19_pass_kernel<T, PASS>, grid, block, 0, st, P, a,
-                      static_cast<const T *>(phi), s.rows);
+    if constexpr (sizeof(T) == 4) {
+        const dim3 block(TXP, TY3);
+        if (P.nx % 2 == 0)
+            return launch_pdl(d3q19_pass32_kernel<PASS, true>, grid, block, 0, st, P, a,
+                              static_cast<const float *>(phi), s.rows);
+        return launch_pdl(d3q19_pass32_kernel<PASS, false>, grid, block, 0, st, P, a,
+                          static_cast<const float *>(phi), s.rows);
+    } else {
+        return launch_pdl(d3q19_pass_kernel<PASS>, grid, dim3(TX3, TY3), 0, st, P, a,
+                          static_cast<const T *>(phi), s.rows);
+    }
 }
 
 template <typename T>
@@ -474,9 +765,9 @@ int d3q19_ctas_per_sm(int precision)
     int n = 0;
     cudaError_t e = precision == 0
                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &n, d3q19_pass_kernel<double, PASS_STATE>, TX3 * TY3, 0)
+                              &n, d3q19_pass_kernel<PASS_STATE>, TX3 * TY3, 0)
                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &n, d3q19_pass_kernel<float, PASS_STATE>, TX3 * TY3, 0);
+                              &n, d3q19_pass32_kernel<PASS_STATE, true>, PAIR_NT, 0);
     return e == cudaSuccess && n > 0 ? n : 2;
 }
 

@@ -41,6 +41,7 @@
 #include "d3q19_lattice.cuh"
 #include "launch.cuh"
 #include "lbm_internal.h"
+#include "pair32.cuh"
 
 namespace wblbm {
 namespace {
@@ -144,25 +145,6 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 
 // ------------------------------------------------------------------ pass 2
 
-// The paired FP32 datapath: two independent lanes per instruction, each
-// rounding as the scalar instruction does.  The lanes are the thread's two
-// nodes.
-__device__ __forceinline__ float2 f2(float s) { return make_float2(s, s); }
-__device__ __forceinline__ float2 add2(float2 x, float2 y) { return __fadd2_rn(x, y); }
-__device__ __forceinline__ float2 mul2(float2 x, float2 y) { return __fmul2_rn(x, y); }
-__device__ __forceinline__ float2 fma2(float2 x, float2 y, float2 z) { return __ffma2_rn(x, y, z); }
-// x - y as one multiply-add by -1 (the same single rounding)
-__device__ __forceinline__ float2 sub2(float2 x, float2 y) { return __ffma2_rn(y, f2(-1.0f), x); }
-__device__ __forceinline__ float2 neg2(float2 x) { return __fmul2_rn(x, f2(-1.0f)); }
-// sum_d c_d v_d of a velocity c (components 0, 1, -1; the first non-zero one may be -1)
-__device__ __forceinline__ float2 dot_c(int cx, int cy, int cz, float2 x, float2 y, float2 z)
-{
-    float2 s = cx ? (cx > 0 ? x : neg2(x)) : (cy ? (cy > 0 ? y : neg2(y)) : (cz > 0 ? z : neg2(z)));
-    if (cx && cy) s = cy > 0 ? add2(s, y) : sub2(s, y);
-    if ((cx || cy) && cz) s = cz > 0 ? add2(s, z) : sub2(s, z);
-    return s;
-}
-
 // What bounds this pass: instruction issue and the latency of the pulls.
 // Rebuilding 38 populations per node from their offsets took 1570 instructions
 // per node with one node per thread (256^3 FP16: 1.135 ms, issue slots 60% busy
@@ -180,11 +162,8 @@ __device__ __forceinline__ float2 dot_c(int cx, int cy, int cz, float2 x, float2
 // (333 us: the load/store units take one word per thread at a time), the next
 // plane's pulls in registers during the collisions at two CTAs per SM (238 us),
 // or while its mu is formed (264 us: they spill).
-constexpr int TXP = 16;           // pairs per row of a tile: TX3 = 2 TXP nodes
-static_assert(TX3 == 2 * TXP, "tile width");
-constexpr int OFF_NT = TXP * TY3;  // threads per CTA
 template <class C, int PASS, bool EVEN>
-__global__ void __launch_bounds__(OFF_NT, 3)
+__global__ void __launch_bounds__(PAIR_NT, 3)
     d3q19_off_pass_kernel(const StepParams<float> P, PassArgs a, const OffBuf src, const OffBuf dst,
                           const float *__restrict__ target, const float *__restrict__ phif,
                           int planes)
@@ -223,17 +202,17 @@ __global__ void __launch_bounds__(OFF_NT, 3)
     const bool smx = nx < PX + 2, smy = ny < PY + 2, smz = nz < 8;
     // this thread's elements of a phi plane and nodes of a mu / macro plane:
     // ring index and in-plane offset in the grid (nodes past the halo repeat)
-    constexpr int KP = (PA + OFF_NT - 1) / OFF_NT, KM = (MN + OFF_NT - 1) / OFF_NT;
+    constexpr int KP = (PA + PAIR_NT - 1) / PAIR_NT, KM = (MN + PAIR_NT - 1) / PAIR_NT;
     unsigned poff[KP], moff[KM];
     int mring[KM];  // index in a stored plane (row stride MX, x halo 2)
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
-        const int q = tid + k * OFF_NT;
+        const int q = tid + k * PAIR_NT;
         poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
     }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-        const int q = tid + k * OFF_NT;
+        const int q = tid + k * PAIR_NT;
         moff[k] = (unsigned)wrapc(y0 - 1 + q / MW, ny, smy) * nx + wrapc(x0 - 1 + q % MW, nx, smx);
         mring[k] = q / MW * MX + q % MW + 1;
     }
@@ -246,7 +225,7 @@ __global__ void __launch_bounds__(OFF_NT, 3)
         float *d = mus + sm * MA;
 #pragma unroll
         for (int k = 0; k < KM; ++k) {
-            if (tid + k * OFF_NT >= MN) break;
+            if (tid + k * PAIR_NT >= MN) break;
             const int c = mring[k] + PX;  // one phi row further (halo 2 against 1)
             const float v = p0[c];
             const float fa = (p0[c + 1] - v) + (p0[c - 1] - v) + (p0[c + PX] - v) +
@@ -279,13 +258,13 @@ __global__ void __launch_bounds__(OFF_NT, 3)
         const unsigned zo = (unsigned)wrapc(z0 - 2 + d, nz, smz) * plane;
 #pragma unroll
         for (int k = 0; k < KP; ++k)
-            if (tid + k * OFF_NT < PA) phs[d * PA + tid + k * OFF_NT] = phif[zo + poff[k]];
+            if (tid + k * PAIR_NT < PA) phs[d * PA + tid + k * PAIR_NT] = phif[zo + poff[k]];
     }
     for (int d = 0; d < 3; ++d) {
         const unsigned zo = (unsigned)wrapc(z0 - 1 + d, nz, smz) * plane;
 #pragma unroll
         for (int k = 0; k < KM; ++k) {
-            if (tid + k * OFF_NT >= MN) break;
+            if (tid + k * PAIR_NT >= MN) break;
             float m6[6];
 #pragma unroll
             for (int c = 0; c < 6; ++c) m6[c] = __ldg(src.M + (c * N + zo + moff[k]));
@@ -317,15 +296,15 @@ __global__ void __launch_bounds__(OFF_NT, 3)
             float *d = phs + wrapr(sp + 4, RP) * PA + tid;
 #pragma unroll
             for (int k = 0; k < KP; ++k)
-                if (tid + k * OFF_NT < PA) cp_async4(d + k * OFF_NT, phif + (zo + poff[k]));
+                if (tid + k * PAIR_NT < PA) cp_async4(d + k * PAIR_NT, phif + (zo + poff[k]));
             const unsigned zm = (unsigned)wrapc(zz + 2, nz, smz) * plane;
 #pragma unroll
             for (int k = 0; k < KM; ++k) {
-                if (tid + k * OFF_NT >= MN) break;
+                if (tid + k * PAIR_NT >= MN) break;
                 const float *m = src.M + (zm + moff[k]);
 #pragma unroll
                 for (int c = 0; c < 6; ++c)
-                    cp_async4(mraw + c * MN + tid + k * OFF_NT, m + (size_t)c * N);
+                    cp_async4(mraw + c * MN + tid + k * PAIR_NT, m + (size_t)c * N);
             }
             cp_commit();
         }
@@ -363,11 +342,6 @@ __global__ void __launch_bounds__(OFF_NT, 3)
 
         // populations after streaming, rebuilt from offsets and source macros
         const int c0 = (ty + 1) * MX + 2 * tx + 2;  // ring index of the first node (even)
-        // the pair at ring index c, c + 1 of a plane (one 64-bit read where c is even)
-        auto pair_at = [&](const float *pl, int c, bool even) -> float2 {
-            if (even) return *reinterpret_cast<const float2 *>(pl + c);
-            return make_float2(pl[c], pl[c + 1]);
-        };
         const float2 sf2 = f2(s_f), sg2 = f2(s_g);
         float2 fv[19], gv[19];
         float2 flo;  // rest population minus its high word phi_hi
@@ -408,35 +382,12 @@ __global__ void __launch_bounds__(OFF_NT, 3)
         const float2 bp = sub2(phi, phi_hi);
         const float2 r = add2(sub2(phi_hi, sub2(phi, bp)), sub2(lo_sum, bp));
 
-        // Eq. gradient on D3Q19: (1/6) face differences + (1/12) edge differences
-        auto grad3 = [&](const float *m, const float *z, const float *p, int c, float2 out[3]) {
-            const int SX = PX;  // both rings have the same row stride
-            const float2 xe = pair_at(z, c + 1, false), xw_ = pair_at(z, c - 1, false);
-            const float2 yn = pair_at(z, c + SX, true), ys = pair_at(z, c - SX, true);
-            const float2 pc = pair_at(p, c, true), mc = pair_at(m, c, true);
-            const float2 ne = pair_at(z, c + SX + 1, false), nw = pair_at(z, c + SX - 1, false);
-            const float2 se = pair_at(z, c - SX + 1, false), sw = pair_at(z, c - SX - 1, false);
-            const float2 pe = pair_at(p, c + 1, false), pw = pair_at(p, c - 1, false);
-            const float2 me = pair_at(m, c + 1, false), mw = pair_at(m, c - 1, false);
-            const float2 pn = pair_at(p, c + SX, true), ps = pair_at(p, c - SX, true);
-            const float2 mn = pair_at(m, c + SX, true), ms = pair_at(m, c - SX, true);
-            const float2 k6 = f2(1.0f / 6.0f), k12 = f2(1.0f / 12.0f);
-            out[0] = fma2(k6, sub2(xe, xw_),
-                          mul2(k12, add2(add2(add2(sub2(ne, nw), sub2(se, sw)), sub2(pe, pw)),
-                                         sub2(me, mw))));
-            out[1] = fma2(k6, sub2(yn, ys),
-                          mul2(k12, add2(add2(add2(sub2(ne, se), sub2(nw, sw)), sub2(pn, ps)),
-                                         sub2(mn, ms))));
-            out[2] = fma2(k6, sub2(pc, mc),
-                          mul2(k12, add2(add2(add2(sub2(pe, me), sub2(pw, mw)), sub2(pn, mn)),
-                                         sub2(ps, ms))));
-        };
         const int cp = (ty + 2) * PX + 2 * tx + 2;
         const float *m0 = mus + sq0 * MA, *mm = mus + sq * MA, *mp = mus + sqp * MA;
         const float2 mu = pair_at(m0, c0, true);
         float2 gp[3], gm[3];
-        grad3(phs + sp * PA, phs + sp0 * PA, phs + spp * PA, cp, gp);
-        grad3(mm, m0, mp, c0, gm);
+        grad3_pair(phs + sp * PA, phs + sp0 * PA, phs + spp * PA, cp, PX, gp);
+        grad3_pair(mm, m0, mp, c0, MX, gm);
 
         float2 F[3], gr[3], u[3];
         const float2 dphi = sub2(phi, f2(P.phiv));
@@ -593,10 +544,10 @@ __global__ void __launch_bounds__(OFF_NT, 3)
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < KM; ++k) {  // own copies: no barrier needed
-            if (tid + k * OFF_NT >= MN) break;
+            if (tid + k * PAIR_NT >= MN) break;
             float m6[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MN + tid + k * OFF_NT];
+            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MN + tid + k * PAIR_NT];
             put_macros(sq, mring[k], m6);
         }
         // phi planes zz + 1 .. zz + 3 -> mu plane zz + 2 in the slot of zz - 1
@@ -616,7 +567,7 @@ __global__ void __launch_bounds__(OFF_NT, 3)
             d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
             d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
         }
-        constexpr int NW = OFF_NT / 32;
+        constexpr int NW = PAIR_NT / 32;
         __shared__ double red[7][NW];
         const int lane = tid & 31, wid = tid >> 5;
         if (lane == 0) {
@@ -859,7 +810,7 @@ int off_ctas_per_sm_t()
 {
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, d3q19_off_pass_kernel<C, PASS_STATE, true>, OFF_NT, 0);
+        &n, d3q19_off_pass_kernel<C, PASS_STATE, true>, PAIR_NT, 0);
     return e == cudaSuccess && n > 0 ? n : 2;
 }
 
