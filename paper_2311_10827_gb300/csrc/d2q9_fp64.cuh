@@ -20,7 +20,7 @@
 // About 153 FP64 operations per node against about 250 in the form shared with
 // the FP32 kernel before.  Measured with per-step launches, whole runs of 40
 // and 400 steps: 1024 x 1024 505 -> 363 us per step (the operations alone take
-// 255 us), 16 x 128 16.5 -> 9.9 us.
+// 255 us), 16 x 128 16.5 -> 9.9 us; with 64-column tiles 341 us.
 #pragma once
 
 // shared memory of one FP64 tile march
@@ -302,5 +302,170 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                d_bad = sm.bad ? 1.0 : 0.0;
         write_partial<NW>(sm.red, lin, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
                           a.partials + part);
+    }
+}
+
+// The FP64 time step of a grid too small to fill the chip.  A warp takes 64
+// cycles for any FP64 instruction, whatever its active lanes, and each of the
+// SM's four schedulers has one such pipe; with fewer warps than pipes the step
+// takes the operations of one warp, one after the other (7.2 us for the 177 of
+// two rows of d2q9_tile64).  Here a tile of 16 x 2 nodes is one CTA of four
+// warps, one per scheduler, that share the node update: every warp holds the 32
+// nodes and does a part of their operations, so that about 85 of them are in
+// sequence.  Each value is formed by the expressions of d2q9_tile64.  16 x 128:
+// 9.5 -> 5.1 us per step.
+//   1  phi of the tile and two halo rows and columns (one node per thread)
+//   2  v, d of one halo row                 warp 3: rho u's sum, sum of g
+//   3  mu of one halo row and column          (while 1 .. 3 run elsewhere)
+//   4  warp 0: F    warp 1: rho, 1/rho, 1/tau_g and what follows from them
+//      warp 2: 2 grad(phi)
+//   5  warp 0: f and S     warp 1: g along the axes
+//      warp 2, 3: g along one diagonal each, warp 3 the rest population
+constexpr int SM64_TX = 16, SM64_NT = 128;
+struct SmallSmem64 {
+    static constexpr int WP = SM64_TX + 4, WM = SM64_TX + 2;
+    double phs[6 * WP], vs[4 * WP], ds[4 * WP], mus[4 * WM];
+    double snz[32];               // sum of the moving f of the tile's nodes
+    double w[14][32];             // stage 2 .. 4 results per node
+};
+__global__ void __launch_bounds__(SM64_NT, 4)
+    d2q9_small64_kernel(const StepParams<double> P, PassArgs a)
+{
+    constexpr int TX = SM64_TX, WP = SmallSmem64::WP, WM = SmallSmem64::WM;
+    __shared__ SmallSmem64 sm;
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nx = P.nx, ny = P.ny;
+    const unsigned N = (unsigned)P.N;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * 2;
+    const double *__restrict__ fsrc = static_cast<const double *>(a.f_src);
+    const double *__restrict__ gsrc = static_cast<const double *>(a.g_src);
+    // this thread's node in stages 2 .. 5
+    const int tx = lane & 15, ty = lane >> 4;
+    const int xo = x0 + tx, yo = y0 + ty;
+    const bool ok = xo < nx && yo < ny;
+    const unsigned xO = wrapi(xo, nx), xOm = wrapi(xo - 1, nx), xOp = wrapi(xo + 1, nx);
+    const unsigned rm = (unsigned)wrapi(yo - 1, ny) * nx, r0 = (unsigned)wrapi(yo, ny) * nx,
+                   rp = (unsigned)wrapi(yo + 1, ny) * nx;
+    const unsigned n = r0 + xO;
+    double v[9], Sprev = 0.0;  // warp 0: the node's f; else its g
+    pull9<true>(warp == 0 ? fsrc : gsrc, N, rm, r0, rp, xOm, xO, xOp, v);
+    if (warp == 0) Sprev = __ldcs(static_cast<const double *>(a.S) + n);
+
+    if (tid < 6 * WP) {  // stage 1: ring rows y0 - 2 .. y0 + 3, columns x0 - 2 .. x0 + 17
+        const int r = tid / WP, c = tid - r * WP;
+        const int xx = x0 - 2 + c, yy = y0 - 2 + r;
+        const unsigned q0 = (unsigned)wrapi(yy, ny) * nx, qm = (unsigned)wrapi(yy - 1, ny) * nx,
+                       qp = (unsigned)wrapi(yy + 1, ny) * nx;
+        double h[9];
+        pull9<true>(fsrc, N, qm, q0, qp, (unsigned)wrapi(xx - 1, nx), (unsigned)wrapi(xx, nx),
+                    (unsigned)wrapi(xx + 1, nx), h);
+        const double s = sum_moving(h);
+        sm.phs[tid] = h[0] + s;
+        if (r >= 2 && r < 4 && c >= 2 && c < TX + 2) sm.snz[(r - 2) * 16 + c - 2] = s;
+    }
+    __syncthreads();
+    if (tid < 4 * WP) {  // stage 2: rows y0 - 1 .. y0 + 2 (ring rows 1 .. 4)
+        const double c = sm.phs[tid + WP], nn = sm.phs[tid + 2 * WP], ss = sm.phs[tid];
+        sm.vs[tid] = (nn - c) + (ss - c);
+        sm.ds[tid] = nn - ss;
+    }
+    if (warp == 3) {
+        const double ga = v[5] - v[7], gb = v[8] - v[6];
+        sm.w[0][lane] = (v[2] - v[4]) + (ga + gb);
+        sm.w[1][lane] = (v[3] - v[1]) + (ga - gb);
+        sm.w[2][lane] = sum_moving(v);
+    }
+    // (warp 3 joins the barrier of stage 2 late; stage 3 is 72 nodes of warps 0 .. 2)
+    __syncthreads();
+    if (tid < 4 * WM) {  // stage 3: the same rows, columns x0 - 1 .. x0 + 16
+        const int r = tid / WM, j = tid - r * WM + 1;
+        const double *p0 = sm.phs + (r + 1) * WP, *vr = sm.vs + r * WP;
+        const double c = p0[j];
+        const double h = (p0[j + 1] - c) + (p0[j - 1] - c);
+        const double t = c - P.phibar, hd = 0.5 * (P.phil - P.phiv);
+        double mu = ((4.0 * P.beta) * t) * fma(t, t, -(hd * hd));
+        mu = fma(-P.kappa, h, mu);
+        mu = fma(-(P.kappa * (2.0 / 3.0)), vr[j], mu);
+        sm.mus[tid] = fma(-(P.kappa * (1.0 / 6.0)), vr[j + 1] + vr[j - 1], mu);
+    }
+    __syncthreads();
+    const int j = tx + 2, k = tx + 1;
+    const double *p0 = sm.phs + (ty + 2) * WP, *vr = sm.vs + (ty + 1) * WP,
+                 *dr = sm.ds + (ty + 1) * WP;
+    const double *mm = sm.mus + ty * WM, *m0 = mm + WM, *mp = m0 + WM;
+    const double phi = p0[j];
+    if (warp == 0) {  // stage 4
+        const double da = mp[k + 1] - mm[k - 1], db = mm[k + 1] - mp[k - 1];
+        const double f3 = (-1.0 / 3.0) * phi;
+        sm.w[3][lane] = fma(f3, fma(0.25, da + db, m0[k + 1] - m0[k - 1]), P.G[0]);
+        sm.w[4][lane] = fma(f3, fma(0.25, da - db, mp[k] - mm[k]), P.G[1]);
+    } else if (warp == 1) {
+        const double dphi = phi - P.phiv;
+        const double rho = fma(P.drho, dphi, P.rhov);
+        const double taug = fma(3.0 * P.dnu, dphi, fma(3.0, P.nuv, 0.5));
+        const double inv = rcp64(rho * taug);
+        const double itg = inv * rho, it9 = (1.0 / 9.0) * itg, ri = rho * it9;
+        const double k9 = fma(-0.5, it9, 1.0 / 9.0);
+        sm.w[5][lane] = rho;
+        sm.w[6][lane] = inv * taug;
+        sm.w[7][lane] = itg;
+        sm.w[8][lane] = it9;
+        sm.w[9][lane] = ri;
+        sm.w[10][lane] = k9;
+    } else if (warp == 2) {
+        sm.w[11][lane] = fma(1.0 / 6.0, vr[j + 1] - vr[j - 1], p0[j + 1] - p0[j - 1]);
+        sm.w[12][lane] = fma(1.0 / 6.0, dr[j + 1] + dr[j - 1], (2.0 / 3.0) * dr[j]);
+    }
+    __syncthreads();
+    if (!ok) return;
+    // stage 5
+    const double Fx = sm.w[3][lane], Fy = sm.w[4][lane], irho = sm.w[6][lane];
+    const double qx = sm.w[11][lane], qy = sm.w[12][lane];
+    const double ux = fma(0.5, Fx, sm.w[0][lane]) * irho, uy = fma(0.5, Fy, sm.w[1][lane]) * irho;
+    const double S2 = fma(ux, qx, uy * qy);
+    double *__restrict__ fd = static_cast<double *>(a.f_dst);
+    double *__restrict__ gd = static_cast<double *>(a.g_dst);
+    if (warp == 0) {
+        static_cast<double *>(a.S_out)[n] = 0.5 * S2;
+        const double Sh = fma(0.75, S2, -0.5 * Sprev);
+        const double itf = P.inv_tauf, omf = 1.0 - itf;
+        const double z = (itf * P.alpha) * m0[k];
+        fd[n] = fma(itf, sm.snz[lane], fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, v[0])));
+        const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) fd[i * N + n] = fma(omf, v[i], i < 5 ? ka : kd);
+        return;
+    }
+    const double rho = sm.w[5][lane], itg = sm.w[7][lane], it9 = sm.w[8][lane],
+                 ri = sm.w[9][lane], k9 = sm.w[10][lane];
+    const double uu = fma(ux, ux, uy * uy), ruu = rho * uu;
+    const double p3 = 1.8 * fma(-2.0 / 3.0, ruu, fma(0.25 * P.drho, S2, sm.w[2][lane]));
+    const double A = fma(-1.5, ruu, p3), omg = 1.0 - itg;
+    const double e0 = it9 * A, e1 = 4.5 * ri, o1 = 3.0 * ri;
+    const double e2 = (1.5 * P.drho) * k9, o2 = 3.0 * k9;
+    auto pair = [&](double cu, double cF, double cq, double &s, double &d) {
+        const double E = fma(cu, fma(e2, cq, e1 * cu), e0);
+        const double O = fma(o2, cF, o1 * cu);
+        s = E + O;
+        d = E - O;
+    };
+    double s, d;
+    if (warp == 1) {
+        pair(ux, Fx, qx, s, d);
+        gd[2 * N + n] = fma(omg, v[2], s);
+        gd[4 * N + n] = fma(omg, v[4], d);
+        pair(uy, Fy, qy, s, d);
+        gd[3 * N + n] = fma(omg, v[3], s);
+        gd[1 * N + n] = fma(omg, v[1], d);
+    } else if (warp == 2) {
+        pair(ux + uy, Fx + Fy, qx + qy, s, d);
+        gd[5 * N + n] = fma(0.25, s, omg * v[5]);
+        gd[7 * N + n] = fma(0.25, d, omg * v[7]);
+    } else {
+        gd[n] = fma(omg, v[0], itg * fma(4.0 / 9.0, A, -p3));
+        pair(uy - ux, Fy - Fx, qy - qx, s, d);
+        gd[6 * N + n] = fma(0.25, s, omg * v[6]);
+        gd[8 * N + n] = fma(0.25, d, omg * v[8]);
     }
 }

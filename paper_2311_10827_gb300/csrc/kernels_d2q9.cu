@@ -1413,11 +1413,53 @@ cudaError_t seg_attrs()
     return e;
 }
 
+// Most tiles for which d2q9_small64_kernel is used: one per SM.  With two per SM
+// its schedulers hold two warps of about 85 operations each, no fewer than the
+// one warp of 177 that d2q9_tile64 gives them on such a grid, and more in all.
+constexpr int SM64_MAX_TILES = 152;
+
+// Rows per 64-column tile of an FP64 step.  A scheduler's FP64 pipe takes the
+// warps it holds one operation after the other, so a step takes the most tiles
+// that an SM gets times their operations: about 165 for two rows and 69 to
+// start a march, more where so few tiles share an SM that their barriers and
+// loads show (measured: one tile per SM 1.4, two 1.15).  64 columns rather than
+// 128 halve the warps per scheduler of a tile: 128 x 128 20.4 -> 14.5 us, 301 x 203
+// 43.7 -> 33.4, 512 x 512 101 -> 95, 1024 x 1024 350 -> 341 (multi-step launches).
+int rows64(int nx, int ny, int num_sms)
+{
+    const long long strips = (nx + 63) / 64, sms = num_sms > 0 ? num_sms : 152;
+    double best = 0.0;
+    int rows = 2;
+    for (int r = 2; r <= 64; r += 2) {
+        const long long k = (strips * ((ny + r - 1) / r) + sms - 1) / sms;
+        const double alone = k == 1 ? 1.4 : (k == 2 ? 1.15 : (k == 3 ? 1.08 : (k == 4 ? 1.05 : 1.0)));
+        const double cost = (double)k * (r / 2 * 165 + 69) * alone;
+        if (r == 2 || cost < best) {
+            best = cost;
+            rows = r;
+        }
+    }
+    return rows;
+}
+
 template <typename T, int PASS>
 cudaError_t launch_pass(const void *params, const PassArgs &a, const LaunchShape &s,
                         cudaStream_t st)
 {
     const StepParams<T> &P = *static_cast<const StepParams<T> *>(params);
+    if constexpr (sizeof(T) == 8 && !(PASS & (PASS_DIAG | PASS_MACROS))) {
+        if constexpr (PASS == PASS_STATE) {
+            const dim3 tiles((P.nx + SM64_TX - 1) / SM64_TX, (P.ny + 1) / 2);
+            if (tiles.x * (long long)tiles.y <= SM64_MAX_TILES)
+                return launch_pdl(d2q9_small64_kernel, tiles, SM64_NT, 0, st, P, a);
+        }
+        // no partial records: the tiles need not be those of `s`
+        const int rows = rows64(P.nx, P.ny, s.num_sms);
+        const dim3 tiles((P.nx + 63) / 64, (P.ny + rows - 1) / rows);
+        if (tiles.y <= 65535)
+            return launch_pdl(d2q9_pass_kernel<T, 64, PASS>, tiles, dim3(64, TYB),
+                              tile_dyn_bytes<T, 64>(), st, P, a, rows);
+    }
     constexpr int dyn = tile_dyn_bytes<T, TXW>();
     dim3 grid(s.grid_x, s.grid_y), block(TXW, TYB);
     return launch_pdl(d2q9_pass_kernel<T, TXW, PASS>, grid, block, dyn, st, P, a, s.rows);
@@ -1544,6 +1586,7 @@ LaunchShape d2q9_shape(int nx, int ny, int num_sms)
 {
     LaunchShape s;
     s.variant = TXW;
+    s.num_sms = num_sms;
     s.grid_x = (nx + TXW - 1) / TXW;
     // one wave of resident CTAs (4 per SM at the FP32 register budget) when
     // the grid allows it; rows even (two rows per iteration).  Small grids

@@ -153,6 +153,7 @@ struct LaunchShape {
     int grid_x, grid_y;
     int nblocks;
     int variant;   // kernel variant (strip width) where several exist
+    int num_sms;   // D2Q9: the device's SMs
 };
 
 // One grid of a batch (device-resident table): parameters in both

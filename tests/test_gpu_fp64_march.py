@@ -49,3 +49,44 @@ def test_fp64_march_against_oracle(oracle_mod, shape):
     assert abs(d["sum_phi"] - d6["sum_phi"]) <= 1e-12 * abs(d6["sum_phi"]) + N * atol
     assert abs(d["u_max"] - d6["umax"]) <= 1e-12 * d6["umax"] + 4 * atol
     s.close()
+
+
+@pytest.mark.parametrize("shape", [(16, 128), (17, 33), (31, 2), (1, 1), (3, 5), (48, 50), (150, 29),
+                                   (2431, 1)])
+def test_small_grid_kernel_equals_march(oracle_mod, shape):
+    """Grids of at most 152 tiles of 16 x 2 nodes take a kernel that splits the
+    node update over four warps.  Its expressions are those of the tile march,
+    which the same flow takes when it is repeated in y (periodic) until it has
+    more tiles: the same bits, and the oracle's step within the FP64 bound."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_10827_gb300 import build, sim
+    build.build()
+    nx, ny = shape
+    tiles = lambda h: ((nx + 15) // 16) * ((h + 1) // 2)  # noqa: E731
+    times = 1
+    while tiles(ny * times) <= 152:
+        times += 1
+    assert tiles(ny) <= 152
+    o = oracle_mod.Oracle(shape, **PRM)
+    o.init_phi(wl.droplet(nx, ny, 0.3 * min(nx, ny) + 1.0, 4.0))
+    f, g, S = o.get_state()
+    g = g + wl.perturbed_state(g.shape, 1e-3, 13)
+    S = S + wl.perturbed_state(S.shape, 1e-4, 14)
+    o.set_state(f, g, S, 0)
+    rep = lambda a: np.concatenate([a.reshape(-1, ny, nx)] * times, axis=1)  # noqa: E731
+    a = sim.Simulation(shape, precision="fp64", **PRM)
+    b = sim.Simulation((nx, ny * times), precision="fp64", **PRM)
+    a.set_state(f, g, S, 0)
+    b.set_state(rep(f), rep(g), rep(S), 0)
+    a.step(5)
+    b.step(5)
+    o.step(5)
+    got, ref = a.get_state(), o.get_state()
+    atol = 1e-14 * max(np.abs(ref[0]).max(), np.abs(ref[1]).max())
+    for x, y, z in zip(got, b.get_state(), ref):
+        assert np.array_equal(rep(x).ravel(), y.ravel())
+        assert np.abs(x - z).max() <= 1e-12 * np.abs(z).max() + atol
+    a.close()
+    b.close()
