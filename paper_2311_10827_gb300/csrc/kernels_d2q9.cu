@@ -345,6 +345,195 @@ __device__ __forceinline__ bool seg_ok(int nx, const void *f, const void *g, con
            (((unsigned long long)f | (unsigned long long)g | (unsigned long long)S) & 15) == 0;
 }
 
+// The update of one node (FP32): its moments, forces, both collisions and the
+// stores (or the moments and diagnostics that PASS asks for).  pm, p0, pp and
+// mm, m0, mp: the phi and mu rows at y - 1, y, y + 1, the own column at j and k;
+// f, lo: the pulled populations of f (rest population as a pair); gv: those of g;
+// n: the node's index.
+template <typename T, int PASS, int NT>
+__device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs &a, const T *pm,
+                              const T *p0, const T *pp, const T *mm, const T *m0,
+                              const T *mp, int j, int k, const T fcur[9], T locur,
+                              const T gv[9], T Sprev, T a_src, T a_dst, unsigned n,
+                              int lin, T (*dacc)[NT], T (*facc)[NT], int *dbad)
+{
+    constexpr bool REST_PAIR = true;
+    const unsigned N = (unsigned)P.N;
+    // phi from the pulled values (Eq. order-parameter)
+    const T snz = sum_moving(fcur);
+    const T phi = fcur[0] + (locur + snz);
+    const T mu = m0[k];
+    T gpx, gpy, Fx, Fy, rho, inv_rho, itg, ux, uy, grx, gry, ugr, uu, S;
+    // Eq. gradient: grad = 3 sum_{i!=0} w_i c_i Psi(x + c_i)
+    //   = (1/3)(axis differences) + (1/12)(diagonal differences)
+    {
+        // x and y components as the two lanes of paired instructions
+        const float2 gp = fma2(
+            f2(1.0f / 3.0f), sub2(make_float2(p0[j + 1], pp[j]), make_float2(p0[j - 1], pm[j])),
+            mul2(f2(1.0f / 12.0f),
+                 add2(sub2(make_float2(pp[j + 1], pp[j + 1]), make_float2(pp[j - 1], pm[j + 1])),
+                      sub2(make_float2(pm[j + 1], pp[j - 1]), make_float2(pm[j - 1], pm[j - 1])))));
+        const float2 gm = fma2(
+            f2(1.0f / 3.0f), sub2(make_float2(m0[k + 1], mp[k]), make_float2(m0[k - 1], mm[k])),
+            mul2(f2(1.0f / 12.0f),
+                 add2(sub2(make_float2(mp[k + 1], mp[k + 1]), make_float2(mp[k - 1], mm[k + 1])),
+                      sub2(make_float2(mm[k + 1], mp[k - 1]), make_float2(mm[k - 1], mm[k - 1])))));
+        gpx = gp.x;
+        gpy = gp.y;
+        // F = -phi grad(mu) + G; rho, nu linear in phi (Eq. vis)
+        const float2 F = fma2(f2(-phi), gm, make_float2(P.G[0], P.G[1]));
+        Fx = F.x;
+        Fy = F.y;
+        const float2 rn = fma2(f2(phi - P.phiv), make_float2(P.drho, P.dnu),
+                               make_float2(P.rhov, P.nuv));
+        rho = rn.x;
+        inv_rho = Arith<T>::rcp(rho);
+        itg = Arith<T>::rcp(fmaf(3.0f, rn.y, 0.5f));  // nu = cs2 (tau_g - 1/2)
+        // rho u = sum_i c_i g_i + F/2
+        const float jx = (gv[2] - gv[4]) + ((gv[5] - gv[6]) + (gv[8] - gv[7]));
+        const float jy = (gv[3] - gv[1]) + ((gv[5] + gv[6]) - (gv[7] + gv[8]));
+        const float2 u = mul2(fma2(f2(0.5f), F, make_float2(jx, jy)), f2(inv_rho));
+        ux = u.x;
+        uy = u.y;
+        const float2 gr = mul2(f2(P.drho), gp);  // grad rho (chain rule)
+        grx = gr.x;
+        gry = gr.y;
+        // u.grad(rho) and S = u.grad(phi) as the two lanes
+        const float2 us = fma2(f2(ux), make_float2(grx, gpx), mul2(f2(uy), make_float2(gry, gpy)));
+        ugr = us.x;
+        S = us.y;
+        uu = fmaf(ux, ux, uy * uy);
+    }
+    // p = cs2/(1-w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0(u)],
+    // rho s_0 = -(2/3) rho |u|^2 for D2Q9
+    const T p = T(0.6) * (sum_moving(gv) + T(0.5) * ugr - T(2.0 / 3.0) * rho * uu);
+
+    if (PASS & PASS_DIAG) {
+        {
+            // (hi, lo) += x with an exact two-sum on the high word
+            auto acc2 = [&](int q, float x) {
+                const float hi = dacc[q][lin];
+                const float s = hi + x, bp = s - hi;
+                dacc[q + 1][lin] += (hi - (s - bp)) + (x - bp);
+                dacc[q][lin] = s;
+            };
+            acc2(0, phi);
+            acc2(2, 0.5f * rho * uu);
+            acc2(4, S);
+            acc2(6, Sprev);
+        }
+        facc[0][lin] = fmax(facc[0][lin], uu);
+        facc[1][lin] = fmin(facc[1][lin], mu);
+        facc[2][lin] = fmax(facc[2][lin], mu);
+        if (!isfinite(phi) || !isfinite(p) || !isfinite(uu) || !isfinite(mu)) *dbad = 1;
+    }
+    if (PASS & PASS_MACROS) {
+        if (a.out_phi) a.out_phi[n] = (double)phi;
+        if (a.out_p) a.out_p[n] = (double)p;
+        if (a.out_mu) a.out_mu[n] = (double)mu;
+        if (a.out_u) {
+            a.out_u[n] = (double)ux;
+            a.out_u[(size_t)N + n] = (double)uy;
+        }
+    }
+    if (PASS & PASS_MACROS_T) {
+        static_cast<T *>(a.mt_phi)[n] = phi;
+        static_cast<T *>(a.mt_p)[n] = p;
+        static_cast<T *>(a.mt_mu)[n] = mu;
+        static_cast<T *>(a.mt_u)[n] = ux;
+        static_cast<T *>(a.mt_u)[(size_t)N + n] = uy;
+    }
+    if (PASS & PASS_STATE) {
+        T *__restrict__ fd = static_cast<T *>(a.f_dst);
+        T *__restrict__ gd = static_cast<T *>(a.g_dst);
+        st_stream(static_cast<T *>(a.S_out) + n, S);
+
+        // CH population, Eq. BGK with Eq. H_i and Eq. F_i:
+        // f* = f - (f - f^eq)/tau_f + w_i b_i (1.5 S - 0.5 S_prev),
+        // b = -2, -1/2, 1 (rest, axis, diagonal); f_0 - f_0^eq is formed
+        // as (5/9) alpha mu - sum_{i!=0} f_i (no cancellation against phi).
+        // Every population is updated by its own small increment, so
+        // the increments sum to sum_i F_i up to unbiased rounding (the
+        // form f (1 - 1/tau) + f^eq/tau would add (1 - 1/tau + 1/tau - 1)
+        // sum_{i!=0} f_i, a systematic FP32 drift of the phi mass).
+        const T Sh = fmaf(T(1.5), S, -(T(0.5) * Sprev));
+        // alpha mu in the source buffer's shifted variables; dsh moves
+        // the written values to the target shift (0 unless it changed)
+        const T am = P.alpha * mu - a_src;
+        const T dsh = a_src - a_dst;
+        const T itf = P.inv_tauf;
+        {
+            // f_0* = f_0 - (f_0 - f_0^eq)/tau_f - (8/9) Sh with
+            // f_0 - f_0^eq = (5/9) alpha mu - sum_{i!=0} f_i
+            const T d0 = -(T(5.0 / 9.0) * am - snz) * itf - T(8.0 / 9.0) * Sh -
+                         T(5.0 / 9.0) * dsh;
+            if (REST_PAIR) {
+                // (hi, lo) + d0 with an exact two-sum on the high word
+                const T sl = locur + d0;
+                const T hi = fcur[0] + sl;
+                const T bp = hi - fcur[0];
+                const T lo = (fcur[0] - (hi - bp)) + (sl - bp);
+                st_stream(fd + n, hi);
+                st_stream(fd + (9u * N + n), lo);
+            } else {
+                st_stream(fd + n, fcur[0] + d0);
+            }
+        }
+        const T ea = T(1.0 / 9.0) * am, ed = T(1.0 / 36.0) * am;
+        // (explicit multiply-adds: every kernel that inlines this rounds alike)
+        const T sa = fmaf(T(-1.0 / 18.0), Sh, T(1.0 / 9.0) * dsh);
+        const T sd = fmaf(T(1.0 / 36.0), Sh, T(1.0 / 36.0) * dsh);
+        // Hydrodynamic population, Eq. BGK-NS with Eqs. G_i, Siu, GGi:
+        // g* = g + (g^eq - g)/tau_g + G_i.  With A = 3p - 1.5 rho |u|^2,
+        // g^eq_i = w_i [A + 4.5 rho (c.u)^2] + 3 w_i rho (c.u) (i != 0), and
+        // G_i = (1 - 1/(2 tau_g)) w_i [u.grad rho + c.F/cs2
+        //       + ((c.u)(c.grad rho) - cs2 u.grad rho)/cs2]
+        //     = 3 w_i k [c.F + (c.u)(c.grad rho)], k = 1 - 1/(2 tau_g)
+        // (the two u.grad rho terms cancel).  Opposite directions share
+        // the even part and flip the odd part.
+        const T kg = T(1) - T(0.5) * itg;
+        const T A = fmaf(-(T(1.5) * rho), uu, T(3) * p);
+        st_stream(gd + n, gv[0] + ((T(4.0 / 9.0) * A - T(3) * p) - gv[0]) * itg);  // G_0 = 0
+        {
+            // two populations per paired instruction: f 1..4 and 5..8 in
+            // pairs; g the two axis and the two diagonal direction pairs
+            const float2 it2 = f2(itf);
+#pragma unroll
+            for (int i = 1; i <= 7; i += 2) {
+                const float2 v = make_float2(fcur[i], fcur[i + 1]);
+                const float2 o = add2(v, fma2(sub2(f2(i < 5 ? ea : ed), v), it2,
+                                              f2(i < 5 ? sa : sd)));
+                st_stream(fd + (i * N + n), o.x);
+                st_stream(fd + ((i + 1) * N + n), o.y);
+            }
+            const float2 itg2 = f2(itg), A2 = f2(A), r45 = f2(4.5f * rho);
+#pragma unroll
+            for (int grp = 0; grp < 2; ++grp) {
+                // lanes: directions (2, 3) / (4, 1) on the axes, (5, 6) / (7, 8) on the diagonals
+                const float w = grp == 0 ? 1.0f / 9.0f : 1.0f / 36.0f;
+                const float2 cu = grp == 0 ? make_float2(ux, uy) : make_float2(ux + uy, uy - ux);
+                const float2 cF = grp == 0 ? make_float2(Fx, Fy) : make_float2(Fx + Fy, Fy - Fx);
+                const float2 cg = grp == 0 ? make_float2(grx, gry)
+                                           : make_float2(grx + gry, gry - grx);
+                const int p0i = grp == 0 ? 2 : 5, p1i = grp == 0 ? 3 : 6;
+                const int m0i = grp == 0 ? 4 : 7, m1i = grp == 0 ? 1 : 8;
+                const float2 eq_s = mul2(f2(w), fma2(mul2(r45, cu), cu, A2));
+                const float2 eq_a = mul2(f2(3.0f * w * rho), cu);
+                const float2 wk = f2(3.0f * w * kg);
+                const float2 G_s = mul2(mul2(wk, cu), cg), G_a = mul2(wk, cF);
+                const float2 gp = make_float2(gv[p0i], gv[p1i]);
+                const float2 gm = make_float2(gv[m0i], gv[m1i]);
+                const float2 op = add2(gp, fma2(sub2(add2(eq_s, eq_a), gp), itg2, add2(G_s, G_a)));
+                const float2 om = add2(gm, fma2(sub2(sub2(eq_s, eq_a), gm), itg2, sub2(G_s, G_a)));
+                st_stream(gd + (p0i * N + n), op.x);
+                st_stream(gd + (p1i * N + n), op.y);
+                st_stream(gd + (m0i * N + n), om.x);
+                st_stream(gd + (m1i * N + n), om.y);
+            }
+        }
+    }
+}
+
 // One tile: columns [x0, x0 + TX), rows [y0, yend), marching in direction
 // dir (+1 down from y0, -1 up from yend - 1); diagnostics partial record
 // `part` (PASS_DIAG).  Shared by the single-grid and the batched kernels.
@@ -651,190 +840,9 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                 for (int i = 0; i < 9; ++i) gv[i] = G[i * SL::W + tx + 4 - cxv(i)];
                 if (STAGE_S) Sprev = stg[st * SL::STAGE + SL::SOFF + ty * TX + tx];
             }
-            const T *pm = phs + sm * WP;
-            const T *p0 = phs + s0 * WP;
-            const T *pp = phs + sp * WP;
-            const T *mm = mus + sm * WM;
-            const T *m0 = mus + s0 * WM;
-            const T *mp = mus + sp * WM;
-            const int j = tx + 2;  // phi ring index of the own column
-            const int k = tx + 1;  // mu ring index of the own column
-
-            // phi from the pulled values (Eq. order-parameter)
-            const T snz = sum_moving(fcur);
-            const T phi = fcur[0] + (locur + snz);
-            const T mu = m0[k];
-            T gpx, gpy, Fx, Fy, rho, inv_rho, itg, ux, uy, grx, gry, ugr, uu, S;
-            // Eq. gradient: grad = 3 sum_{i!=0} w_i c_i Psi(x + c_i)
-            //   = (1/3)(axis differences) + (1/12)(diagonal differences)
-            {
-                // x and y components as the two lanes of paired instructions
-                const float2 gp = fma2(
-                    f2(1.0f / 3.0f), sub2(make_float2(p0[j + 1], pp[j]), make_float2(p0[j - 1], pm[j])),
-                    mul2(f2(1.0f / 12.0f),
-                         add2(sub2(make_float2(pp[j + 1], pp[j + 1]), make_float2(pp[j - 1], pm[j + 1])),
-                              sub2(make_float2(pm[j + 1], pp[j - 1]), make_float2(pm[j - 1], pm[j - 1])))));
-                const float2 gm = fma2(
-                    f2(1.0f / 3.0f), sub2(make_float2(m0[k + 1], mp[k]), make_float2(m0[k - 1], mm[k])),
-                    mul2(f2(1.0f / 12.0f),
-                         add2(sub2(make_float2(mp[k + 1], mp[k + 1]), make_float2(mp[k - 1], mm[k + 1])),
-                              sub2(make_float2(mm[k + 1], mp[k - 1]), make_float2(mm[k - 1], mm[k - 1])))));
-                gpx = gp.x;
-                gpy = gp.y;
-                // F = -phi grad(mu) + G; rho, nu linear in phi (Eq. vis)
-                const float2 F = fma2(f2(-phi), gm, make_float2(P.G[0], P.G[1]));
-                Fx = F.x;
-                Fy = F.y;
-                const float2 rn = fma2(f2(phi - P.phiv), make_float2(P.drho, P.dnu),
-                                       make_float2(P.rhov, P.nuv));
-                rho = rn.x;
-                inv_rho = Arith<T>::rcp(rho);
-                itg = Arith<T>::rcp(fmaf(3.0f, rn.y, 0.5f));  // nu = cs2 (tau_g - 1/2)
-                // rho u = sum_i c_i g_i + F/2
-                const float jx = (gv[2] - gv[4]) + ((gv[5] - gv[6]) + (gv[8] - gv[7]));
-                const float jy = (gv[3] - gv[1]) + ((gv[5] + gv[6]) - (gv[7] + gv[8]));
-                const float2 u = mul2(fma2(f2(0.5f), F, make_float2(jx, jy)), f2(inv_rho));
-                ux = u.x;
-                uy = u.y;
-                const float2 gr = mul2(f2(P.drho), gp);  // grad rho (chain rule)
-                grx = gr.x;
-                gry = gr.y;
-                // u.grad(rho) and S = u.grad(phi) as the two lanes
-                const float2 us = fma2(f2(ux), make_float2(grx, gpx), mul2(f2(uy), make_float2(gry, gpy)));
-                ugr = us.x;
-                S = us.y;
-                uu = fmaf(ux, ux, uy * uy);
-            }
-            // p = cs2/(1-w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0(u)],
-            // rho s_0 = -(2/3) rho |u|^2 for D2Q9
-            const T p = T(0.6) * (sum_moving(gv) + T(0.5) * ugr - T(2.0 / 3.0) * rho * uu);
-
-            if (PASS & PASS_DIAG) {
-                {
-                    // (hi, lo) += x with an exact two-sum on the high word
-                    auto acc2 = [&](int q, float x) {
-                        const float hi = dacc[q][lin];
-                        const float s = hi + x, bp = s - hi;
-                        dacc[q + 1][lin] += (hi - (s - bp)) + (x - bp);
-                        dacc[q][lin] = s;
-                    };
-                    acc2(0, phi);
-                    acc2(2, 0.5f * rho * uu);
-                    acc2(4, S);
-                    acc2(6, Sprev);
-                }
-                facc[0][lin] = fmax(facc[0][lin], uu);
-                facc[1][lin] = fmin(facc[1][lin], mu);
-                facc[2][lin] = fmax(facc[2][lin], mu);
-                if (!isfinite(phi) || !isfinite(p) || !isfinite(uu) || !isfinite(mu)) *dbad = 1;
-            }
-            if (PASS & PASS_MACROS) {
-                const size_t n = (size_t)nrow + xo;
-                if (a.out_phi) a.out_phi[n] = (double)phi;
-                if (a.out_p) a.out_p[n] = (double)p;
-                if (a.out_mu) a.out_mu[n] = (double)mu;
-                if (a.out_u) {
-                    a.out_u[n] = (double)ux;
-                    a.out_u[(size_t)N + n] = (double)uy;
-                }
-            }
-            if (PASS & PASS_MACROS_T) {
-                const size_t n = (size_t)nrow + xo;
-                static_cast<T *>(a.mt_phi)[n] = phi;
-                static_cast<T *>(a.mt_p)[n] = p;
-                static_cast<T *>(a.mt_mu)[n] = mu;
-                static_cast<T *>(a.mt_u)[n] = ux;
-                static_cast<T *>(a.mt_u)[(size_t)N + n] = uy;
-            }
-            if (PASS & PASS_STATE) {
-                const unsigned n = nrow + xo;
-                T *__restrict__ fd = static_cast<T *>(a.f_dst);
-                T *__restrict__ gd = static_cast<T *>(a.g_dst);
-                st_stream(static_cast<T *>(a.S_out) + n, S);
-
-                // CH population, Eq. BGK with Eq. H_i and Eq. F_i:
-                // f* = f - (f - f^eq)/tau_f + w_i b_i (1.5 S - 0.5 S_prev),
-                // b = -2, -1/2, 1 (rest, axis, diagonal); f_0 - f_0^eq is formed
-                // as (5/9) alpha mu - sum_{i!=0} f_i (no cancellation against phi).
-                // Every population is updated by its own small increment, so
-                // the increments sum to sum_i F_i up to unbiased rounding (the
-                // form f (1 - 1/tau) + f^eq/tau would add (1 - 1/tau + 1/tau - 1)
-                // sum_{i!=0} f_i, a systematic FP32 drift of the phi mass).
-                const T Sh = T(1.5) * S - T(0.5) * Sprev;
-                // alpha mu in the source buffer's shifted variables; dsh moves
-                // the written values to the target shift (0 unless it changed)
-                const T am = P.alpha * mu - a_src;
-                const T dsh = a_src - a_dst;
-                const T itf = P.inv_tauf;
-                {
-                    // f_0* = f_0 - (f_0 - f_0^eq)/tau_f - (8/9) Sh with
-                    // f_0 - f_0^eq = (5/9) alpha mu - sum_{i!=0} f_i
-                    const T d0 = -(T(5.0 / 9.0) * am - snz) * itf - T(8.0 / 9.0) * Sh -
-                                 T(5.0 / 9.0) * dsh;
-                    if (REST_PAIR) {
-                        // (hi, lo) + d0 with an exact two-sum on the high word
-                        const T sl = locur + d0;
-                        const T hi = fcur[0] + sl;
-                        const T bp = hi - fcur[0];
-                        const T lo = (fcur[0] - (hi - bp)) + (sl - bp);
-                        st_stream(fd + n, hi);
-                        st_stream(fd + (9u * N + n), lo);
-                    } else {
-                        st_stream(fd + n, fcur[0] + d0);
-                    }
-                }
-                const T ea = T(1.0 / 9.0) * am, ed = T(1.0 / 36.0) * am;
-                const T sa = T(-1.0 / 18.0) * Sh + T(1.0 / 9.0) * dsh;
-                const T sd = T(1.0 / 36.0) * Sh + T(1.0 / 36.0) * dsh;
-                // Hydrodynamic population, Eq. BGK-NS with Eqs. G_i, Siu, GGi:
-                // g* = g + (g^eq - g)/tau_g + G_i.  With A = 3p - 1.5 rho |u|^2,
-                // g^eq_i = w_i [A + 4.5 rho (c.u)^2] + 3 w_i rho (c.u) (i != 0), and
-                // G_i = (1 - 1/(2 tau_g)) w_i [u.grad rho + c.F/cs2
-                //       + ((c.u)(c.grad rho) - cs2 u.grad rho)/cs2]
-                //     = 3 w_i k [c.F + (c.u)(c.grad rho)], k = 1 - 1/(2 tau_g)
-                // (the two u.grad rho terms cancel).  Opposite directions share
-                // the even part and flip the odd part.
-                const T kg = T(1) - T(0.5) * itg;
-                const T A = T(3) * p - T(1.5) * rho * uu;
-                st_stream(gd + n, gv[0] + ((T(4.0 / 9.0) * A - T(3) * p) - gv[0]) * itg);  // G_0 = 0
-                {
-                    // two populations per paired instruction: f 1..4 and 5..8 in
-                    // pairs; g the two axis and the two diagonal direction pairs
-                    const float2 it2 = f2(itf);
-#pragma unroll
-                    for (int i = 1; i <= 7; i += 2) {
-                        const float2 v = make_float2(fcur[i], fcur[i + 1]);
-                        const float2 o = add2(v, fma2(sub2(f2(i < 5 ? ea : ed), v), it2,
-                                                      f2(i < 5 ? sa : sd)));
-                        st_stream(fd + (i * N + n), o.x);
-                        st_stream(fd + ((i + 1) * N + n), o.y);
-                    }
-                    const float2 itg2 = f2(itg), A2 = f2(A), r45 = f2(4.5f * rho);
-#pragma unroll
-                    for (int grp = 0; grp < 2; ++grp) {
-                        // lanes: directions (2, 3) / (4, 1) on the axes, (5, 6) / (7, 8) on the diagonals
-                        const float w = grp == 0 ? 1.0f / 9.0f : 1.0f / 36.0f;
-                        const float2 cu = grp == 0 ? make_float2(ux, uy) : make_float2(ux + uy, uy - ux);
-                        const float2 cF = grp == 0 ? make_float2(Fx, Fy) : make_float2(Fx + Fy, Fy - Fx);
-                        const float2 cg = grp == 0 ? make_float2(grx, gry)
-                                                   : make_float2(grx + gry, gry - grx);
-                        const int p0i = grp == 0 ? 2 : 5, p1i = grp == 0 ? 3 : 6;
-                        const int m0i = grp == 0 ? 4 : 7, m1i = grp == 0 ? 1 : 8;
-                        const float2 eq_s = mul2(f2(w), fma2(mul2(r45, cu), cu, A2));
-                        const float2 eq_a = mul2(f2(3.0f * w * rho), cu);
-                        const float2 wk = f2(3.0f * w * kg);
-                        const float2 G_s = mul2(mul2(wk, cu), cg), G_a = mul2(wk, cF);
-                        const float2 gp = make_float2(gv[p0i], gv[p1i]);
-                        const float2 gm = make_float2(gv[m0i], gv[m1i]);
-                        const float2 op = add2(gp, fma2(sub2(add2(eq_s, eq_a), gp), itg2, add2(G_s, G_a)));
-                        const float2 om = add2(gm, fma2(sub2(sub2(eq_s, eq_a), gm), itg2, sub2(G_s, G_a)));
-                        st_stream(gd + (p0i * N + n), op.x);
-                        st_stream(gd + (p1i * N + n), op.y);
-                        st_stream(gd + (m0i * N + n), om.x);
-                        st_stream(gd + (m1i * N + n), om.y);
-                    }
-                }
-            }
+            d2q9_node<T, PASS, NT>(P, a, phs + sm * WP, phs + s0 * WP, phs + sp * WP, mus + sm * WM,
+                                   mus + s0 * WM, mus + sp * WM, tx + 2, tx + 1, fcur, locur, gv,
+                                   Sprev, a_src, a_dst, nrow + xo, lin, dacc, facc, dbad);
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) fcur[i] = fnext[i];
@@ -893,6 +901,93 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     unsigned bph = 0;  // no bulk staging here
     run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, blockIdx.x * TX, y0,
                            min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + blockIdx.x, bph);
+}
+
+// The FP32 step of a small or mid-sized grid: one 64 x 4 tile per CTA of as many
+// threads, without a march.  On such grids d2q9_pass_kernel runs marches of one
+// or two iterations, whose start (two phi rows at a time, each with its own
+// wait for its loads) takes longer than the iterations; here every load of the
+// tile is issued at the start, and the phi rows beside it are shared by four
+// output rows instead of two.  32 x 8 tiles (fewer halo values, spread evenly)
+// took 2.7 against 2.4 us at 32 x 32 and 8.3 against 8.0 at 512 x 512; five CTAs
+// per SM (48 registers, spills) 2.7 and 8.5.
+constexpr int SHX = 64, SHY = 4;
+struct ShotSmem {
+    static constexpr int WP = SHX + 4, WM = SHX + 2;
+    float phs[(SHY + 4) * WP];
+    float mus[(SHY + 2) * WM];
+};
+template <int PASS>
+__global__ void __launch_bounds__(SHX *SHY, 4)
+    d2q9_shot_kernel(const StepParams<float> P, PassArgs a)
+{
+    constexpr int WP = ShotSmem::WP, WM = ShotSmem::WM, NT = SHX * SHY;
+    __shared__ ShotSmem sm;
+    pdl_wait();
+    const int tx = threadIdx.x, ty = threadIdx.y, lin = ty * SHX + tx;
+    const int nx = P.nx, ny = P.ny;
+    const unsigned N = (unsigned)P.N;
+    const bool small = ny < 8;
+    const int x0 = blockIdx.x * SHX, y0 = blockIdx.y * SHY;
+    const float *__restrict__ fsrc = static_cast<const float *>(a.f_src);
+    const float *__restrict__ gsrc = static_cast<const float *>(a.g_src);
+    const int xo = x0 + tx, yo = y0 + ty;
+    const bool ok = xo < nx && yo < ny;
+    const unsigned xO = wrapi(xo, nx), xOm = wrapi(xo - 1, nx), xOp = wrapi(xo + 1, nx);
+    float a_src = 0.0f, a_dst = 0.0f;
+    if (PASS & PASS_STATE) {
+        a_src = *a.eqs_src;
+        a_dst = *a.eqs_target;
+        if (a.eqs_dst && blockIdx.x == 0 && blockIdx.y == 0 && lin == 0) *a.eqs_dst = a_dst;
+    }
+    auto pull = [&](const float *s, int y, unsigned xm, unsigned x, unsigned xp, float v[9],
+                    float *lo) {
+        const unsigned rm = (unsigned)wrap_row(y - 1, ny, small) * nx;
+        const unsigned r0 = (unsigned)wrap_row(y, ny, small) * nx;
+        const unsigned rp = (unsigned)wrap_row(y + 1, ny, small) * nx;
+        pull9<true>(s, N, rm, r0, rp, xm, x, xp, v);
+        if (lo) *lo = __ldg(s + (9u * N + r0 + x));
+    };
+    // own row; a row above or below the tile; columns beside it (the last warp:
+    // 8 rows x 4 columns); the own node's g and S
+    float f[9], h[9], gv[9], lo, hlo, Sprev = 0.0f;
+    const int hy = ty < 2 ? ty : ty + 4;  // ring row of the halo row: 0, 1, 6, 7
+    pull(fsrc, yo, xOm, xO, xOp, f, &lo);
+    pull(fsrc, y0 - 2 + hy, xOm, xO, xOp, h, &hlo);
+    const int e = lin - (NT - 32), ey = e >> 2, ej = (e & 3) < 2 ? (e & 3) : SHX + (e & 3);
+    if (e >= 0) {
+        const int c = x0 - 2 + ej;
+        float q[9], qlo;
+        pull(fsrc, y0 - 2 + ey, wrapi(c - 1, nx), wrapi(c, nx), wrapi(c + 1, nx), q, &qlo);
+        sm.phs[ey * WP + ej] = q[0] + (qlo + sum_moving(q));
+    }
+    pull(gsrc, yo, xOm, xO, xOp, gv, nullptr);
+    const unsigned n = (unsigned)wrap_row(yo, ny, small) * nx + xO;
+    if (PASS & PASS_STATE) Sprev = __ldcs(static_cast<const float *>(a.S) + n);
+    sm.phs[(ty + 2) * WP + tx + 2] = f[0] + (lo + sum_moving(f));
+    sm.phs[hy * WP + tx + 2] = h[0] + (hlo + sum_moving(h));
+    __syncthreads();
+    // mu of the tile's rows and one row and column around it (the arithmetic of
+    // d2q9_tile's mu_at); r: mu ring row (phi ring row r + 1), j: mu ring column
+    auto mu_at = [&](int r, int j) {
+        const float *p0 = sm.phs + (r + 1) * WP, *pm = p0 - WP, *pp = p0 + WP;
+        const float c = p0[j + 1];
+        const float ax = (p0[j + 2] - c) + (p0[j] - c) + (pp[j + 1] - c) + (pm[j + 1] - c);
+        const float dg = (pp[j + 2] - c) + (pp[j] - c) + (pm[j + 2] - c) + (pm[j] - c);
+        const float lap = float(2.0 / 3.0) * ax + float(1.0 / 6.0) * dg;
+        const float bulk = 4.0f * P.beta * (c - P.phil) * (c - P.phiv) * (c - P.phibar);
+        sm.mus[r * WM + j] = bulk - P.kappa * lap;
+    };
+    mu_at(ty + 1, tx + 1);
+    if (ty < 2)
+        mu_at(ty == 0 ? 0 : SHY + 1, tx + 1);
+    else if (ty == 2 && tx < 2 * (SHY + 2))
+        mu_at(tx >> 1, (tx & 1) ? SHX + 1 : 0);
+    __syncthreads();
+    if (!ok) return;
+    const float *p0 = sm.phs + (ty + 2) * WP, *m0 = sm.mus + (ty + 1) * WM;
+    d2q9_node<float, PASS, NT>(P, a, p0 - WP, p0, p0 + WP, m0 - WM, m0, m0 + WM, tx + 2, tx + 1, f,
+                               lo, gv, Sprev, a_src, a_dst, n, lin, nullptr, nullptr, nullptr);
 }
 
 // Batched: CTA k runs tile k of a flat tile table over many independent grids
@@ -1442,6 +1537,14 @@ int rows64(int nx, int ny, int num_sms)
     return rows;
 }
 
+// Largest FP32 grid whose steps d2q9_shot_kernel runs: while both population
+// buffers (160 B per node) stay within about 100 MB of L2, its redundant halo
+// loads hit there; beyond, the march's fewer loads win.  Measured, march -> shot,
+// us per step: 32^2 3.8 -> 2.3, 128^2 4.0 -> 2.8, 301 x 203 6.5 -> 3.9, 512^2 10.7 ->
+// 8.0, 700^2 18.2 -> 15.1, 780^2 22.2 -> 20.1, 850^2 23.3 -> 24.9, 1024^2 33.2 -> 37.3,
+// 50 x 3000 12.6 -> 6.6, 3000 x 50 7.5 -> 6.2.
+constexpr long long SHOT_MAX_NODES = 640000;
+
 template <typename T, int PASS>
 cudaError_t launch_pass(const void *params, const PassArgs &a, const LaunchShape &s,
                         cudaStream_t st)
@@ -1459,6 +1562,11 @@ cudaError_t launch_pass(const void *params, const PassArgs &a, const LaunchShape
         if (tiles.y <= 65535)
             return launch_pdl(d2q9_pass_kernel<T, 64, PASS>, tiles, dim3(64, TYB),
                               tile_dyn_bytes<T, 64>(), st, P, a, rows);
+    }
+    if constexpr (sizeof(T) == 4 && (PASS & PASS_STATE) && !(PASS & (PASS_DIAG | PASS_MACROS))) {
+        const dim3 tiles((P.nx + SHX - 1) / SHX, (P.ny + SHY - 1) / SHY);
+        if (P.N <= SHOT_MAX_NODES && tiles.y <= 65535)
+            return launch_pdl(d2q9_shot_kernel<PASS>, tiles, dim3(SHX, SHY), 0, st, P, a);
     }
     constexpr int dyn = tile_dyn_bytes<T, TXW>();
     dim3 grid(s.grid_x, s.grid_y), block(TXW, TYB);
