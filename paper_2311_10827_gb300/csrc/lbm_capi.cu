@@ -1821,6 +1821,7 @@ struct lbm_adjoint {
     int K, max_steps, nsteps, recorded;
     size_t snap;        // bytes of one state snapshot (f, g, S at the context's precision)
     size_t slot;        // bytes of one segment slot: a snapshot, then its moments
+    char *mem;          // the one allocation that holds every buffer below
     char *ckpt;         // (max_steps / K + 1) snapshots
     char *seg;          // K slots of the segment being reversed
     int real;           // adjoint arithmetic: 0 FP64, 1 FP32 (the context's precision)
@@ -1859,10 +1860,7 @@ int restore(lbm_ctx *ctx, const char *src, long long step)
 
 void adjoint_free(lbm_adjoint *a)
 {
-    void *p[] = {a->ckpt, a->seg, a->phi0, a->lf[0], a->lf[1], a->lg[0], a->lg[1],
-                 a->lS[0], a->lS[1], a->lpt, a->macro, a->work, a->dpar};
-    for (void *q : p)
-        if (q) cudaFree(q);
+    if (a->mem) cudaFree(a->mem);
     free(a);
 }
 
@@ -1890,21 +1888,36 @@ int lbm_adjoint_create(lbm_ctx *ctx, int checkpoint_every, int max_steps, lbm_ad
     const size_t nck = (size_t)(max_steps / checkpoint_every + 1);
     a->real = ctx->prm.precision == LBM_FP64 ? 0 : 1;
     a->rsz = a->real == 0 ? sizeof(double) : sizeof(float);
-    bool ok = cudaMalloc((void **)&a->ckpt, nck * a->snap) == cudaSuccess &&
-              cudaMalloc((void **)&a->seg, (size_t)checkpoint_every * a->slot) == cudaSuccess &&
-              cudaMalloc((void **)&a->phi0, N * sizeof(double)) == cudaSuccess &&
-              cudaMalloc((void **)&a->macro, N * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&a->work, 6 * N * a->rsz) == cudaSuccess &&
-              cudaMalloc(&a->lpt, N * a->rsz) == cudaSuccess &&
-              cudaMalloc((void **)&a->dpar, 3 * sizeof(double)) == cudaSuccess;
-    for (int b = 0; b < 2 && ok; ++b)
-        ok = cudaMalloc(&a->lf[b], Q * N * a->rsz) == cudaSuccess &&
-             cudaMalloc(&a->lg[b], Q * N * a->rsz) == cudaSuccess &&
-             cudaMalloc(&a->lS[b], N * a->rsz) == cudaSuccess;
-    if (!ok) {
+    // one allocation for every buffer (each 256-byte aligned): a recorder is
+    // created and destroyed by every differentiated run, and freeing 13 buffers
+    // one by one costs a synchronisation each
+    struct {
+        void **p;
+        size_t bytes;
+    } const part[] = {{(void **)&a->ckpt, nck * a->snap},
+                      {(void **)&a->seg, (size_t)checkpoint_every * a->slot},
+                      {(void **)&a->phi0, N * sizeof(double)},
+                      {(void **)&a->macro, N * sizeof(double)},
+                      {&a->work, 6 * N * a->rsz},
+                      {&a->lpt, N * a->rsz},
+                      {(void **)&a->dpar, 3 * sizeof(double)},
+                      {&a->lf[0], Q * N * a->rsz},
+                      {&a->lf[1], Q * N * a->rsz},
+                      {&a->lg[0], Q * N * a->rsz},
+                      {&a->lg[1], Q * N * a->rsz},
+                      {&a->lS[0], N * a->rsz},
+                      {&a->lS[1], N * a->rsz}};
+    size_t total = 0;
+    for (const auto &q : part) total += (q.bytes + 255) / 256 * 256;
+    if (cudaMalloc((void **)&a->mem, total) != cudaSuccess) {
         cudaGetLastError();
         adjoint_free(a);
         return LBM_ERR_OOM;
+    }
+    size_t off = 0;
+    for (const auto &q : part) {
+        *q.p = a->mem + off;
+        off += (q.bytes + 255) / 256 * 256;
     }
     ctx->recentre = 0;  // the recorded states keep one equilibrium shift
     *out = a;
