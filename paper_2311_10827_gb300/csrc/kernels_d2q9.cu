@@ -38,6 +38,7 @@
 
 #include "launch.cuh"
 #include "lbm_internal.h"
+#include "rcp64.cuh"
 
 namespace wblbm {
 namespace {
