@@ -156,6 +156,8 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 // formed once per march: 1030 instructions per node, 160^3 279 -> 233 us, whole
 // 256^3 runs 1.40 -> 1.17 ms per step.  EVEN: rows of an even number of nodes,
 // which is what those words need; other grids load and store single values.
+// The asynchronous copies of phi and macros move pairs too where rows are even
+// (256^3 1068 -> 1061 us per step, 64^3 26.1 -> 25.2, 32^3 13.5 -> 12.4).
 // Three CTAs of 128 threads per SM at 168 registers; four spill (83 ms against
 // 47 ms per 40 steps at 256^3).  Measured and not kept, all bit-identical: the
 // pulls staged a plane ahead in shared memory by 4-byte asynchronous copies
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     __shared__ __align__(16) float phs[RP * PA];
     __shared__ __align__(16) float mus[RM * MA];
     // the source macros of the plane two ahead, copied while a plane is updated
-    __shared__ float mraw[6 * MN];
+    __shared__ __align__(16) float mraw[6 * MA];
     // per source node {alpha mu, A = 3p - 3/2 rho |u|^2, rho u_x, rho u_y, rho u_z, 9 / (2 rho)}:
     // g^eq_i = w_i (A + 3 c.j + (9/2)(c.j)^2 / rho); ring of three planes per quantity
     __shared__ __align__(16) float qs[6][RM * MA];
@@ -200,22 +202,38 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
 
     // grids narrower than a tile plus halo wrap by division (uniform flags)
     const bool smx = nx < PX + 2, smy = ny < PY + 2, smz = nz < 8;
-    // this thread's elements of a phi plane and nodes of a mu / macro plane:
-    // ring index and in-plane offset in the grid (nodes past the halo repeat)
-    constexpr int KP = (PA + PAIR_NT - 1) / PAIR_NT, KM = (MN + PAIR_NT - 1) / PAIR_NT;
-    unsigned poff[KP], moff[KM];
+    // this thread's nodes of a mu / macro plane: ring index and in-plane offset in
+    // the grid (nodes past the halo repeat)
+    constexpr int KM = (MN + PAIR_NT - 1) / PAIR_NT;
+    unsigned moff[KM];
     int mring[KM];  // index in a stored plane (row stride MX, x halo 2)
-#pragma unroll
-    for (int k = 0; k < KP; ++k) {
-        const int q = tid + k * PAIR_NT;
-        poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
-    }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
         const int q = tid + k * PAIR_NT;
         moff[k] = (unsigned)wrapc(y0 - 1 + q / MW, ny, smy) * nx + wrapc(x0 - 1 + q % MW, nx, smx);
         mring[k] = q / MW * MX + q % MW + 1;
     }
+    // what it copies of a phi plane and of a macro plane: pairs (EVEN; a pair stays
+    // one after the periodic wrap) or single elements
+    constexpr int VW = EVEN ? 2 : 1;
+    constexpr int KP = (PA / VW + PAIR_NT - 1) / PAIR_NT, KC = (MA / VW + PAIR_NT - 1) / PAIR_NT;
+    unsigned poff[KP], coff[KC];
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+        const int q = VW * (tid + k * PAIR_NT);
+        poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
+    }
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        const int q = VW * (tid + k * PAIR_NT);
+        coff[k] = (unsigned)wrapc(y0 - 1 + q / MX, ny, smy) * nx + wrapc(x0 - 2 + q % MX, nx, smx);
+    }
+    auto copy_v = [](float *d, const float *v) {
+        if (EVEN)
+            cp_async8(d, v);
+        else
+            cp_async4(d, v);
+    };
     // ring slots of plane z0 + d: phi (d + 2) mod 5, mu and macros (d + 1) mod 3
     auto wrapr = [](int v, int n) { return v >= n ? v - n : v; };
     // Eq. chemical_potencial with Eq. Laplace on D3Q19, from the phi slots of the
@@ -258,8 +276,10 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         const unsigned zo = (unsigned)wrapc(z0 - 2 + d, nz, smz) * plane;
 #pragma unroll
         for (int k = 0; k < KP; ++k)
-            if (tid + k * PAIR_NT < PA) phs[d * PA + tid + k * PAIR_NT] = phif[zo + poff[k]];
+            if (VW * (tid + k * PAIR_NT) < PA)
+                copy_v(phs + d * PA + VW * (tid + k * PAIR_NT), phif + (zo + poff[k]));
     }
+    cp_commit();
     for (int d = 0; d < 3; ++d) {
         const unsigned zo = (unsigned)wrapc(z0 - 1 + d, nz, smz) * plane;
 #pragma unroll
@@ -271,6 +291,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
             put_macros(d, mring[k], m6);
         }
     }
+    cp_wait_all();
     __syncthreads();
     for (int d = 0; d < 3; ++d) mu_plane(d, d + 1, d + 2, d);
     __syncthreads();
@@ -293,18 +314,18 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         const int sq0 = wrapr(sq + 1, RM), sqp = wrapr(sq + 2, RM);
         {
             const unsigned zo = (unsigned)wrapc(zz + 3, nz, smz) * plane;
-            float *d = phs + wrapr(sp + 4, RP) * PA + tid;
+            float *d = phs + wrapr(sp + 4, RP) * PA + VW * tid;
 #pragma unroll
             for (int k = 0; k < KP; ++k)
-                if (tid + k * PAIR_NT < PA) cp_async4(d + k * PAIR_NT, phif + (zo + poff[k]));
+                if (VW * (tid + k * PAIR_NT) < PA) copy_v(d + VW * k * PAIR_NT, phif + (zo + poff[k]));
             const unsigned zm = (unsigned)wrapc(zz + 2, nz, smz) * plane;
 #pragma unroll
-            for (int k = 0; k < KM; ++k) {
-                if (tid + k * PAIR_NT >= MN) break;
-                const float *m = src.M + (zm + moff[k]);
+            for (int k = 0; k < KC; ++k) {
+                if (VW * (tid + k * PAIR_NT) >= MA) break;
+                const float *m = src.M + (zm + coff[k]);
 #pragma unroll
                 for (int c = 0; c < 6; ++c)
-                    cp_async4(mraw + c * MN + tid + k * PAIR_NT, m + (size_t)c * N);
+                    copy_v(mraw + c * MA + VW * (tid + k * PAIR_NT), m + (size_t)c * N);
             }
             cp_commit();
         }
@@ -543,11 +564,11 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         cp_wait_all();
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < KM; ++k) {  // own copies: no barrier needed
+        for (int k = 0; k < KM; ++k) {
             if (tid + k * PAIR_NT >= MN) break;
             float m6[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MN + tid + k * PAIR_NT];
+            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MA + mring[k]];
             put_macros(sq, mring[k], m6);
         }
         // phi planes zz + 1 .. zz + 3 -> mu plane zz + 2 in the slot of zz - 1
