@@ -796,16 +796,45 @@ __global__ void d3q19_off_poke_k(const StepParams<float> P, OffBuf o, int field,
 // ---------------------------------------------------------------- scales
 
 // max over |stored value| bit patterns (monotonic in the magnitude for both
-// formats); NaN patterns are larger than INF_BITS
-__global__ void off_absmax_k(const unsigned short *__restrict__ v, size_t count,
-                             unsigned *__restrict__ out)
+// formats; NaN patterns are larger than INF_BITS) of the f and the g offsets
+// (blockIdx.y 0, 1) into out[0], out[1].  HBM bounds it: eight values per
+// 16-byte load, four loads in flight per thread (one value at a time took
+// 885 us per field at 256^3, 0.7 TB/s).  v is 16-byte aligned.
+__global__ void __launch_bounds__(256)
+    off_absmax_k(const unsigned short *__restrict__ f, const unsigned short *__restrict__ g,
+                 size_t count, unsigned *__restrict__ out)
 {
-    unsigned m = 0;
-    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < count;
-         q += (size_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned)(__ldg(v + q) & 0x7fffu));
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    const unsigned short *v = blockIdx.y ? g : f;
+    const uint4 *w = reinterpret_cast<const uint4 *>(v);
+    const size_t nv = count / 8, step = (size_t)gridDim.x * 256;
+    const size_t i0 = (size_t)blockIdx.x * 256 + threadIdx.x;
+    unsigned m2 = 0;  // two 16-bit maxima
+    auto take = [&](uint4 q) {
+        m2 = __vmaxu2(m2, q.x & 0x7fff7fffu);
+        m2 = __vmaxu2(m2, q.y & 0x7fff7fffu);
+        m2 = __vmaxu2(m2, q.z & 0x7fff7fffu);
+        m2 = __vmaxu2(m2, q.w & 0x7fff7fffu);
+    };
+    size_t i = i0;
+    for (; i + 3 * step < nv; i += 4 * step) {
+        const uint4 a = __ldg(w + i), b = __ldg(w + i + step), c = __ldg(w + i + 2 * step),
+                    d = __ldg(w + i + 3 * step);
+        take(a);
+        take(b);
+        take(c);
+        take(d);
+    }
+    for (; i < nv; i += step) take(__ldg(w + i));
+    unsigned m = max(m2 & 0xffffu, m2 >> 16);
+    if (i0 < count - nv * 8) m = max(m, (unsigned)(__ldg(v + nv * 8 + i0) & 0x7fffu));
+    m = __reduce_max_sync(0xffffffffu, m);
+    __shared__ unsigned wm[8];
+    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) m = max(m, wm[k]);
+        if (m) atomicMax(out + blockIdx.y, m);
+    }
 }
 
 template <class C>
@@ -952,9 +981,11 @@ cudaError_t offset_refresh(int codec, long long N, int Q, const void *f, const v
     cudaError_t e = cudaMemsetAsync(maxbits, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     const size_t count = (size_t)Q * (size_t)N;
-    const unsigned nb = (unsigned)(4 * (num_sms > 0 ? num_sms : 152));
-    off_absmax_k<<<nb, 256, 0, st>>>((const unsigned short *)f, count, maxbits);
-    off_absmax_k<<<nb, 256, 0, st>>>((const unsigned short *)g, count, maxbits + 1);
+    // four resident CTAs of each field per SM, fewer where the field is small
+    const size_t want = (count / 8 + 255) / 256, most = (size_t)(4 * (num_sms > 0 ? num_sms : 152));
+    const unsigned nb = (unsigned)(want < 1 ? 1 : (want < most ? want : most));
+    off_absmax_k<<<dim3(nb, 2), 256, 0, st>>>((const unsigned short *)f, (const unsigned short *)g,
+                                              count, maxbits);
     const OffBuf cur = off_view(f, g, N);
     if (codec == OFFSET_F16)
         off_target_k<CodecF16><<<1, 1, 0, st>>>(cur, maxbits, target);
