@@ -145,6 +145,51 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 
 // ------------------------------------------------------------------ pass 2
 
+// One CTA's diagnostics partial from its NT threads' values (all of them call it)
+template <int NT>
+__device__ __forceinline__ void off_partial(int tid, double d_phi, double d_E, double d_u2,
+                                            double d_mumin, double d_mumax, double d_bud,
+                                            double d_bad, DiagPartial *out)
+{
+    for (int o = 16; o > 0; o >>= 1) {
+        d_phi += __shfl_xor_sync(0xffffffffu, d_phi, o);
+        d_E += __shfl_xor_sync(0xffffffffu, d_E, o);
+        d_bud += __shfl_xor_sync(0xffffffffu, d_bud, o);
+        d_u2 = fmax(d_u2, __shfl_xor_sync(0xffffffffu, d_u2, o));
+        d_mumin = fmin(d_mumin, __shfl_xor_sync(0xffffffffu, d_mumin, o));
+        d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
+        d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
+    }
+    constexpr int NW = NT / 32;
+    __shared__ double red[7][NW];
+    const int lane = tid & 31, wid = tid >> 5;
+    if (lane == 0) {
+        red[0][wid] = d_phi;
+        red[1][wid] = d_E;
+        red[2][wid] = d_u2;
+        red[3][wid] = d_mumin;
+        red[4][wid] = d_mumax;
+        red[5][wid] = d_bud;
+        red[6][wid] = d_bad;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        DiagPartial o;
+        o.sum_phi = 0.0, o.E = 0.0, o.u2max = 0.0, o.mu_min = DBL_MAX, o.mu_max = -DBL_MAX;
+        o.budget = 0.0, o.nonfinite = 0.0, o.pad = 0.0;
+        for (int w = 0; w < NW; ++w) {
+            o.sum_phi += red[0][w];
+            o.E += red[1][w];
+            o.u2max = fmax(o.u2max, red[2][w]);
+            o.mu_min = fmin(o.mu_min, red[3][w]);
+            o.mu_max = fmax(o.mu_max, red[4][w]);
+            o.budget += red[5][w];
+            o.nonfinite = fmax(o.nonfinite, red[6][w]);
+        }
+        *out = o;
+    }
+}
+
 // What bounds this pass: instruction issue and the latency of the pulls.
 // Rebuilding 38 populations per node from their offsets took 1570 instructions
 // per node with one node per thread (256^3 FP16: 1.135 ms, issue slots 60% busy
@@ -154,9 +199,8 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 // as one 32-bit word where their alignment allows (every store, and the pulls
 // without an x component), and the plane offsets of the asynchronous copies are
 // formed once per march: 1030 instructions per node, 160^3 279 -> 233 us, whole
-// 256^3 runs 1.40 -> 1.17 ms per step.  EVEN: rows of an even number of nodes,
-// which is what those words need; other grids load and store single values.
-// The asynchronous copies of phi and macros move pairs too where rows are even
+// 256^3 runs 1.40 -> 1.17 ms per step.  For rows of an even number of nodes, which is
+// what those words need.  The asynchronous copies of phi and macros move pairs too
 // (256^3 1068 -> 1061 us per step, 64^3 26.1 -> 25.2, 32^3 13.5 -> 12.4).
 // Three CTAs of 128 threads per SM at 168 registers; four spill (83 ms against
 // 47 ms per 40 steps at 256^3).  Measured and not kept, all bit-identical: the
@@ -164,7 +208,7 @@ __global__ void d3q19_off_prep_k(const StepParams<float> P, OffBuf o)
 // (333 us: the load/store units take one word per thread at a time), the next
 // plane's pulls in registers during the collisions at two CTAs per SM (238 us),
 // or while its mu is formed (264 us: they spill).
-template <class C, int PASS, bool EVEN>
+template <class C, int PASS>
 __global__ void __launch_bounds__(PAIR_NT, 3)
     d3q19_off_pass_kernel(const StepParams<float> P, PassArgs a, const OffBuf src, const OffBuf dst,
                           const float *__restrict__ target, const float *__restrict__ phif,
@@ -190,7 +234,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
     const int x = x0 + 2 * tx, y = y0 + ty;
-    const bool okA = x < nx && y < ny, okB = EVEN ? okA : (x + 1 < nx && y < ny);
+    const bool ok = x < nx && y < ny;  // (both nodes: nx is even)
     const unsigned plane = (unsigned)nx * ny;
     const float s_f = __ldg(src.sc), s_g = __ldg(src.sc + 1);
     const float t_f = __ldg(target), t_g = __ldg(target + 1);
@@ -213,27 +257,20 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         moff[k] = (unsigned)wrapc(y0 - 1 + q / MW, ny, smy) * nx + wrapc(x0 - 1 + q % MW, nx, smx);
         mring[k] = q / MW * MX + q % MW + 1;
     }
-    // what it copies of a phi plane and of a macro plane: pairs (EVEN; a pair stays
-    // one after the periodic wrap) or single elements
-    constexpr int VW = EVEN ? 2 : 1;
-    constexpr int KP = (PA / VW + PAIR_NT - 1) / PAIR_NT, KC = (MA / VW + PAIR_NT - 1) / PAIR_NT;
+    // the pairs it copies of a phi plane and of a macro plane (a pair stays one
+    // after the periodic wrap)
+    constexpr int KP = (PA / 2 + PAIR_NT - 1) / PAIR_NT, KC = (MA / 2 + PAIR_NT - 1) / PAIR_NT;
     unsigned poff[KP], coff[KC];
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
-        const int q = VW * (tid + k * PAIR_NT);
+        const int q = 2 * (tid + k * PAIR_NT);
         poff[k] = (unsigned)wrapc(y0 - 2 + q / PX, ny, smy) * nx + wrapc(x0 - 2 + q % PX, nx, smx);
     }
 #pragma unroll
     for (int k = 0; k < KC; ++k) {
-        const int q = VW * (tid + k * PAIR_NT);
+        const int q = 2 * (tid + k * PAIR_NT);
         coff[k] = (unsigned)wrapc(y0 - 1 + q / MX, ny, smy) * nx + wrapc(x0 - 2 + q % MX, nx, smx);
     }
-    auto copy_v = [](float *d, const float *v) {
-        if (EVEN)
-            cp_async8(d, v);
-        else
-            cp_async4(d, v);
-    };
     // ring slots of plane z0 + d: phi (d + 2) mod 5, mu and macros (d + 1) mod 3
     auto wrapr = [](int v, int n) { return v >= n ? v - n : v; };
     // Eq. chemical_potencial with Eq. Laplace on D3Q19, from the phi slots of the
@@ -276,8 +313,8 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         const unsigned zo = (unsigned)wrapc(z0 - 2 + d, nz, smz) * plane;
 #pragma unroll
         for (int k = 0; k < KP; ++k)
-            if (VW * (tid + k * PAIR_NT) < PA)
-                copy_v(phs + d * PA + VW * (tid + k * PAIR_NT), phif + (zo + poff[k]));
+            if (2 * (tid + k * PAIR_NT) < PA)
+                cp_async8(phs + d * PA + 2 * (tid + k * PAIR_NT), phif + (zo + poff[k]));
     }
     cp_commit();
     for (int d = 0; d < 3; ++d) {
@@ -303,42 +340,39 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     // (read) and zz+3 (being written); mu and macros zz-1..zz+1; once every
     // thread is past the update, macro plane zz+2 and mu plane zz+2 take the
     // slots of zz-1.
-    const unsigned xw = okA ? (unsigned)x : 0, yw = okA ? (unsigned)y : 0;
+    const unsigned xw = ok ? (unsigned)x : 0, yw = ok ? (unsigned)y : 0;
     Nb b = make_nb((int)xw, (int)yw, z0, nx, ny, nz);
-    const unsigned xB = okB ? xw + 1 : 0;                   // the second node's column
-    const unsigned xp2 = (unsigned)wrap1((int)xw + 2, nx);  // and its +x neighbour (nx >= 2)
-    const unsigned xpp = nx == 1 ? 0u : xp2;
+    const unsigned xp2 = (unsigned)wrap1((int)xw + 2, nx);  // the second node's +x neighbour
     int sp = 1, sq = 0;  // phi slot of plane zz - 1, mu / macro slot of plane zz - 1
     for (int zz = z0; zz < zend; ++zz) {
         const int sp0 = wrapr(sp + 1, RP), spp = wrapr(sp + 2, RP);
         const int sq0 = wrapr(sq + 1, RM), sqp = wrapr(sq + 2, RM);
         {
             const unsigned zo = (unsigned)wrapc(zz + 3, nz, smz) * plane;
-            float *d = phs + wrapr(sp + 4, RP) * PA + VW * tid;
+            float *d = phs + wrapr(sp + 4, RP) * PA + 2 * tid;
 #pragma unroll
             for (int k = 0; k < KP; ++k)
-                if (VW * (tid + k * PAIR_NT) < PA) copy_v(d + VW * k * PAIR_NT, phif + (zo + poff[k]));
+                if (2 * (tid + k * PAIR_NT) < PA) cp_async8(d + 2 * k * PAIR_NT, phif + (zo + poff[k]));
             const unsigned zm = (unsigned)wrapc(zz + 2, nz, smz) * plane;
 #pragma unroll
             for (int k = 0; k < KC; ++k) {
-                if (VW * (tid + k * PAIR_NT) >= MA) break;
+                if (2 * (tid + k * PAIR_NT) >= MA) break;
                 const float *m = src.M + (zm + coff[k]);
 #pragma unroll
                 for (int c = 0; c < 6; ++c)
-                    copy_v(mraw + c * MA + VW * (tid + k * PAIR_NT), m + (size_t)c * N);
+                    cp_async8(mraw + c * MA + 2 * (tid + k * PAIR_NT), m + (size_t)c * N);
             }
             cp_commit();
         }
-        if (okA) {
+        if (ok) {
         nb_plane(b, zz, nx, ny, nz);
         const unsigned row = b.zs[1] + b.ys[1], n = row + xw;
         // the offsets of the two nodes share one register (the first in the low half)
         unsigned hp[19], kp[19];
         auto pull = [&](const unsigned short *v, int i) -> unsigned {
             const unsigned r = i * N + b.zs[1 - c3z(i)] + b.ys[1 - c3y(i)];
-            if (c3x(i) == 0 && EVEN) return __ldg(reinterpret_cast<const unsigned *>(v + (r + xw)));
-            const unsigned ca = c3x(i) > 0 ? b.xs[0] : (c3x(i) < 0 ? b.xs[2] : xw);
-            const unsigned cb = c3x(i) > 0 ? xw : (c3x(i) < 0 ? xpp : xB);
+            if (c3x(i) == 0) return __ldg(reinterpret_cast<const unsigned *>(v + (r + xw)));
+            const unsigned ca = c3x(i) > 0 ? b.xs[0] : b.xs[2], cb = c3x(i) > 0 ? xw : xp2;
             return (unsigned)__ldg(v + (r + ca)) | ((unsigned)__ldg(v + (r + cb)) << 16);
         };
 #pragma unroll
@@ -347,17 +381,10 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
             kp[i] = pull(src.k, i);
         }
         // an FP32 value of each of the two nodes
-        auto own = [&](const float *v) -> float2 {
-            if (EVEN) return __ldg(reinterpret_cast<const float2 *>(v + n));
-            return make_float2(__ldg(v + n), __ldg(v + (row + xB)));
-        };
+        auto own = [&](const float *v) { return __ldg(reinterpret_cast<const float2 *>(v + n)); };
         float2 Sprev = f2(0.0f);
         if (PASS & (PASS_STATE | PASS_DIAG)) {
-            const float *S = static_cast<const float *>(a.S);
-            if (EVEN)
-                Sprev = __ldcs(reinterpret_cast<const float2 *>(S + n));
-            else
-                Sprev = make_float2(__ldcs(S + n), __ldcs(S + (row + xB)));
+            Sprev = __ldcs(reinterpret_cast<const float2 *>(static_cast<const float *>(a.S) + n));
         }
         const float2 phi_hi = own(src.M), p_own = own(src.M + 2 * N);
 
@@ -451,12 +478,12 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
                 if (!isfinite(ph) || !isfinite(pp) || !isfinite(u2f) || !isfinite(m)) d_bad = 1.0;
             };
             acc(phi.x, r.x, rho.x, uu.x, mu.x, S.x, Sprev.x, p.x);
-            if (okB) acc(phi.y, r.y, rho.y, uu.y, mu.y, S.y, Sprev.y, p.y);
+            acc(phi.y, r.y, rho.y, uu.y, mu.y, S.y, Sprev.y, p.y);
         }
         if (PASS & PASS_MACROS) {
             auto put = [&](double *o, double va, double vb) {
                 o[n] = va;
-                if (okB) o[n + 1] = vb;
+                o[n + 1] = vb;
             };
             if (a.out_phi)
                 put(a.out_phi, (double)phi.x + (double)r.x, (double)phi.y + (double)r.y);
@@ -469,22 +496,9 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
             }
         }
         if (PASS & PASS_STATE) {
-            auto put = [&](float *o, float2 v) {
-                if (EVEN) {
-                    __stcs(reinterpret_cast<float2 *>(o + n), v);
-                } else {
-                    __stcs(o + n, v.x);
-                    if (okB) __stcs(o + n + 1, v.y);
-                }
-            };
+            auto put = [&](float *o, float2 v) { __stcs(reinterpret_cast<float2 *>(o + n), v); };
             auto put16 = [&](unsigned short *o, float2 v) {
-                const unsigned e = C::enc2(v);
-                if (EVEN) {
-                    __stcs(reinterpret_cast<unsigned *>(o + n), e);
-                } else {
-                    __stcs(o + n, (unsigned short)(e & 0xffffu));
-                    if (okB) __stcs(o + n + 1, (unsigned short)(e >> 16));
-                }
+                __stcs(reinterpret_cast<unsigned *>(o + n), C::enc2(v));
             };
             put(static_cast<float *>(a.S), S);
             put(dst.M, phi);
@@ -560,7 +574,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
                 put16(dst.k + o * N, mul2(fma2(mwk, cF, fma2(wkcu, cg, mul2(to, omg))), itg2));
             }
         }
-        }  // okA
+        }  // ok
         cp_wait_all();
         __syncthreads();
 #pragma unroll
@@ -578,45 +592,331 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
         sq = sq0;
     }
 
-    if (PASS & PASS_DIAG) {
-        for (int o = 16; o > 0; o >>= 1) {
-            d_phi += __shfl_xor_sync(0xffffffffu, d_phi, o);
-            d_E += __shfl_xor_sync(0xffffffffu, d_E, o);
-            d_bud += __shfl_xor_sync(0xffffffffu, d_bud, o);
-            d_u2 = fmax(d_u2, __shfl_xor_sync(0xffffffffu, d_u2, o));
-            d_mumin = fmin(d_mumin, __shfl_xor_sync(0xffffffffu, d_mumin, o));
-            d_mumax = fmax(d_mumax, __shfl_xor_sync(0xffffffffu, d_mumax, o));
-            d_bad = fmax(d_bad, __shfl_xor_sync(0xffffffffu, d_bad, o));
-        }
-        constexpr int NW = PAIR_NT / 32;
-        __shared__ double red[7][NW];
-        const int lane = tid & 31, wid = tid >> 5;
-        if (lane == 0) {
-            red[0][wid] = d_phi;
-            red[1][wid] = d_E;
-            red[2][wid] = d_u2;
-            red[3][wid] = d_mumin;
-            red[4][wid] = d_mumax;
-            red[5][wid] = d_bud;
-            red[6][wid] = d_bad;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            DiagPartial o;
-            o.sum_phi = 0.0, o.E = 0.0, o.u2max = 0.0, o.mu_min = DBL_MAX, o.mu_max = -DBL_MAX;
-            o.budget = 0.0, o.nonfinite = 0.0, o.pad = 0.0;
-            for (int w = 0; w < NW; ++w) {
-                o.sum_phi += red[0][w];
-                o.E += red[1][w];
-                o.u2max = fmax(o.u2max, red[2][w]);
-                o.mu_min = fmin(o.mu_min, red[3][w]);
-                o.mu_max = fmax(o.mu_max, red[4][w]);
-                o.budget += red[5][w];
-                o.nonfinite = fmax(o.nonfinite, red[6][w]);
-            }
-            a.partials[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = o;
-        }
+    if (PASS & PASS_DIAG)
+        off_partial<PAIR_NT>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
+                             a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+}
+
+// The same pass with one node per thread, for rows of an odd number of nodes:
+// there the two-node form has to load and store single values (twice the
+// requests for the same sectors) and was 2 to 10% slower than this one
+// (177 x 44 x 219 FP16 188 against 170 us per step).  Each value is formed by the same
+// operations in the same order, so both give the same bits.
+template <class C, int PASS>
+__global__ void __launch_bounds__(TX3 *TY3)
+    d3q19_off_pass1_kernel(const StepParams<float> P, PassArgs a, const OffBuf src, const OffBuf dst,
+                           const float *__restrict__ target, const float *__restrict__ phif,
+                           int planes)
+{
+    constexpr int PX = TX3 + 4, PY = TY3 + 4, PA = PX * PY;  // phi plane (halo 2)
+    constexpr int MX = TX3 + 2, MY = TY3 + 2, MA = MX * MY;  // mu / macro plane (halo 1)
+    constexpr int RP = 5, RM = 3, RQ = 3;
+    __shared__ float phs[RP * PA];
+    __shared__ float mus[RM * MA];
+    // the source macros of the plane two ahead, copied while a plane is updated
+    __shared__ float mraw[6 * MA];
+    // per source node: {alpha mu, A = 3p - 3/2 rho |u|^2, rho ux, rho uy} and
+    // {rho uz, 9 / (2 rho)}: g^eq_i = w_i (A + 3 c.j + (9/2)(c.j)^2 / rho)
+    __shared__ float4 qa[RQ * MA];
+    __shared__ float2 qb[RQ * MA];
+
+    pdl_wait();
+    const int nx = P.nx, ny = P.ny, nz = P.nz;
+    const unsigned N = (unsigned)P.N;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
+    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
+    const int x = x0 + tx, y = y0 + ty;
+    const bool col_ok = x < nx && y < ny;
+    const unsigned plane = (unsigned)nx * ny;
+    const float s_f = __ldg(src.sc), s_g = __ldg(src.sc + 1);
+    const float t_f = __ldg(target), t_g = __ldg(target + 1);
+    const float it_f = 1.0f / t_f, it_g = 1.0f / t_g;  // powers of two: exact
+    if ((PASS & PASS_STATE) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) {
+        dst.sc[0] = t_f;
+        dst.sc[1] = t_g;
     }
+
+    auto pslot = [&](int zz) { return (zz - z0 + 2) % RP; };
+    auto mslot = [&](int zz) { return (zz - z0 + 1) % RM; };
+    auto qslot = [&](int zz) { return (zz - z0 + 1) % RQ; };
+
+    // grids narrower than a tile plus halo wrap by division (uniform flags)
+    const bool smx = nx < PX + 2, smy = ny < PY + 2, smz = nz < 8;
+    auto load_phi_plane = [&](int zz) {
+        float *d = phs + pslot(zz) * PA;
+        const unsigned zo = (unsigned)wrapc(zz, nz, smz) * plane;
+        for (int q = tid; q < PA; q += TX3 * TY3) {
+            const int lx = q % PX, ly = q / PX;
+            const unsigned xx = wrapc(x0 - 2 + lx, nx, smx), yy = wrapc(y0 - 2 + ly, ny, smy);
+            d[q] = phif[zo + yy * nx + xx];
+        }
+    };
+    // Eq. chemical_potencial with Eq. Laplace on D3Q19
+    auto mu_plane = [&](int zz) {
+        const float *pm = phs + pslot(zz - 1) * PA, *p0 = phs + pslot(zz) * PA,
+                    *pp = phs + pslot(zz + 1) * PA;
+        float *d = mus + mslot(zz) * MA;
+        for (int q = tid; q < MA; q += TX3 * TY3) {
+            const int lx = q % MX + 1, ly = q / MX + 1;
+            const int c = ly * PX + lx;
+            const float v = p0[c];
+            const float fa = (p0[c + 1] - v) + (p0[c - 1] - v) + (p0[c + PX] - v) +
+                             (p0[c - PX] - v) + (pp[c] - v) + (pm[c] - v);
+            const float ed = ((p0[c + PX + 1] - v) + (p0[c + PX - 1] - v) + (p0[c - PX + 1] - v) +
+                              (p0[c - PX - 1] - v)) +
+                             ((pp[c + 1] - v) + (pp[c - 1] - v) + (pm[c + 1] - v) + (pm[c - 1] - v)) +
+                             ((pp[c + PX] - v) + (pp[c - PX] - v) + (pm[c + PX] - v) +
+                              (pm[c - PX] - v));
+            const float lap = (1.0f / 3.0f) * fa + (1.0f / 6.0f) * ed;
+            d[q] = 4.0f * P.beta * (v - P.phil) * (v - P.phiv) * (v - P.phibar) - P.kappa * lap;
+        }
+    };
+    // equilibrium data of the source state's macros (ph, mu, p, u) at item q
+    // of a macro plane (tile + 1 halo)
+    auto put_macros = [&](int slot, int q, const float m6[6]) {
+        const float rho = P.rhov + (m6[0] - P.phiv) * P.drho;
+        qa[slot * MA + q] = make_float4(P.alpha * m6[1],
+                                        3.0f * m6[2] - 1.5f * rho * (m6[3] * m6[3] + m6[4] * m6[4] + m6[5] * m6[5]),
+                                        rho * m6[3], rho * m6[4]);
+        qb[slot * MA + q] = make_float2(rho * m6[5], 4.5f / rho);
+    };
+    auto macro_node = [&](int zz, int q) {
+        const unsigned m = (unsigned)wrapc(zz, nz, smz) * plane +
+                           (unsigned)wrapc(y0 - 1 + q / MX, ny, smy) * nx + wrapc(x0 - 1 + q % MX, nx, smx);
+        return m;
+    };
+    auto macro_plane = [&](int zz) {
+        for (int q = tid; q < MA; q += TX3 * TY3) {
+            const unsigned m = macro_node(zz, q);
+            float m6[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) m6[k] = __ldg(src.M + k * N + m);
+            put_macros(qslot(zz), q, m6);
+        }
+    };
+    auto grad3 = [&](const float *m, const float *c0, const float *p, int c, int SX, float out[3]) {
+        out[0] = (1.0f / 6.0f) * (c0[c + 1] - c0[c - 1]) +
+                 (1.0f / 12.0f) * ((c0[c + SX + 1] - c0[c + SX - 1]) + (c0[c - SX + 1] - c0[c - SX - 1]) +
+                                   (p[c + 1] - p[c - 1]) + (m[c + 1] - m[c - 1]));
+        out[1] = (1.0f / 6.0f) * (c0[c + SX] - c0[c - SX]) +
+                 (1.0f / 12.0f) * ((c0[c + SX + 1] - c0[c - SX + 1]) + (c0[c + SX - 1] - c0[c - SX - 1]) +
+                                   (p[c + SX] - p[c - SX]) + (m[c + SX] - m[c - SX]));
+        out[2] = (1.0f / 6.0f) * (p[c] - m[c]) +
+                 (1.0f / 12.0f) * ((p[c + 1] - m[c + 1]) + (p[c - 1] - m[c - 1]) +
+                                   (p[c + SX] - m[c + SX]) + (p[c - SX] - m[c - SX]));
+    };
+
+    double d_phi = 0.0, d_E = 0.0, d_u2 = 0.0, d_mumin = DBL_MAX, d_mumax = -DBL_MAX,
+           d_bud = 0.0, d_bad = 0.0;
+
+    for (int q = 0; q < 5; ++q) load_phi_plane(z0 - 2 + q);
+    macro_plane(z0 - 1);
+    macro_plane(z0);
+    macro_plane(z0 + 1);
+    __syncthreads();
+    mu_plane(z0 - 1);
+    mu_plane(z0);
+    mu_plane(z0 + 1);
+    __syncthreads();
+
+    // Plane zz + 3 of phi (into its ring slot) and the raw source macros of
+    // plane zz + 2 (into mraw) are copied asynchronously while plane zz is
+    // updated, so their loads overlap the node's own pulls and hold no
+    // registers.  Ring use during the update of plane zz: phi zz-1..zz+1
+    // (read) and zz+3 (being written); mu and macros zz-1..zz+1; once every
+    // thread is past the update, macro plane zz+2 and mu plane zz+2 take the
+    // slots of zz-1.
+    const unsigned xw = col_ok ? (unsigned)x : 0, yw = col_ok ? (unsigned)y : 0;
+    Nb b = make_nb(xw, yw, z0, nx, ny, nz);
+    for (int zz = z0; zz < zend; ++zz) {
+        {
+            const unsigned zo = (unsigned)wrapc(zz + 3, nz, smz) * plane;
+            float *d = phs + pslot(zz + 3) * PA;
+            for (int q = tid; q < PA; q += TX3 * TY3) {
+                const unsigned xx = wrapc(x0 - 2 + q % PX, nx, smx), yy = wrapc(y0 - 2 + q / PX, ny, smy);
+                cp_async4(d + q, phif + (zo + yy * nx + xx));
+            }
+            for (int q = tid; q < MA; q += TX3 * TY3) {
+                const unsigned m = macro_node(zz + 2, q);
+#pragma unroll
+                for (int c = 0; c < 6; ++c) cp_async4(mraw + c * MA + q, src.M + ((size_t)c * N + m));
+            }
+            cp_commit();
+        }
+        if (col_ok) {
+        nb_plane(b, zz, nx, ny, nz);
+        const unsigned n = b.at(0, 0, 0);
+        // the two 16-bit offsets of direction i share one register
+        unsigned hk[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            const unsigned s = b.at(-c3x(i), -c3y(i), -c3z(i));
+            hk[i] = (unsigned)__ldg(src.h + (i * N + s)) | ((unsigned)__ldg(src.k + (i * N + s)) << 16);
+        }
+        auto hr = [&](int i) { return (unsigned short)(hk[i] & 0xffffu); };
+        auto kr = [&](int i) { return (unsigned short)(hk[i] >> 16); };
+        float Sprev = 0.0f;
+        if (PASS & (PASS_STATE | PASS_DIAG)) Sprev = __ldcs(static_cast<const float *>(a.S) + n);
+        const float phi_hi = __ldg(src.M + n), p_own = __ldg(src.M + 2 * N + n);
+
+        // populations after streaming, rebuilt from offsets and source macros
+        const int cq = (ty + 1) * MX + (tx + 1);
+        float fv[19], gv[19];
+        float flo;  // rest population minus its high word phi_hi
+        {
+            const float4 A0 = qa[qslot(zz) * MA + cq];
+            flo = -(2.0f / 3.0f) * A0.x + s_f * C::dec(hr(0));
+            gv[0] = (1.0f / 3.0f) * A0.y - 3.0f * p_own + s_g * C::dec(kr(0));
+            fv[0] = 0.0f;
+        }
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            const int c = qslot(zz - c3z(i)) * MA + cq - c3y(i) * MX - c3x(i);
+            const float4 A = qa[c];
+            const float2 B = qb[c];
+            const float w = (float)w3(i);
+            fv[i] = w * A.x + s_f * C::dec(hr(i));
+            float cj = 0.0f;
+            if (c3x(i)) cj += (float)c3x(i) * A.z;
+            if (c3y(i)) cj += (float)c3y(i) * A.w;
+            if (c3z(i)) cj += (float)c3z(i) * B.x;
+            gv[i] = w * (A.y + cj * (3.0f + B.y * cj)) + s_g * C::dec(kr(i));
+        }
+
+        float snz = 0.0f, sg = 0.0f;
+#pragma unroll
+        for (int i = 1; i < 19; i += 2) {
+            snz += fv[i] + fv[i + 1];
+            sg += gv[i] + gv[i + 1];
+        }
+        // phi = phi_hi + (flo + snz) as an exact two-sum: phi (FP32) + r
+        const float lo_sum = flo + snz;
+        const float phi = phi_hi + lo_sum;
+        const float bp = phi - phi_hi;
+        const float r = (phi_hi - (phi - bp)) + (lo_sum - bp);
+
+        const int cp = (ty + 2) * PX + (tx + 2), cm = cq;
+        const float *mz = mus + mslot(zz) * MA;
+        const float mu = mz[cm];
+        float gp[3], gm[3];
+        grad3(phs + pslot(zz - 1) * PA, phs + pslot(zz) * PA, phs + pslot(zz + 1) * PA, cp, PX, gp);
+        grad3(mus + mslot(zz - 1) * MA, mz, mus + mslot(zz + 1) * MA, cm, MX, gm);
+
+        float F[3], gr[3], u[3];
+        const float dphi = phi - P.phiv;
+        const float rho = P.rhov + dphi * P.drho;
+        const float nu = P.nuv + dphi * P.dnu;
+        const float inv_rho = __fdividef(1.0f, rho);
+        const float itg = __fdividef(1.0f, 0.5f + 3.0f * nu);
+        float j3[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            if (c3x(i)) j3[0] += (float)c3x(i) * gv[i];
+            if (c3y(i)) j3[1] += (float)c3y(i) * gv[i];
+            if (c3z(i)) j3[2] += (float)c3z(i) * gv[i];
+        }
+        float ugr = 0.0f, uu = 0.0f, S = 0.0f;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            F[d] = -phi * gm[d] + P.G[d];
+            gr[d] = P.drho * gp[d];
+            u[d] = (j3[d] + 0.5f * F[d]) * inv_rho;
+            ugr += u[d] * gr[d];
+            uu += u[d] * u[d];
+            S += u[d] * gp[d];
+        }
+        const float p = 0.5f * (sg + 0.5f * ugr - 0.5f * rho * uu);
+
+        if (PASS & PASS_DIAG) {
+            const double u2 = (double)uu;
+            d_phi += (double)phi + (double)r;
+            d_E += 0.5 * (double)rho * u2;
+            d_u2 = fmax(d_u2, u2);
+            d_mumin = fmin(d_mumin, (double)mu);
+            d_mumax = fmax(d_mumax, (double)mu);
+            d_bud += 1.5 * (double)S - 0.5 * (double)Sprev;
+            if (!isfinite(phi) || !isfinite(p) || !isfinite(uu) || !isfinite(mu)) d_bad = 1.0;
+        }
+        if (PASS & PASS_MACROS) {
+            if (a.out_phi) a.out_phi[n] = (double)phi + (double)r;
+            if (a.out_p) a.out_p[n] = (double)p;
+            if (a.out_mu) a.out_mu[n] = (double)mu;
+            if (a.out_u) {
+                a.out_u[n] = (double)u[0];
+                a.out_u[(size_t)N + n] = (double)u[1];
+                a.out_u[2 * (size_t)N + n] = (double)u[2];
+            }
+        }
+        if (PASS & PASS_STATE) {
+            __stcs(static_cast<float *>(a.S) + n, S);
+            __stcs(dst.M + n, phi);
+            __stcs(dst.M + N + n, mu);
+            __stcs(dst.M + 2 * N + n, p);
+            __stcs(dst.M + 3 * N + n, u[0]);
+            __stcs(dst.M + 4 * N + n, u[1]);
+            __stcs(dst.M + 5 * N + n, u[2]);
+            {
+                // B = phi + alpha sum_{i != 0} w_i (mu(x + c_i) - mu(x)) from the mu ring
+                const float *m0 = mz, *mm = mus + mslot(zz - 1) * MA, *mp = mus + mslot(zz + 1) * MA;
+                const float fa = (m0[cm + 1] - mu) + (m0[cm - 1] - mu) + (m0[cm + MX] - mu) +
+                                 (m0[cm - MX] - mu) + (mp[cm] - mu) + (mm[cm] - mu);
+                const float ed = ((m0[cm + MX + 1] - mu) + (m0[cm + MX - 1] - mu) +
+                                  (m0[cm - MX + 1] - mu) + (m0[cm - MX - 1] - mu)) +
+                                 ((mp[cm + 1] - mu) + (mp[cm - 1] - mu) + (mm[cm + 1] - mu) +
+                                  (mm[cm - 1] - mu)) +
+                                 ((mp[cm + MX] - mu) + (mp[cm - MX] - mu) + (mm[cm + MX] - mu) +
+                                  (mm[cm - MX] - mu));
+                __stcs(dst.M + 6 * N + n, phi + P.alpha * ((1.0f / 18.0f) * fa + (1.0f / 36.0f) * ed));
+            }
+            // CH population (Eqs. BGK, F_i): offset = (f - f^eq)(1 - 1/tau_f) + F_i,
+            // b = -5/2, -1, 1/2; the rest offset also carries the residual r of phi
+            const float Sh = 1.5f * S - 0.5f * Sprev;
+            const float am = P.alpha * mu;
+            const float omf = 1.0f - P.inv_tauf;
+            const float d0 = ((2.0f / 3.0f) * am - snz) * omf + r - (5.0f / 6.0f) * Sh;
+            __stcs(dst.h + n, C::enc(d0 * it_f));
+            const float fa = -(1.0f / 18.0f) * Sh, fe = (1.0f / 72.0f) * Sh;
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                const float w = (float)w3(i);
+                __stcs(dst.h + (i * N + n), C::enc(((fv[i] - w * am) * omf + (i <= 6 ? fa : fe)) * it_f));
+            }
+            // hydrodynamic population (Eqs. g_i, G_i): offset = (g - g^eq)(1 - 1/tau_g) + G_i
+            const float kg = 1.0f - 0.5f * itg, omg = 1.0f - itg;
+            const float A = 3.0f * p - 1.5f * rho * uu;
+            __stcs(dst.k + n, C::enc((gv[0] - ((1.0f / 3.0f) * A - 3.0f * p)) * omg * it_g));
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                const int o = (i <= 6) ? (i % 2 ? i + 1 : i - 1)
+                                       : (i <= 10 ? 17 - i : (i <= 14 ? 25 - i : 33 - i));
+                if (o < i) continue;  // each pair once, from its first member
+                const float w = (float)w3(i);
+                const float cu = (float)c3x(i) * u[0] + (float)c3y(i) * u[1] + (float)c3z(i) * u[2];
+                const float cF = (float)c3x(i) * F[0] + (float)c3y(i) * F[1] + (float)c3z(i) * F[2];
+                const float cg = (float)c3x(i) * gr[0] + (float)c3y(i) * gr[1] + (float)c3z(i) * gr[2];
+                const float eq_s = w * (A + 4.5f * rho * cu * cu), eq_a = 3.0f * w * rho * cu;
+                const float G_s = 3.0f * w * kg * cu * cg, G_a = 3.0f * w * kg * cF;
+                __stcs(dst.k + (i * N + n), C::enc(((gv[i] - eq_s - eq_a) * omg + G_s + G_a) * it_g));
+                __stcs(dst.k + (o * N + n), C::enc(((gv[o] - eq_s + eq_a) * omg + G_s - G_a) * it_g));
+            }
+        }
+        }  // col_ok
+        cp_wait_all();
+        __syncthreads();
+        for (int q = tid; q < MA; q += TX3 * TY3) {  // own copies: no barrier needed
+            float m6[6];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) m6[c] = mraw[c * MA + q];
+            put_macros(qslot(zz + 2), q, m6);
+        }
+        mu_plane(zz + 2);
+        __syncthreads();
+    }
+
+    if (PASS & PASS_DIAG)
+        off_partial<TX3 * TY3>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
+                               a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
 // ------------------------------------------------- state in the paper's form
@@ -856,11 +1156,13 @@ __global__ void off_target_k(const OffBuf cur, const unsigned *__restrict__ maxb
 }
 
 template <class C>
-int off_ctas_per_sm_t()
+int off_ctas_per_sm_t(bool even)
 {
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, d3q19_off_pass_kernel<C, PASS_STATE, true>, PAIR_NT, 0);
+    cudaError_t e = even ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                               &n, d3q19_off_pass_kernel<C, PASS_STATE>, PAIR_NT, 0)
+                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                               &n, d3q19_off_pass1_kernel<C, PASS_STATE>, TX3 * TY3, 0);
     return e == cudaSuccess && n > 0 ? n : 2;
 }
 
@@ -872,11 +1174,11 @@ cudaError_t launch_off(const StepParams<float> &P, const PassArgs &a, const Laun
     const dim3 pg((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz);
     const cudaError_t e = launch_pdl(d3q19_off_phi_kernel<C>, pg, PHI_TX, 0, st, P, src, phi);
     if (e != cudaSuccess) return e;
-    const dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y)), block(TXP, TY3);
+    const dim3 grid(s.grid_x, s.grid_y, s.nblocks / (s.grid_x * s.grid_y));
     if (P.nx % 2 == 0)
-        return launch_pdl(d3q19_off_pass_kernel<C, PASS, true>, grid, block, 0, st, P, a, src, dst,
-                          target, phi, s.rows);
-    return launch_pdl(d3q19_off_pass_kernel<C, PASS, false>, grid, block, 0, st, P, a, src, dst,
+        return launch_pdl(d3q19_off_pass_kernel<C, PASS>, grid, dim3(TXP, TY3), 0, st, P, a, src,
+                          dst, target, phi, s.rows);
+    return launch_pdl(d3q19_off_pass1_kernel<C, PASS>, grid, dim3(TX3, TY3), 0, st, P, a, src, dst,
                       target, phi, s.rows);
 }
 
@@ -896,9 +1198,10 @@ cudaError_t pass_off_t(int pass, const StepParams<float> &P, const PassArgs &a,
 
 }  // namespace
 
-int d3q19_off_ctas_per_sm(int codec)
+int d3q19_off_ctas_per_sm(int codec, int nx)
 {
-    return codec == OFFSET_F16 ? off_ctas_per_sm_t<CodecF16>() : off_ctas_per_sm_t<CodecBF16>();
+    const bool even = nx % 2 == 0;
+    return codec == OFFSET_F16 ? off_ctas_per_sm_t<CodecF16>(even) : off_ctas_per_sm_t<CodecBF16>(even);
 }
 
 cudaError_t d3q19_off_pass(int codec, int pass, const void *params32, const PassArgs &a,

@@ -424,7 +424,7 @@ int create_impl(const lbm_grid *grid, int lattice, const lbm_params *params, voi
     }
     ctx->nsm = nsm;
     if (lattice == LBM_D3Q19) {
-        const int occ = ctx->codec >= 0 ? d3q19_off_ctas_per_sm(ctx->codec)
+        const int occ = ctx->codec >= 0 ? d3q19_off_ctas_per_sm(ctx->codec, grid->nx)
                                         : d3q19_ctas_per_sm(params->precision);
         ctx->shape = d3q19_shape(grid->nx, grid->ny, grid->nz, nsm, occ);
     } else {

@@ -237,7 +237,7 @@ cudaError_t d2q9_set_state(int precision, int nx, int ny, void *f, void *g, void
 LaunchShape d3q19_shape(int nx, int ny, int nz, int num_sms, int ctas_per_sm);
 // resident CTAs per SM of the time-step kernel (occupancy query)
 int d3q19_ctas_per_sm(int precision);
-int d3q19_off_ctas_per_sm(int codec);
+int d3q19_off_ctas_per_sm(int codec, int nx);
 cudaError_t d3q19_pass(int precision, int pass, const void *params, const PassArgs &a,
                        const LaunchShape &s, void *phi_work, cudaStream_t st);
 cudaError_t d3q19_init(int precision, const void *params, const double *phi0, void *f, void *g,
