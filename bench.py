@@ -880,6 +880,7 @@ def run_coalescence3d(args, rank, world, local_rank):
                      "peak_source": f"{src} copy bandwidth (hbm_gbs)",
                      "algorithmic_bytes_per_node": bpn, "step_ms": step_s * 1e3,
                      "kernel": ("d3q19_off_phi_kernel + d3q19_off_pass_kernel" if "off" in args.precision
+                                else "d3q19_phi_kernel + d3q19_pass32_kernel" if args.precision == "fp32"
                                 else "d3q19_phi_kernel + d3q19_pass_kernel") + " (whole step)"},
         "e2e": {"value": nodes * args.steps * world / e2e_s / 1e6, "unit": "MLUPS",
                 "h2d_bytes_per_step": 8 * nodes / args.steps,
