@@ -1,6 +1,6 @@
 """The offset-storage pass updates two x-neighbours per thread, with 32-bit
-loads and stores of both where rows have an even number of nodes and single
-values where they do not.  Both forms do the same arithmetic, so a grid of odd
+loads and stores of both, where rows have an even number of nodes, and one node
+per thread where they do not.  Both forms do the same arithmetic, so a grid of odd
 width and the same grid repeated twice in x (periodic: the same flow) give the
 same bits, at widths around the 32-node tile; and both agree with the oracle.
 """
