@@ -17,7 +17,7 @@
 //    formed once per node and direction class;
 //  * the halo columns of both thread rows are one warp's extra work instead
 //    of two warps'.
-// About 153 FP64 operations per node against about 250 in the form shared with
+// About 155 FP64 operations per node against about 250 in the form shared with
 // the FP32 kernel before.  Measured with per-step launches, whole runs of 40
 // and 400 steps: 1024 x 1024 505 -> 363 us per step (the operations alone take
 // 255 us), 16 x 128 16.5 -> 9.9 us; with 64-column tiles 341 us.
@@ -76,7 +76,7 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
 
     const int first = dir > 0 ? y0 : yend - 1;
     const int nout = yend - y0;
-    const double beta4 = 4.0 * P.beta, hd = 0.5 * (P.phil - P.phiv), q0 = hd * hd;
+    const double beta4 = 4.0 * P.beta;
     const double kap = P.kappa, k23 = P.kappa * (2.0 / 3.0), k16 = P.kappa * (1.0 / 6.0);
 
     // ring rows of march coordinate m >= -2
@@ -124,13 +124,14 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
         if (halo_phi) vd_at(mb + hq, jH);
     };
     // Eq. chemical_potencial; j is the phi ring index.  The double-well
-    // derivative is 4 beta t (t^2 - (dphi/2)^2) with t = phi - phibar
+    // derivative is left as its three factors: exactly zero in both bulk phases,
+    // and relatively accurate beside them (as t (t^2 - (dphi/2)^2), two operations
+    // less per node, it carries the rounding of t^2 there)
     auto mu_at = [&](int m, int j) {
         const double *p0 = prow(m), *v = vrow(m);
         const double c = p0[j];
         const double h = (p0[j + 1] - c) + (p0[j - 1] - c);
-        const double t = c - P.phibar;
-        double mu = (beta4 * t) * fma(t, t, -q0);
+        double mu = beta4 * (c - P.phil) * (c - P.phiv) * (c - P.phibar);
         mu = fma(-kap, h, mu);
         mu = fma(-k23, v[j], mu);
         mrow(m)[j - 1] = fma(-k16, v[j + 1] + v[j - 1], mu);
@@ -372,8 +373,7 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         const double *p0 = sm.phs + (r + 1) * WP, *vr = sm.vs + r * WP;
         const double c = p0[j];
         const double h = (p0[j + 1] - c) + (p0[j - 1] - c);
-        const double t = c - P.phibar, hd = 0.5 * (P.phil - P.phiv);
-        double mu = ((4.0 * P.beta) * t) * fma(t, t, -(hd * hd));
+        double mu = 4.0 * P.beta * (c - P.phil) * (c - P.phiv) * (c - P.phibar);
         mu = fma(-P.kappa, h, mu);
         mu = fma(-(P.kappa * (2.0 / 3.0)), vr[j], mu);
         sm.mus[tid] = fma(-(P.kappa * (1.0 / 6.0)), vr[j + 1] + vr[j - 1], mu);
