@@ -12,7 +12,8 @@
 //    and the gradient (1/2)(phi_E - phi_W) + (1/12)(v_E - v_W),
 //    (1/3) d + (1/12)(d_E + d_W).  Every term stays a difference of
 //    neighbours, so a uniform phase still gives exact zeros;
-//  * one reciprocal of rho tau_g serves 1/rho and 1/tau_g;
+//  * 1/rho and 1/tau_g are three operations each and as accurate as a divide
+//    (rcp64; one reciprocal of rho tau_g for both takes as many, and loses an ulp);
 //  * each collision is one multiply-add per population on coefficients
 //    formed once per node and direction class;
 //  * the halo columns of both thread rows are one warp's extra work instead
@@ -195,8 +196,7 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
             const double dphi = phi - P.phiv;
             const double rho = fma(P.drho, dphi, P.rhov);
             const double taug = fma(3.0 * P.dnu, dphi, fma(3.0, P.nuv, 0.5));
-            const double inv = rcp64(rho * taug);
-            const double irho = inv * taug, itg = inv * rho;
+            const double irho = rcp64(rho), itg = rcp64(taug);
             // rho u = sum_i c_i g_i + F/2
             const double ga = gv[5] - gv[7], gb = gv[8] - gv[6];
             const double jx = (gv[2] - gv[4]) + (ga + gb), jy = (gv[3] - gv[1]) + (ga - gb);
@@ -393,11 +393,10 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         const double dphi = phi - P.phiv;
         const double rho = fma(P.drho, dphi, P.rhov);
         const double taug = fma(3.0 * P.dnu, dphi, fma(3.0, P.nuv, 0.5));
-        const double inv = rcp64(rho * taug);
-        const double itg = inv * rho, it9 = (1.0 / 9.0) * itg, ri = rho * it9;
+        const double itg = rcp64(taug), it9 = (1.0 / 9.0) * itg, ri = rho * it9;
         const double k9 = fma(-0.5, it9, 1.0 / 9.0);
         sm.w[5][lane] = rho;
-        sm.w[6][lane] = inv * taug;
+        sm.w[6][lane] = rcp64(rho);
         sm.w[7][lane] = itg;
         sm.w[8][lane] = it9;
         sm.w[9][lane] = ri;

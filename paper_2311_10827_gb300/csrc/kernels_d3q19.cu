@@ -98,8 +98,8 @@ __device__ __forceinline__ void write_partial3(int tid, double d_phi, double d_E
 // The FP64 pass: one node per thread.  The FP64 pipe bounds it (one warp
 // operation per 16 cycles and SM), so the update is written for the fewest
 // operations: sums and differences of opposite populations serve the moments,
-// diagonal differences serve two gradient components, one reciprocal serves
-// rho and tau_g, and a collision is one or two multiply-adds per population on
+// diagonal differences serve two gradient components, a reciprocal is three
+// operations, and a collision is one or two multiply-adds per population on
 // coefficients formed once per node.  100^3 1515 -> 1117 us per step, 200^3 9.0 ->
 // 6.6 ms.
 template <int PASS>
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(TX3 *TY3)
         const T dphi = phi - P.phiv;
         const T rho = fma(P.drho, dphi, P.rhov);
         const T taug = fma(T(3) * P.dnu, dphi, fma(T(3), P.nuv, T(0.5)));
-        const T inv = rcp64(rho * taug), irho = inv * taug, itg = inv * rho;
+        const T irho = rcp64(rho), itg = rcp64(taug);
         const T f6 = T(-1.0 / 6.0) * phi;
         T uu = T(0), S6 = T(0);  // S6: 6 u.grad(phi)
 #pragma unroll

@@ -5,15 +5,23 @@
 
 namespace wblbm {
 
-// 1/x to about one rounding: the hardware's 20-bit estimate r and one step of
-// Householder's third-order iteration, e = 1 - x r, r (1 + e + e^2), whose
-// error is e^3 < 2^-57.  x = rho tau_g, positive and of order one.
+// 1/x: the hardware's estimate r and one step of Householder's third-order
+// iteration, e = 1 - x r, r (1 + e + e^2), whose error is e^3.  An estimate good to
+// 2^-19 leaves 1/16 of an ulp beside the final rounding's half.  For every
+// positive or negative x for which x and 1/x are normal numbers (that is any
+// density and relaxation time of a run); where the estimate is infinite or zero
+// (x zero, subnormal, infinite or at least 2^1022) it is the result, which for
+// zeros, infinities and NaN is the divide's.  The estimate's exponent is tested as an
+// integer: the FP64 pipe, which bounds the kernels that use this, gets three
+// operations.
 __device__ __forceinline__ double rcp64(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r, 1.0);
-    return fma(fma(e, e, e), r, r);
+    const double y = fma(fma(e, e, e), r, r);
+    const unsigned k = ((unsigned)__double2hiint(r) >> 20) & 0x7ffu;
+    return k - 1u < 0x7feu ? y : r;
 }
 
 }  // namespace wblbm
