@@ -14,8 +14,9 @@
 //    neighbours, so a uniform phase still gives exact zeros;
 //  * 1/rho and 1/tau_g are three operations each and as accurate as a divide
 //    (rcp64; one reciprocal of rho tau_g for both takes as many, and loses an ulp);
-//  * each collision is one multiply-add per population on coefficients
-//    formed once per node and direction class;
+//  * each collision is one multiply-add per population (two for relaxation
+//    times above 2, see relax64) on coefficients formed once per node and
+//    direction class;
 //  * the halo columns of both thread rows are one warp's extra work instead
 //    of two warps'.
 // About 155 FP64 operations per node against about 250 in the form shared with
@@ -246,8 +247,15 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                 const double z = (itf * P.alpha) * mu;
                 fd[n] = fma(itf, scur, fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, fcur[0])));
                 const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
+                auto collide_f = [&](auto inc) {
 #pragma unroll
-                for (int i = 1; i < 9; ++i) fd[i * N + n] = fma(omf, fcur[i], i < 5 ? ka : kd);
+                    for (int i = 1; i < 9; ++i)
+                        fd[i * N + n] = relax64<inc.value>(fcur[i], itf, omf, i < 5 ? ka : kd);
+                };
+                if (P.incr & INCR_F)
+                    collide_f(std::true_type{});
+                else
+                    collide_f(std::false_type{});
                 // Eq. BGK-NS with Eqs. G_i, GGi.  Per direction pair: even part
                 // E = w [itg A + c.u (4.5 rho itg c.u + 3 k drho c.grad phi)], odd part
                 // O = w [3 rho itg c.u + 3 k c.F], k = 1 - itg/2, A = 3p - 1.5 rho |u|^2;
@@ -255,7 +263,6 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                 const double A = fma(-1.5, ruu, p3);
                 const double omg = 1.0 - itg;
                 const double it9 = (1.0 / 9.0) * itg, k9 = fma(-0.5, it9, 1.0 / 9.0);
-                gd[n] = fma(omg, gv[0], itg * fma(4.0 / 9.0, A, -p3));
                 const double e0 = it9 * A, ri = rho * it9, e1 = 4.5 * ri, o1 = 3.0 * ri;
                 const double e2 = (1.5 * P.drho) * k9, o2 = 3.0 * k9;
                 auto pair = [&](double cu, double cF, double cq, double &s, double &d) {
@@ -264,19 +271,27 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                     s = E + O;
                     d = E - O;
                 };
-                double s, d;
-                pair(ux, Fx, qx, s, d);
-                gd[2 * N + n] = fma(omg, gv[2], s);
-                gd[4 * N + n] = fma(omg, gv[4], d);
-                pair(uy, Fy, qy, s, d);
-                gd[3 * N + n] = fma(omg, gv[3], s);
-                gd[1 * N + n] = fma(omg, gv[1], d);
-                pair(ux + uy, Fx + Fy, qx + qy, s, d);
-                gd[5 * N + n] = fma(0.25, s, omg * gv[5]);
-                gd[7 * N + n] = fma(0.25, d, omg * gv[7]);
-                pair(uy - ux, Fy - Fx, qy - qx, s, d);
-                gd[6 * N + n] = fma(0.25, s, omg * gv[6]);
-                gd[8 * N + n] = fma(0.25, d, omg * gv[8]);
+                auto collide_g = [&](auto inc) {
+                    constexpr bool INC = inc.value;
+                    double s, d;
+                    gd[n] = relax64<INC>(gv[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
+                    pair(ux, Fx, qx, s, d);
+                    gd[2 * N + n] = relax64<INC>(gv[2], itg, omg, s);
+                    gd[4 * N + n] = relax64<INC>(gv[4], itg, omg, d);
+                    pair(uy, Fy, qy, s, d);
+                    gd[3 * N + n] = relax64<INC>(gv[3], itg, omg, s);
+                    gd[1 * N + n] = relax64<INC>(gv[1], itg, omg, d);
+                    pair(ux + uy, Fx + Fy, qx + qy, s, d);
+                    gd[5 * N + n] = relax64<INC>(gv[5], itg, omg, 0.25 * s);
+                    gd[7 * N + n] = relax64<INC>(gv[7], itg, omg, 0.25 * d);
+                    pair(uy - ux, Fy - Fx, qy - qx, s, d);
+                    gd[6 * N + n] = relax64<INC>(gv[6], itg, omg, 0.25 * s);
+                    gd[8 * N + n] = relax64<INC>(gv[8], itg, omg, 0.25 * d);
+                };
+                if (P.incr & INCR_G)
+                    collide_g(std::true_type{});
+                else
+                    collide_g(std::false_type{});
             }
         }
 #pragma unroll
@@ -421,8 +436,15 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         const double z = (itf * P.alpha) * m0[k];
         fd[n] = fma(itf, sm.snz[lane], fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, v[0])));
         const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
+        auto collide_f = [&](auto inc) {
 #pragma unroll
-        for (int i = 1; i < 9; ++i) fd[i * N + n] = fma(omf, v[i], i < 5 ? ka : kd);
+            for (int i = 1; i < 9; ++i)
+                fd[i * N + n] = relax64<inc.value>(v[i], itf, omf, i < 5 ? ka : kd);
+        };
+        if (P.incr & INCR_F)
+            collide_f(std::true_type{});
+        else
+            collide_f(std::false_type{});
         return;
     }
     const double rho = sm.w[5][lane], itg = sm.w[7][lane], it9 = sm.w[8][lane],
@@ -438,22 +460,29 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         s = E + O;
         d = E - O;
     };
-    double s, d;
-    if (warp == 1) {
-        pair(ux, Fx, qx, s, d);
-        gd[2 * N + n] = fma(omg, v[2], s);
-        gd[4 * N + n] = fma(omg, v[4], d);
-        pair(uy, Fy, qy, s, d);
-        gd[3 * N + n] = fma(omg, v[3], s);
-        gd[1 * N + n] = fma(omg, v[1], d);
-    } else if (warp == 2) {
-        pair(ux + uy, Fx + Fy, qx + qy, s, d);
-        gd[5 * N + n] = fma(0.25, s, omg * v[5]);
-        gd[7 * N + n] = fma(0.25, d, omg * v[7]);
-    } else {
-        gd[n] = fma(omg, v[0], itg * fma(4.0 / 9.0, A, -p3));
-        pair(uy - ux, Fy - Fx, qy - qx, s, d);
-        gd[6 * N + n] = fma(0.25, s, omg * v[6]);
-        gd[8 * N + n] = fma(0.25, d, omg * v[8]);
-    }
+    auto collide_g = [&](auto inc) {
+        constexpr bool INC = inc.value;
+        double s, d;
+        if (warp == 1) {
+            pair(ux, Fx, qx, s, d);
+            gd[2 * N + n] = relax64<INC>(v[2], itg, omg, s);
+            gd[4 * N + n] = relax64<INC>(v[4], itg, omg, d);
+            pair(uy, Fy, qy, s, d);
+            gd[3 * N + n] = relax64<INC>(v[3], itg, omg, s);
+            gd[1 * N + n] = relax64<INC>(v[1], itg, omg, d);
+        } else if (warp == 2) {
+            pair(ux + uy, Fx + Fy, qx + qy, s, d);
+            gd[5 * N + n] = relax64<INC>(v[5], itg, omg, 0.25 * s);
+            gd[7 * N + n] = relax64<INC>(v[7], itg, omg, 0.25 * d);
+        } else {
+            gd[n] = relax64<INC>(v[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
+            pair(uy - ux, Fy - Fx, qy - qx, s, d);
+            gd[6 * N + n] = relax64<INC>(v[6], itg, omg, 0.25 * s);
+            gd[8 * N + n] = relax64<INC>(v[8], itg, omg, 0.25 * d);
+        }
+    };
+    if (P.incr & INCR_G)
+        collide_g(std::true_type{});
+    else
+        collide_g(std::false_type{});
 }

@@ -294,14 +294,20 @@ __global__ void __launch_bounds__(TX3 *TY3)
             const T itf = P.inv_tauf, omf = T(1) - itf, z = (itf * P.alpha) * mu;
             __stcs(fd + n, fma(itf, snz, fma(T(-2.0 / 3.0), z, fma(T(-5.0 / 6.0), Sh, fv[0]))));
             const T ka = T(1.0 / 18.0) * (z - Sh), ke = T(1.0 / 36.0) * fma(T(0.5), Sh, z);
+            auto collide_f = [&](auto inc) {
 #pragma unroll
-            for (int i = 1; i < 19; ++i) __stcs(fd + (i * N + n), fma(omf, fv[i], i <= 6 ? ka : ke));
+                for (int i = 1; i < 19; ++i)
+                    __stcs(fd + (i * N + n), relax64<inc.value>(fv[i], itf, omf, i <= 6 ? ka : ke));
+            };
+            if (P.incr & INCR_F)
+                collide_f(std::true_type{});
+            else
+                collide_f(std::false_type{});
             // hydrodynamic population, pairs of opposite directions: even part
             // E = w [A/tau_g + c.u (4.5 rho/tau_g c.u + 3 k c.grad rho)], odd part
             // O = w [3 rho/tau_g c.u + 3 k c.F], k = 1 - 1/(2 tau_g); coefficients at the
             // faces' weight, the edges take half at the end
             const T p3 = T(3) * p, A = fma(T(-1.5), ruu, p3), omg = T(1) - itg;
-            __stcs(gd + n, fma(omg, gv[0], itg * fma(T(1.0 / 3.0), A, -p3)));
             const T itw = T(1.0 / 18.0) * itg, kw = fma(T(-0.5), itw, T(1.0 / 18.0));
             const T e0 = itw * A, ri = rho * itw, e1 = T(4.5) * ri, o1 = T(3) * ri;
             const T e2 = (T(0.5) * P.drho) * kw, o2 = T(3) * kw;
@@ -311,21 +317,25 @@ __global__ void __launch_bounds__(TX3 *TY3)
                 if ((cx || cy) && cz) s = cz > 0 ? s + v[2] : s - v[2];
                 return s;
             };
+            auto collide_g = [&](auto inc) {
+                constexpr bool INC = inc.value;
+                __stcs(gd + n, relax64<INC>(gv[0], itg, omg, itg * fma(T(1.0 / 3.0), A, -p3)));
 #pragma unroll
-            for (int i = 1; i < 19; ++i) {
-                const int o = opp(i);
-                if (o < i) continue;
-                const T cu = dot(c3x(i), c3y(i), c3z(i), u), cF = dot(c3x(i), c3y(i), c3z(i), F);
-                const T cq = dot(c3x(i), c3y(i), c3z(i), q);
-                const T E = fma(cu, fma(e2, cq, e1 * cu), e0), O = fma(o2, cF, o1 * cu);
-                if (i <= 6) {
-                    __stcs(gd + (i * N + n), fma(omg, gv[i], E + O));
-                    __stcs(gd + (o * N + n), fma(omg, gv[o], E - O));
-                } else {
-                    __stcs(gd + (i * N + n), fma(T(0.5), E + O, omg * gv[i]));
-                    __stcs(gd + (o * N + n), fma(T(0.5), E - O, omg * gv[o]));
+                for (int i = 1; i < 19; ++i) {
+                    const int o = opp(i);
+                    if (o < i) continue;
+                    const T cu = dot(c3x(i), c3y(i), c3z(i), u), cF = dot(c3x(i), c3y(i), c3z(i), F);
+                    const T cq = dot(c3x(i), c3y(i), c3z(i), q);
+                    const T E = fma(cu, fma(e2, cq, e1 * cu), e0), O = fma(o2, cF, o1 * cu);
+                    const T w = i <= 6 ? T(1) : T(0.5);
+                    __stcs(gd + (i * N + n), relax64<INC>(gv[i], itg, omg, w * (E + O)));
+                    __stcs(gd + (o * N + n), relax64<INC>(gv[o], itg, omg, w * (E - O)));
                 }
-            }
+            };
+            if (P.incr & INCR_G)
+                collide_g(std::true_type{});
+            else
+                collide_g(std::false_type{});
         }
         }  // col_ok
         {

@@ -16,6 +16,7 @@ namespace wblbm {
 template <typename T>
 struct StepParams {
     int nx, ny, nz;
+    int incr;            // FP64: INCR_* populations relax by their increments
     long long N;         // nodes
     T kappa, beta;       // Eqs. beta, suiface_tension
     T phil, phiv, phibar;
@@ -24,6 +25,9 @@ struct StepParams {
     T nuv, dnu;          // nu  = nuv  + (phi - phiv) * dnu  (Eq. vis)
     T G[3];              // body force
 };
+
+// Bits of StepParams::incr: f, g with relaxation times above 2 (see relax64).
+enum : int { INCR_F = 1, INCR_G = 2 };
 
 // ------------------------------------------------ parameters (host only)
 
@@ -125,6 +129,9 @@ void fill_step_params(StepParams<T> &P, const lbm_grid &g, const lbm_params &p, 
     P.ny = g.ny;
     P.nz = g.nz;
     P.N = (long long)g.nx * g.ny * g.nz;
+    // (nu with a tenth of its range to spare: phi overshoots its phases a little)
+    const double nu = fmax(p.nu_l, p.nu_v) + 0.1 * fabs(p.nu_l - p.nu_v);
+    P.incr = (d.tau_f > 2.0 ? INCR_F : 0) | (0.5 + 3.0 * nu > 2.0 ? INCR_G : 0);
     P.kappa = (T)d.kappa;
     P.beta = (T)d.beta;
     P.phil = (T)p.phi_l;

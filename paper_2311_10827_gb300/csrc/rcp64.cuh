@@ -1,7 +1,10 @@
-// The FP64 reciprocal of the step kernels.  Internal header.
+// The FP64 reciprocal and the relaxation of a population in the step kernels.
+// Internal header.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 namespace wblbm {
 
@@ -22,6 +25,20 @@ __device__ __forceinline__ double rcp64(double x)
     const double y = fma(fma(e, e, e), r, r);
     const unsigned k = ((unsigned)__double2hiint(r) >> 20) & 0x7ffu;
     return k - 1u < 0x7feu ? y : r;
+}
+
+// x relaxed by a rate r plus s, omr = 1 - r.  For r >= 1/2, 1 - r is exact and x (1 - r) + s
+// one operation.  Below (tau > 2) it is rounded, and every population would
+// relax by up to 2^-54 more or less than the r that the equilibrium part is
+// multiplied by: a drift of the sums that should stay (phi, momentum) that
+// grows with every step, where independent roundings average out.  There (INC)
+// the population is moved by its increment -r x + s, one operation more.  A
+// run's parameters choose (StepParams::incr), not a node's rate: warps on an
+// interface would run both forms (64^3 238 -> 312 us per step).
+template <bool INC>
+__device__ __forceinline__ double relax64(double x, double r, double omr, double s)
+{
+    return INC ? x + fma(-r, x, s) : fma(omr, x, s);
 }
 
 }  // namespace wblbm
