@@ -954,18 +954,18 @@ __device__ inline double geq_of(const EqData &e, float p, int i)
 // Initial state: macros (phi0, mu0, p = 0, u = 0) at every node, f_i(x, 0) =
 // f^eq_i(phi0(x), mu0(x)) stored at x - c_i as an offset from the equilibrium
 // of the storing node's macros; g = g^eq (offsets 0).  Two passes: the first
-// forms mu0 and the node's two distinct moving values fa, fe (faces, edges;
-// FP64 scratch), the second stores their differences from the neighbours'
-// equilibria.  The FP64 pipe bounds both; the scales are powers of two, so
+// forms mu0 and the node's moving values, fa on the faces (FP64 scratch) and
+// exactly half of it on the edges, the second stores their differences from the
+// neighbours' equilibria.  Of the state only the parity that is initialised is
+// written: phi0 may lie in the other one.  The FP64 pipe bounds both; the scales are powers of two, so
 // the division by s_f is a multiplication after the rounding to FP32 (a
 // divide of its own for each of the 19 values made this 13.1 ms at 256^3,
 // against 3.0 ms now).
 template <class C>
 __global__ void __launch_bounds__(256)
     d3q19_off_init_macros_k(const StepParams<double> Pd, const StepParams<float> P,
-                            const double *__restrict__ phi0, double *__restrict__ fa,
-                            double *__restrict__ fe, OffBuf o, float *__restrict__ S, float s_f,
-                            float s_g)
+                            const double *__restrict__ phi0, double *__restrict__ fa, OffBuf o,
+                            float *__restrict__ S, float s_f, float s_g)
 {
     const unsigned N = (unsigned)P.N, n = blockIdx.x * 256u + threadIdx.x;
     if (n == 0) {
@@ -978,8 +978,8 @@ __global__ void __launch_bounds__(256)
     const Nb b = make_nb((int)(n - r * nx), (int)(r % ny), (int)(r / ny), P.nx, P.ny, P.nz);
     const double c = __ldg(phi0 + n);
     const double mu = mu_of_field(Pd, phi0, b, c), am = Pd.alpha * mu;
+    static_assert(2.0 * w3(7) == w3(1), "edge values are half the face values");
     fa[n] = w3(1) * am;
-    fe[n] = w3(7) * am;
     const float phi_hi = (float)c, mu_f = (float)mu;
     o.M[n] = phi_hi;
     o.M[N + n] = mu_f;
@@ -993,8 +993,7 @@ __global__ void __launch_bounds__(256)
 
 template <class C>
 __global__ void __launch_bounds__(256)
-    d3q19_off_init_k(const StepParams<float> P, const double *__restrict__ fa,
-                     const double *__restrict__ fe, OffBuf o, float s_f)
+    d3q19_off_init_k(const StepParams<float> P, const double *__restrict__ fa, OffBuf o, float s_f)
 {
     const unsigned N = (unsigned)P.N, n = blockIdx.x * 256u + threadIdx.x;
     if (n >= N) return;
@@ -1006,7 +1005,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
         const unsigned m = b.at(c3x(i), c3y(i), c3z(i));
-        const double d = i <= 6 ? __ldg(fa + m) - eqa : __ldg(fe + m) - eqe;
+        const double d = i <= 6 ? __ldg(fa + m) - eqa : fma(0.5, __ldg(fa + m), -eqe);
         o.h[i * N + n] = C::enc((float)d * inv);
     }
 #pragma unroll
@@ -1215,8 +1214,8 @@ cudaError_t d3q19_off_pass(int codec, int pass, const void *params32, const Pass
 }
 
 cudaError_t d3q19_off_init(int codec, const void *params64, const void *params32,
-                           const double *phi0, double *tmp_a, double *tmp_e, void *f, void *g,
-                           void *S, const float *target_host, cudaStream_t st)
+                           const double *phi0, double *tmp, void *f, void *g, void *S,
+                           const float *target_host, cudaStream_t st)
 {
     const StepParams<double> &Pd = *static_cast<const StepParams<double> *>(params64);
     const StepParams<float> &P = *static_cast<const StepParams<float> *>(params32);
@@ -1224,13 +1223,13 @@ cudaError_t d3q19_off_init(int codec, const void *params64, const void *params32
     const OffBuf o = off_view(f, g, P.N);
     const float sf = target_host[0], sg = target_host[1];
     if (codec == OFFSET_F16) {
-        d3q19_off_init_macros_k<CodecF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp_a, tmp_e, o,
-                                                              (float *)S, sf, sg);
-        d3q19_off_init_k<CodecF16><<<nb, 256, 0, st>>>(P, tmp_a, tmp_e, o, sf);
+        d3q19_off_init_macros_k<CodecF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp, o, (float *)S, sf,
+                                                              sg);
+        d3q19_off_init_k<CodecF16><<<nb, 256, 0, st>>>(P, tmp, o, sf);
     } else {
-        d3q19_off_init_macros_k<CodecBF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp_a, tmp_e, o,
-                                                               (float *)S, sf, sg);
-        d3q19_off_init_k<CodecBF16><<<nb, 256, 0, st>>>(P, tmp_a, tmp_e, o, sf);
+        d3q19_off_init_macros_k<CodecBF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp, o, (float *)S, sf,
+                                                               sg);
+        d3q19_off_init_k<CodecBF16><<<nb, 256, 0, st>>>(P, tmp, o, sf);
     }
     d3q19_off_prep_k<<<dim3((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz), PHI_TX, 0, st>>>(P, o);
     return cudaGetLastError();

@@ -514,10 +514,8 @@ int lbm_init_phi(lbm_ctx *ctx, const double *phi, int on_device)
         e = cudaMemcpyAsync(ctx->scw, OFFSET_INITIAL_SCALES, sizeof OFFSET_INITIAL_SCALES,
                             cudaMemcpyHostToDevice, ctx->stream);
         if (e == cudaSuccess)
-            // (the other g buffer, 38 N bytes, is free here: scratch)
-            e = d3q19_off_init(ctx->codec, &ctx->pd, &ctx->pf, src, ctx->aux,
-                               static_cast<double *>(ctx->g[1]), ctx->f[0], ctx->g[0], ctx->S,
-                               OFFSET_INITIAL_SCALES, ctx->stream);
+            e = d3q19_off_init(ctx->codec, &ctx->pd, &ctx->pf, src, ctx->aux, ctx->f[0], ctx->g[0],
+                               ctx->S, OFFSET_INITIAL_SCALES, ctx->stream);
     } else if (ctx->lattice == LBM_D3Q19) {
         e = d3q19_init(ctx->prm.precision, &ctx->pd, src, ctx->f[0], ctx->g[0], ctx->S,
                        ctx->stream);

@@ -279,10 +279,10 @@ __host__ __device__ inline OffsetLayout offset_layout(long long N, int Q, int D)
 cudaError_t d3q19_off_pass(int codec, int pass, const void *params32, const PassArgs &a,
                            const LaunchShape &s, void *phi_work, const float *target,
                            cudaStream_t st);
-// tmp_a, tmp_e: scratch of N doubles each
+// tmp: scratch of N doubles
 cudaError_t d3q19_off_init(int codec, const void *params64, const void *params32,
-                           const double *phi0, double *tmp_a, double *tmp_e, void *f, void *g,
-                           void *S, const float *target_host, cudaStream_t st);
+                           const double *phi0, double *tmp, void *f, void *g, void *S,
+                           const float *target_host, cudaStream_t st);
 cudaError_t d3q19_off_get_state(int codec, const void *params32, const void *f, const void *g,
                                 const void *S, double *fo, double *go, double *So, cudaStream_t st);
 cudaError_t d3q19_off_set_state(int codec, const void *params32, void *f, void *g, void *S,
