@@ -57,3 +57,43 @@ def test_phi_may_lie_in_the_other_state_buffers(env, shape, precision, buffer):
         assert np.array_equal(x, y)
     capi.lbm_destroy(a.handle)
     b.close()
+
+
+C3 = [(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1)]
+for _a, _b in ((0, 1), (0, 2), (1, 2)):
+    for _s in ((1, 1), (1, -1), (-1, 1), (-1, -1)):
+        _v = [0, 0, 0]
+        _v[_a], _v[_b] = _s
+        C3.append(tuple(_v))
+
+
+@pytest.mark.parametrize("size", [1e-39, 1e-3])
+@pytest.mark.parametrize("precision", ["f16off", "bf16off"])
+def test_initial_offsets_round_once(env, precision, size):
+    """The stored moving offsets of an initial field are (f - f^eq)/s rounded to FP32
+    and then to 16 bits, also where f - f^eq is below the smallest normal FP32
+    value (the scale s = 2^-16 lifts it back into the range of BF16)."""
+    torch, capi, sim = env
+    shape, N = (20, 6, 5), 600
+    rng = np.random.default_rng(5)
+    phi0 = size * rng.uniform(0.5, 1.5, shape[::-1])
+    s, bufs = on_caller_buffers(env, shape, precision)
+    s.init_phi(phi0)
+    s.sync()
+    raw = bufs[0].cpu()
+    h = raw[:38 * N].view(torch.int16).numpy().reshape((19,) + phi0.shape)
+    off = (38 * N + 255) // 256 * 256
+    mu_f = raw[off:off + 8 * N].view(torch.float32).numpy()[N:].reshape(phi0.shape)
+    at = lambda a, c: np.roll(a, (-c[2], -c[1], -c[0]), axis=(0, 1, 2))  # noqa: E731
+    d = [at(phi0, c) - phi0 for c in C3]
+    lap = sum(d[1:7]) / 3.0 + sum(d[7:]) / 6.0
+    mu = 4.0 * s.beta * (phi0 - 1.0) * phi0 * (phi0 - 0.5) - s.kappa * lap
+    for i, c in enumerate(C3):
+        if i == 0:
+            continue
+        w = 1.0 / 18.0 if i < 7 else 1.0 / 36.0
+        eq = (np.float32(w) * (np.float32(s.alpha) * mu_f)).astype(np.float64)
+        v = torch.tensor(((at(w * s.alpha * mu, c) - eq) * 65536.0).astype(np.float32))
+        want = v.to(torch.float16 if precision == "f16off" else torch.bfloat16).view(torch.int16)
+        assert np.array_equal(h[i], want.numpy())
+    capi.lbm_destroy(s.handle)
