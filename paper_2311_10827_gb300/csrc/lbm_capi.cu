@@ -10,6 +10,7 @@
 
 #include "lbm.h"
 #include "lbm_internal.h"
+#include "parts.h"
 
 using namespace wblbm;
 
@@ -1819,7 +1820,7 @@ struct lbm_adjoint {
     int K, max_steps, nsteps, recorded;
     size_t snap;        // bytes of one state snapshot (f, g, S at the context's precision)
     size_t slot;        // bytes of one segment slot: a snapshot, then its moments
-    char *mem;          // the one allocation that holds every buffer below
+    void *mem[13];      // the blocks that hold the buffers below (null: unused)
     char *ckpt;         // (max_steps / K + 1) snapshots
     char *seg;          // K slots of the segment being reversed
     int real;           // adjoint arithmetic: 0 FP64, 1 FP32 (the context's precision)
@@ -1858,7 +1859,8 @@ int restore(lbm_ctx *ctx, const char *src, long long step)
 
 void adjoint_free(lbm_adjoint *a)
 {
-    if (a->mem) cudaFree(a->mem);
+    for (void *q : a->mem)
+        if (q) cudaFree(q);
     free(a);
 }
 
@@ -1886,36 +1888,31 @@ int lbm_adjoint_create(lbm_ctx *ctx, int checkpoint_every, int max_steps, lbm_ad
     const size_t nck = (size_t)(max_steps / checkpoint_every + 1);
     a->real = ctx->prm.precision == LBM_FP64 ? 0 : 1;
     a->rsz = a->real == 0 ? sizeof(double) : sizeof(float);
-    // one allocation for every buffer (each 256-byte aligned): a recorder is
-    // created and destroyed by every differentiated run, and freeing 13 buffers
-    // one by one costs a synchronisation each
-    struct {
-        void **p;
-        size_t bytes;
-    } const part[] = {{(void **)&a->ckpt, nck * a->snap},
-                      {(void **)&a->seg, (size_t)checkpoint_every * a->slot},
-                      {(void **)&a->phi0, N * sizeof(double)},
-                      {(void **)&a->macro, N * sizeof(double)},
-                      {&a->work, 6 * N * a->rsz},
-                      {&a->lpt, N * a->rsz},
-                      {(void **)&a->dpar, 3 * sizeof(double)},
-                      {&a->lf[0], Q * N * a->rsz},
-                      {&a->lf[1], Q * N * a->rsz},
-                      {&a->lg[0], Q * N * a->rsz},
-                      {&a->lg[1], Q * N * a->rsz},
-                      {&a->lS[0], N * a->rsz},
-                      {&a->lS[1], N * a->rsz}};
-    size_t total = 0;
-    for (const auto &q : part) total += (q.bytes + 255) / 256 * 256;
-    if (cudaMalloc((void **)&a->mem, total) != cudaSuccess) {
+    // one allocation where the device gives one that large: a recorder is created
+    // and destroyed by every differentiated run
+    const Part part[] = {{(void **)&a->ckpt, nck * a->snap},
+                         {(void **)&a->seg, (size_t)checkpoint_every * a->slot},
+                         {(void **)&a->phi0, N * sizeof(double)},
+                         {(void **)&a->macro, N * sizeof(double)},
+                         {&a->work, 6 * N * a->rsz},
+                         {&a->lpt, N * a->rsz},
+                         {(void **)&a->dpar, 3 * sizeof(double)},
+                         {&a->lf[0], Q * N * a->rsz},
+                         {&a->lf[1], Q * N * a->rsz},
+                         {&a->lg[0], Q * N * a->rsz},
+                         {&a->lg[1], Q * N * a->rsz},
+                         {&a->lS[0], N * a->rsz},
+                         {&a->lS[1], N * a->rsz}};
+    constexpr int nparts = sizeof part / sizeof part[0];
+    static_assert(nparts == sizeof a->mem / sizeof a->mem[0], "one entry per part");
+    auto alloc = [](void **q, size_t bytes) {
+        if (cudaMalloc(q, bytes) == cudaSuccess) return true;
         cudaGetLastError();
+        return false;
+    };
+    if (!alloc_parts(part, nparts, a->mem, alloc, [](void *q) { cudaFree(q); })) {
         adjoint_free(a);
         return LBM_ERR_OOM;
-    }
-    size_t off = 0;
-    for (const auto &q : part) {
-        *q.p = a->mem + off;
-        off += (q.bytes + 255) / 256 * 256;
     }
     ctx->recentre = 0;  // the recorded states keep one equilibrium shift
     *out = a;
