@@ -338,11 +338,11 @@ __global__ void __launch_bounds__(SM64_NT, 4)
 {
     constexpr int TX = SM64_TX, WP = SmallSmem64::WP, WM = SmallSmem64::WM;
     __shared__ SmallSmem64 sm;
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nx = P.nx, ny = P.ny;
     const unsigned N = (unsigned)P.N;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * 2;
+    const int x0 = bx * TX, y0 = blockIdx.y * 2;
     const double *__restrict__ fsrc = static_cast<const double *>(a.f_src);
     const double *__restrict__ gsrc = static_cast<const double *>(a.g_src);
     // this thread's node in stages 2 .. 5

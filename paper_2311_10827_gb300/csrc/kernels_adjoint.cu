@@ -107,8 +107,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2)
                           R *__restrict__ lphi, R *__restrict__ lmu, R *__restrict__ lgphi,
                           R *__restrict__ lgmu, double *dpar)
 {
-    pdl_wait();
-    const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned n = pdl_wait(blockIdx.x) * blockDim.x + threadIdx.x;
     const unsigned N = geo.N;
     constexpr R IC = R(1.0 / CS2A);
     R itf_part = R(0);
@@ -300,9 +299,9 @@ __global__ void __launch_bounds__(AMX *AMY)
                const R *__restrict__ lgmu, R *__restrict__ lpt_out, double *dpar)
 {
     __shared__ R smu[AHX * AHY];
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * AMX, y0 = blockIdx.y * AMY;
+    const int x0 = bx * AMX, y0 = blockIdx.y * AMY;
     for (int q = tid; q < AHX * AHY; q += AMX * AMY) {
         // any grid size: a full modulo for the (at most 2) halo coordinates
         int xx = (x0 - 1 + q % AHX) % geo.nx, yy = (y0 - 1 + q / AHX) % geo.ny;

@@ -893,15 +893,15 @@ template <typename T, int TX, int PASS>
 __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ctas))
     d2q9_pass_kernel(const StepParams<T> P, PassArgs a, int rows)
 {
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int y0 = blockIdx.y * rows;
     // march direction: alternating between neighbouring row tiles, and
     // reversed on every other step
     const int dir = ((blockIdx.y & 1) ? -1 : 1) * (a.flip ? -1 : 1);
     __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
-    run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, blockIdx.x * TX, y0,
-                           min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + blockIdx.x, bph);
+    run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, bx * TX, y0,
+                          min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + bx, bph);
 }
 
 // The FP32 step of a small or mid-sized grid: one 64 x 4 tile per CTA of as many
@@ -924,12 +924,12 @@ __global__ void __launch_bounds__(SHX *SHY, 4)
 {
     constexpr int WP = ShotSmem::WP, WM = ShotSmem::WM, NT = SHX * SHY;
     __shared__ ShotSmem sm;
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int tx = threadIdx.x, ty = threadIdx.y, lin = ty * SHX + tx;
     const int nx = P.nx, ny = P.ny;
     const unsigned N = (unsigned)P.N;
     const bool small = ny < 8;
-    const int x0 = blockIdx.x * SHX, y0 = blockIdx.y * SHY;
+    const int x0 = bx * SHX, y0 = blockIdx.y * SHY;
     const float *__restrict__ fsrc = static_cast<const float *>(a.f_src);
     const float *__restrict__ gsrc = static_cast<const float *>(a.g_src);
     const int xo = x0 + tx, yo = y0 + ty;
@@ -939,7 +939,7 @@ __global__ void __launch_bounds__(SHX *SHY, 4)
     if (PASS & PASS_STATE) {
         a_src = *a.eqs_src;
         a_dst = *a.eqs_target;
-        if (a.eqs_dst && blockIdx.x == 0 && blockIdx.y == 0 && lin == 0) *a.eqs_dst = a_dst;
+        if (a.eqs_dst && bx == 0 && blockIdx.y == 0 && lin == 0) *a.eqs_dst = a_dst;
     }
     auto pull = [&](const float *s, int y, unsigned xm, unsigned x, unsigned xp, float v[9],
                     float *lo) {
@@ -999,8 +999,8 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     d2q9_batch_kernel(const BatchCase *__restrict__ cases, const BatchTile *__restrict__ tiles,
                       int parity, DiagPartial *partials)
 {
-    pdl_wait();
-    const BatchTile t = tiles[blockIdx.x];
+    const int bx = pdl_wait(blockIdx.x);
+    const BatchTile t = tiles[bx];
     const BatchCase &c = cases[t.c];
     const StepParams<T> P = *reinterpret_cast<const StepParams<T> *>(
         sizeof(T) == 4 ? (const void *)&c.pf : (const void *)&c.pd);
@@ -1019,7 +1019,7 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
     run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, t.x0, t.y0, t.yend,
-                           parity ? -t.dir : t.dir, blockIdx.x, bph);
+                          parity ? -t.dir : t.dir, bx, bph);
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int *p)

@@ -34,9 +34,9 @@ template <typename T>
 __global__ void __launch_bounds__(PHI_TX)
     d3q19_phi_kernel(const StepParams<T> P, const T *__restrict__ f, T *__restrict__ phi)
 {
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
-    const int x = blockIdx.x * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+    const int x = bx * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
     if (x >= nx) return;
     const unsigned N = (unsigned)P.N;
     const Nb b = make_nb(x, y, z, nx, ny, nz);
@@ -114,11 +114,11 @@ __global__ void __launch_bounds__(TX3 *TY3)
     __shared__ T phs[RP * PA];
     __shared__ T mus[RM * MA];
 
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
-    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int x0 = bx * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
     const int x = x0 + tx, y = y0 + ty;
     const bool col_ok = x < nx && y < ny;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(TX3 *TY3)
 
     if (PASS & PASS_DIAG)
         write_partial3<TX3 * TY3>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
-                                  a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+                                  a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + bx);
 }
 
 // The FP32 pass: two nodes adjacent in x per thread (TXP x TY3 threads), their
@@ -380,11 +380,11 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     __shared__ __align__(16) float phs[RP * PA];
     __shared__ __align__(16) float mus[RM * MA];
 
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TXP + tx;
-    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int x0 = bx * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
     const int x = x0 + 2 * tx, y = y0 + ty;
     const bool okA = x < nx && y < ny, okB = EVEN ? okA : (x + 1 < nx && y < ny);
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     if (PASS & PASS_STATE) {
         a_src = *a.eqs_src;
         a_dst = *a.eqs_target;
-        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) *a.eqs_dst = a_dst;
+        if (bx == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) *a.eqs_dst = a_dst;
     }
 
     for (int d = 0; d < 5; ++d) {
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
 
     if (PASS & PASS_DIAG)
         write_partial3<PAIR_NT>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
-                                a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+                                a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + bx);
 }
 
 // ------------------------------------------------------------ initial state

@@ -109,9 +109,9 @@ template <class C>
 __global__ void __launch_bounds__(PHI_TX)
     d3q19_off_phi_kernel(const StepParams<float> P, const OffBuf src, float *__restrict__ phi)
 {
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
-    const int x = blockIdx.x * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+    const int x = bx * PHI_TX + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
     if (x >= nx) return;
     const unsigned N = (unsigned)P.N;
     const Nb b = make_nb(x, y, z, nx, ny, nz);
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(PHI_TX)
     float sh = C::dec(__ldg(src.h + n));
 #pragma unroll
     for (int i = 1; i < 19; ++i) sh += C::dec(__ldg(src.h + (i * N + b.at(-c3x(i), -c3y(i), -c3z(i)))));
-    phi[n] = __ldg(src.M + 6 * N + n) + __ldg(src.sc) * sh;
+    phi[n] = __ldg(src.M + 6 * N + n) + __ldg(after_wait(src.sc)) * sh;
 }
 
 // B(x) from stored macros (after an initial condition or a state exchange)
@@ -227,19 +227,20 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
     // g^eq_i = w_i (A + 3 c.j + (9/2)(c.j)^2 / rho); ring of three planes per quantity
     __shared__ __align__(16) float qs[6][RM * MA];
 
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TXP + tx;
-    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int x0 = bx * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
     const int x = x0 + 2 * tx, y = y0 + ty;
     const bool ok = x < nx && y < ny;  // (both nodes: nx is even)
     const unsigned plane = (unsigned)nx * ny;
-    const float s_f = __ldg(src.sc), s_g = __ldg(src.sc + 1);
-    const float t_f = __ldg(target), t_g = __ldg(target + 1);
+    const float *ssc = after_wait(src.sc), *tsc = after_wait(target);
+    const float s_f = __ldg(ssc), s_g = __ldg(ssc + 1);
+    const float t_f = __ldg(tsc), t_g = __ldg(tsc + 1);
     const float it_f = 1.0f / t_f, it_g = 1.0f / t_g;  // powers of two: exact
-    if ((PASS & PASS_STATE) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) {
+    if ((PASS & PASS_STATE) && bx == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) {
         dst.sc[0] = t_f;
         dst.sc[1] = t_g;
     }
@@ -594,7 +595,7 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
 
     if (PASS & PASS_DIAG)
         off_partial<PAIR_NT>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
-                             a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+                             a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + bx);
 }
 
 // The same pass with one node per thread, for rows of an odd number of nodes:
@@ -620,19 +621,20 @@ __global__ void __launch_bounds__(TX3 *TY3)
     __shared__ float4 qa[RQ * MA];
     __shared__ float2 qb[RQ * MA];
 
-    pdl_wait();
+    const int bx = pdl_wait(blockIdx.x);
     const int nx = P.nx, ny = P.ny, nz = P.nz;
     const unsigned N = (unsigned)P.N;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX3 + tx;
-    const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY3;
+    const int x0 = bx * TX3, y0 = blockIdx.y * TY3;
     const int z0 = blockIdx.z * planes, zend = min(z0 + planes, nz);
     const int x = x0 + tx, y = y0 + ty;
     const bool col_ok = x < nx && y < ny;
     const unsigned plane = (unsigned)nx * ny;
-    const float s_f = __ldg(src.sc), s_g = __ldg(src.sc + 1);
-    const float t_f = __ldg(target), t_g = __ldg(target + 1);
+    const float *ssc = after_wait(src.sc), *tsc = after_wait(target);
+    const float s_f = __ldg(ssc), s_g = __ldg(ssc + 1);
+    const float t_f = __ldg(tsc), t_g = __ldg(tsc + 1);
     const float it_f = 1.0f / t_f, it_g = 1.0f / t_g;  // powers of two: exact
-    if ((PASS & PASS_STATE) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) {
+    if ((PASS & PASS_STATE) && bx == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) {
         dst.sc[0] = t_f;
         dst.sc[1] = t_g;
     }
@@ -916,7 +918,7 @@ __global__ void __launch_bounds__(TX3 *TY3)
 
     if (PASS & PASS_DIAG)
         off_partial<TX3 * TY3>(tid, d_phi, d_E, d_u2, d_mumin, d_mumax, d_bud, d_bad,
-                               a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+                               a.partials + (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + bx);
 }
 
 // ------------------------------------------------- state in the paper's form
