@@ -346,8 +346,25 @@ __device__ __forceinline__ bool seg_ok(int nx, const void *f, const void *g, con
            (((unsigned long long)f | (unsigned long long)g | (unsigned long long)S) & 15) == 0;
 }
 
+// Eq. chemical_potencial with the Laplacian of Eq. Laplace (FP32), written as a
+// sum of differences (cancellation-friendly):
+// lap = (2/3) sum_axis (phi_n - phi) + (1/6) sum_diag (phi_n - phi).
+// pm, p0, pp: the phi rows at y - 1, y, y + 1, the own column at j.
+__device__ __forceinline__ float mu_node(const StepParams<float> &P, const float *pm,
+                                         const float *p0, const float *pp, int j)
+{
+    const float c = p0[j];
+    const float ax = (p0[j + 1] - c) + (p0[j - 1] - c) + (pp[j] - c) + (pm[j] - c);
+    const float dg = (pp[j + 1] - c) + (pp[j - 1] - c) + (pm[j + 1] - c) + (pm[j - 1] - c);
+    const float lap = fmaf(float(2.0 / 3.0), ax, float(1.0 / 6.0) * dg);
+    return fmaf(4.0f * P.beta * (c - P.phil) * (c - P.phiv), c - P.phibar, -(P.kappa * lap));
+}
+
 // The update of one node (FP32): its moments, forces, both collisions and the
-// stores (or the moments and diagnostics that PASS asks for).  pm, p0, pp and
+// stores (or the moments and diagnostics that PASS asks for).  Every multiply-add
+// of a population, a moment or mu (mu_node) is written out, so that each kernel
+// that inlines this rounds alike: a run takes its plain steps and its
+// diagnostics steps through different ones.  pm, p0, pp and
 // mm, m0, mp: the phi and mu rows at y - 1, y, y + 1, the own column at j and k;
 // f, lo: the pulled populations of f (rest population as a pair); gv: those of g;
 // n: the node's index.
@@ -407,7 +424,7 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
     }
     // p = cs2/(1-w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0(u)],
     // rho s_0 = -(2/3) rho |u|^2 for D2Q9
-    const T p = T(0.6) * (sum_moving(gv) + T(0.5) * ugr - T(2.0 / 3.0) * rho * uu);
+    const T p = T(0.6) * fmaf(-(T(2.0 / 3.0) * rho), uu, fmaf(T(0.5), ugr, sum_moving(gv)));
 
     if (PASS & PASS_DIAG) {
         {
@@ -460,14 +477,14 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         const T Sh = fmaf(T(1.5), S, -(T(0.5) * Sprev));
         // alpha mu in the source buffer's shifted variables; dsh moves
         // the written values to the target shift (0 unless it changed)
-        const T am = P.alpha * mu - a_src;
+        const T am = fmaf(P.alpha, mu, -a_src);
         const T dsh = a_src - a_dst;
         const T itf = P.inv_tauf;
         {
             // f_0* = f_0 - (f_0 - f_0^eq)/tau_f - (8/9) Sh with
             // f_0 - f_0^eq = (5/9) alpha mu - sum_{i!=0} f_i
-            const T d0 = -(T(5.0 / 9.0) * am - snz) * itf - T(8.0 / 9.0) * Sh -
-                         T(5.0 / 9.0) * dsh;
+            const T ne = fmaf(T(5.0 / 9.0), am, -snz);
+            const T d0 = fmaf(T(-5.0 / 9.0), dsh, fmaf(T(-8.0 / 9.0), Sh, -(ne * itf)));
             if (REST_PAIR) {
                 // (hi, lo) + d0 with an exact two-sum on the high word
                 const T sl = locur + d0;
@@ -481,7 +498,6 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
             }
         }
         const T ea = T(1.0 / 9.0) * am, ed = T(1.0 / 36.0) * am;
-        // (explicit multiply-adds: every kernel that inlines this rounds alike)
         const T sa = fmaf(T(-1.0 / 18.0), Sh, T(1.0 / 9.0) * dsh);
         const T sd = fmaf(T(1.0 / 36.0), Sh, T(1.0 / 36.0) * dsh);
         // Hydrodynamic population, Eq. BGK-NS with Eqs. G_i, Siu, GGi:
@@ -492,9 +508,10 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         //     = 3 w_i k [c.F + (c.u)(c.grad rho)], k = 1 - 1/(2 tau_g)
         // (the two u.grad rho terms cancel).  Opposite directions share
         // the even part and flip the odd part.
-        const T kg = T(1) - T(0.5) * itg;
+        const T kg = fmaf(T(-0.5), itg, T(1));
         const T A = fmaf(-(T(1.5) * rho), uu, T(3) * p);
-        st_stream(gd + n, gv[0] + ((T(4.0 / 9.0) * A - T(3) * p) - gv[0]) * itg);  // G_0 = 0
+        // G_0 = 0
+        st_stream(gd + n, fmaf(fmaf(T(4.0 / 9.0), A, -(T(3) * p)) - gv[0], itg, gv[0]));
         {
             // two populations per paired instruction: f 1..4 and 5..8 in
             // pairs; g the two axis and the two diagonal direction pairs
@@ -716,18 +733,9 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
         }
     };
 
-    // Eq. chemical_potencial with the Laplacian of Eq. Laplace, written as a
-    // sum of differences (cancellation-friendly in FP32):
-    // lap = (2/3) sum_axis (phi_n - phi) + (1/6) sum_diag (phi_n - phi).
+    // j is the mu ring index; the phi ring index of the same column is j + 1
     auto mu_at = [&](int sm, int s0, int sp, int j) -> T {
-        // j is the mu ring index; the phi ring index of the same column is j+1
-        const T *pm = phs + sm * WP, *p0 = phs + s0 * WP, *pp = phs + sp * WP;
-        const T c = p0[j + 1];
-        const T ax = (p0[j + 2] - c) + (p0[j] - c) + (pp[j + 1] - c) + (pm[j + 1] - c);
-        const T dg = (pp[j + 2] - c) + (pp[j] - c) + (pm[j + 2] - c) + (pm[j] - c);
-        const T lap = T(2.0 / 3.0) * ax + T(1.0 / 6.0) * dg;
-        const T bulk = T(4) * P.beta * (c - P.phil) * (c - P.phiv) * (c - P.phibar);
-        return bulk - P.kappa * lap;
+        return mu_node(P, phs + sm * WP, phs + s0 * WP, phs + sp * WP, j + 1);
     };
     // mu at the row with ring slot s0; sm / sp are the slots of rows y-1 / y+1
     auto mu_row = [&](int sm, int s0, int sp) {
@@ -968,16 +976,11 @@ __global__ void __launch_bounds__(SHX *SHY, 4)
     sm.phs[(ty + 2) * WP + tx + 2] = f[0] + (lo + sum_moving(f));
     sm.phs[hy * WP + tx + 2] = h[0] + (hlo + sum_moving(h));
     __syncthreads();
-    // mu of the tile's rows and one row and column around it (the arithmetic of
-    // d2q9_tile's mu_at); r: mu ring row (phi ring row r + 1), j: mu ring column
+    // mu of the tile's rows and one row and column around it; r: mu ring row (phi
+    // ring row r + 1), j: mu ring column
     auto mu_at = [&](int r, int j) {
-        const float *p0 = sm.phs + (r + 1) * WP, *pm = p0 - WP, *pp = p0 + WP;
-        const float c = p0[j + 1];
-        const float ax = (p0[j + 2] - c) + (p0[j] - c) + (pp[j + 1] - c) + (pm[j + 1] - c);
-        const float dg = (pp[j + 2] - c) + (pp[j] - c) + (pm[j + 2] - c) + (pm[j] - c);
-        const float lap = float(2.0 / 3.0) * ax + float(1.0 / 6.0) * dg;
-        const float bulk = 4.0f * P.beta * (c - P.phil) * (c - P.phiv) * (c - P.phibar);
-        sm.mus[r * WM + j] = bulk - P.kappa * lap;
+        const float *p0 = sm.phs + (r + 1) * WP;
+        sm.mus[r * WM + j] = mu_node(P, p0 - WP, p0, p0 + WP, j + 1);
     };
     mu_at(ty + 1, tx + 1);
     if (ty < 2)
