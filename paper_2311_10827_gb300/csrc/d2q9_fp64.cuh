@@ -164,7 +164,7 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
     mu_rows(-1);
 
     for (int t = 0; t < nout; t += 2) {
-        const int m = t + ty, row = first + dir * m;
+        const int m = t + ty;
         const bool out_ok = col_ok && m < nout;
         const Rows r = rows_of(m);
         double gv[9], Sprev = 0.0;

@@ -368,20 +368,21 @@ __device__ __forceinline__ float mu_node(const StepParams<float> &P, const float
 // mm, m0, mp: the phi and mu rows at y - 1, y, y + 1, the own column at j and k;
 // f, lo: the pulled populations of f (rest population as a pair); gv: those of g;
 // n: the node's index.
-template <typename T, int PASS, int NT>
-__device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs &a, const T *pm,
-                              const T *p0, const T *pp, const T *mm, const T *m0,
-                              const T *mp, int j, int k, const T fcur[9], T locur,
-                              const T gv[9], T Sprev, T a_src, T a_dst, unsigned n,
-                              int lin, T (*dacc)[NT], T (*facc)[NT], int *dbad)
+template <int PASS, int NT>
+__device__ __forceinline__ void d2q9_node(const StepParams<float> &P, const PassArgs &a,
+                                          const float *pm, const float *p0, const float *pp,
+                                          const float *mm, const float *m0, const float *mp, int j,
+                                          int k, const float fcur[9], float locur,
+                                          const float gv[9], float Sprev, float a_src, float a_dst,
+                                          unsigned n, int lin, float (*dacc)[NT],
+                                          float (*facc)[NT], int *dbad)
 {
-    constexpr bool REST_PAIR = true;
     const unsigned N = (unsigned)P.N;
     // phi from the pulled values (Eq. order-parameter)
-    const T snz = sum_moving(fcur);
-    const T phi = fcur[0] + (locur + snz);
-    const T mu = m0[k];
-    T gpx, gpy, Fx, Fy, rho, inv_rho, itg, ux, uy, grx, gry, ugr, uu, S;
+    const float snz = sum_moving(fcur);
+    const float phi = fcur[0] + (locur + snz);
+    const float mu = m0[k];
+    float gpx, gpy, Fx, Fy, rho, inv_rho, itg, ux, uy, grx, gry, ugr, uu, S;
     // Eq. gradient: grad = 3 sum_{i!=0} w_i c_i Psi(x + c_i)
     //   = (1/3)(axis differences) + (1/12)(diagonal differences)
     {
@@ -405,8 +406,8 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         const float2 rn = fma2(f2(phi - P.phiv), make_float2(P.drho, P.dnu),
                                make_float2(P.rhov, P.nuv));
         rho = rn.x;
-        inv_rho = Arith<T>::rcp(rho);
-        itg = Arith<T>::rcp(fmaf(3.0f, rn.y, 0.5f));  // nu = cs2 (tau_g - 1/2)
+        inv_rho = Arith<float>::rcp(rho);
+        itg = Arith<float>::rcp(fmaf(3.0f, rn.y, 0.5f));  // nu = cs2 (tau_g - 1/2)
         // rho u = sum_i c_i g_i + F/2
         const float jx = (gv[2] - gv[4]) + ((gv[5] - gv[6]) + (gv[8] - gv[7]));
         const float jy = (gv[3] - gv[1]) + ((gv[5] + gv[6]) - (gv[7] + gv[8]));
@@ -424,7 +425,8 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
     }
     // p = cs2/(1-w0) [sum_{i!=0} g_i + u.grad(rho)/2 + rho s_0(u)],
     // rho s_0 = -(2/3) rho |u|^2 for D2Q9
-    const T p = T(0.6) * fmaf(-(T(2.0 / 3.0) * rho), uu, fmaf(T(0.5), ugr, sum_moving(gv)));
+    const float p =
+        0.6f * fmaf(-(float(2.0 / 3.0) * rho), uu, fmaf(0.5f, ugr, sum_moving(gv)));
 
     if (PASS & PASS_DIAG) {
         {
@@ -455,16 +457,16 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         }
     }
     if (PASS & PASS_MACROS_T) {
-        static_cast<T *>(a.mt_phi)[n] = phi;
-        static_cast<T *>(a.mt_p)[n] = p;
-        static_cast<T *>(a.mt_mu)[n] = mu;
-        static_cast<T *>(a.mt_u)[n] = ux;
-        static_cast<T *>(a.mt_u)[(size_t)N + n] = uy;
+        static_cast<float *>(a.mt_phi)[n] = phi;
+        static_cast<float *>(a.mt_p)[n] = p;
+        static_cast<float *>(a.mt_mu)[n] = mu;
+        static_cast<float *>(a.mt_u)[n] = ux;
+        static_cast<float *>(a.mt_u)[(size_t)N + n] = uy;
     }
     if (PASS & PASS_STATE) {
-        T *__restrict__ fd = static_cast<T *>(a.f_dst);
-        T *__restrict__ gd = static_cast<T *>(a.g_dst);
-        st_stream(static_cast<T *>(a.S_out) + n, S);
+        float *__restrict__ fd = static_cast<float *>(a.f_dst);
+        float *__restrict__ gd = static_cast<float *>(a.g_dst);
+        st_stream(static_cast<float *>(a.S_out) + n, S);
 
         // CH population, Eq. BGK with Eq. H_i and Eq. F_i:
         // f* = f - (f - f^eq)/tau_f + w_i b_i (1.5 S - 0.5 S_prev),
@@ -474,32 +476,29 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         // the increments sum to sum_i F_i up to unbiased rounding (the
         // form f (1 - 1/tau) + f^eq/tau would add (1 - 1/tau + 1/tau - 1)
         // sum_{i!=0} f_i, a systematic FP32 drift of the phi mass).
-        const T Sh = fmaf(T(1.5), S, -(T(0.5) * Sprev));
+        const float Sh = fmaf(1.5f, S, -(0.5f * Sprev));
         // alpha mu in the source buffer's shifted variables; dsh moves
         // the written values to the target shift (0 unless it changed)
-        const T am = fmaf(P.alpha, mu, -a_src);
-        const T dsh = a_src - a_dst;
-        const T itf = P.inv_tauf;
+        const float am = fmaf(P.alpha, mu, -a_src);
+        const float dsh = a_src - a_dst;
+        const float itf = P.inv_tauf;
         {
             // f_0* = f_0 - (f_0 - f_0^eq)/tau_f - (8/9) Sh with
             // f_0 - f_0^eq = (5/9) alpha mu - sum_{i!=0} f_i
-            const T ne = fmaf(T(5.0 / 9.0), am, -snz);
-            const T d0 = fmaf(T(-5.0 / 9.0), dsh, fmaf(T(-8.0 / 9.0), Sh, -(ne * itf)));
-            if (REST_PAIR) {
-                // (hi, lo) + d0 with an exact two-sum on the high word
-                const T sl = locur + d0;
-                const T hi = fcur[0] + sl;
-                const T bp = hi - fcur[0];
-                const T lo = (fcur[0] - (hi - bp)) + (sl - bp);
-                st_stream(fd + n, hi);
-                st_stream(fd + (9u * N + n), lo);
-            } else {
-                st_stream(fd + n, fcur[0] + d0);
-            }
+            const float ne = fmaf(float(5.0 / 9.0), am, -snz);
+            const float d0 =
+                fmaf(float(-5.0 / 9.0), dsh, fmaf(float(-8.0 / 9.0), Sh, -(ne * itf)));
+            // (hi, lo) + d0 with an exact two-sum on the high word
+            const float sl = locur + d0;
+            const float hi = fcur[0] + sl;
+            const float bp = hi - fcur[0];
+            const float lo = (fcur[0] - (hi - bp)) + (sl - bp);
+            st_stream(fd + n, hi);
+            st_stream(fd + (9u * N + n), lo);
         }
-        const T ea = T(1.0 / 9.0) * am, ed = T(1.0 / 36.0) * am;
-        const T sa = fmaf(T(-1.0 / 18.0), Sh, T(1.0 / 9.0) * dsh);
-        const T sd = fmaf(T(1.0 / 36.0), Sh, T(1.0 / 36.0) * dsh);
+        const float ea = float(1.0 / 9.0) * am, ed = float(1.0 / 36.0) * am;
+        const float sa = fmaf(float(-1.0 / 18.0), Sh, float(1.0 / 9.0) * dsh);
+        const float sd = fmaf(float(1.0 / 36.0), Sh, float(1.0 / 36.0) * dsh);
         // Hydrodynamic population, Eq. BGK-NS with Eqs. G_i, Siu, GGi:
         // g* = g + (g^eq - g)/tau_g + G_i.  With A = 3p - 1.5 rho |u|^2,
         // g^eq_i = w_i [A + 4.5 rho (c.u)^2] + 3 w_i rho (c.u) (i != 0), and
@@ -508,10 +507,10 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
         //     = 3 w_i k [c.F + (c.u)(c.grad rho)], k = 1 - 1/(2 tau_g)
         // (the two u.grad rho terms cancel).  Opposite directions share
         // the even part and flip the odd part.
-        const T kg = fmaf(T(-0.5), itg, T(1));
-        const T A = fmaf(-(T(1.5) * rho), uu, T(3) * p);
+        const float kg = fmaf(-0.5f, itg, 1.0f);
+        const float A = fmaf(-(1.5f * rho), uu, 3.0f * p);
         // G_0 = 0
-        st_stream(gd + n, fmaf(fmaf(T(4.0 / 9.0), A, -(T(3) * p)) - gv[0], itg, gv[0]));
+        st_stream(gd + n, fmaf(fmaf(float(4.0 / 9.0), A, -(3.0f * p)) - gv[0], itg, gv[0]));
         {
             // two populations per paired instruction: f 1..4 and 5..8 in
             // pairs; g the two axis and the two diagonal direction pairs
@@ -561,23 +560,21 @@ __device__ __forceinline__ void d2q9_node(const StepParams<T> &P, const PassArgs
 // each stage waits for next, carried from tile to tile); else each thread
 // loads its own pulls into registers, through the read-only path (NC: data
 // constant for the launch) or from L2 only (multi-step launches).
-template <typename T, int TX, int PASS, bool NC = true, bool SEG = false>
-__device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const StepParams<T> &P,
-                                          const PassArgs &a, int x0, int y0, int yend, int dir,
-                                          int part, unsigned &bph)
+template <int TX, int PASS, bool NC = true, bool SEG = false>
+__device__ __forceinline__ void d2q9_tile(TileSmem<float, TX> &sm, float *dyn,
+                                          const StepParams<float> &P, const PassArgs &a, int x0,
+                                          int y0, int yend, int dir, int part, unsigned &bph)
 {
-    using SM = TileSmem<T, TX>;
+    using SM = TileSmem<float, TX>;
     using SL = SegLayout<TX>;
-    static_assert(sizeof(T) == 4, "FP64 storage runs d2q9_tile64");
     // staged diagnostics step (its own layout of the staging memory)
     constexpr bool DSEG = SEG && (PASS & PASS_DIAG);
     constexpr int R = SM::R, WP = SM::WP, WM = SM::WM;
-    constexpr bool REST_PAIR = true;
-    constexpr int NT = SM::NT, NACC = DiagAcc<T>::NACC, NW = NT / 32;
-    T *const phs = sm.phs;
-    T *const mus = sm.mus;
-    T(*const dacc)[NT] = reinterpret_cast<T(*)[NT]>(dyn + (DSEG ? SL::DACC : 0));
-    T(*const facc)[NT] = dacc + NACC;
+    constexpr int NT = SM::NT, NACC = DiagAcc<float>::NACC, NW = NT / 32;
+    float *const phs = sm.phs;
+    float *const mus = sm.mus;
+    float(*const dacc)[NT] = reinterpret_cast<float(*)[NT]>(dyn + (DSEG ? SL::DACC : 0));
+    float(*const facc)[NT] = dacc + NACC;
     float *const stg = reinterpret_cast<float *>(dyn);
     int *const dbad = &sm.bad;
     const int lin = threadIdx.y * TX + threadIdx.x;
@@ -586,8 +583,8 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
     const unsigned N = (unsigned)P.N;
     const bool small = ny < 4;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const T *__restrict__ fsrc = static_cast<const T *>(a.f_src);
-    const T *__restrict__ gsrc = static_cast<const T *>(a.g_src);
+    const float *__restrict__ fsrc = static_cast<const float *>(a.f_src);
+    const float *__restrict__ gsrc = static_cast<const float *>(a.g_src);
     constexpr bool NEED_S = (PASS & (PASS_STATE | PASS_DIAG)) != 0;
     constexpr bool STAGE_S = NEED_S && SEG && !DSEG;  // S staged (else loaded into registers)
 
@@ -605,8 +602,8 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
     // FP32: equilibrium shift of the source buffer and of the writes (a uniform
     // shift of mu in f^eq; phi, the moments and the stencils do not see it, so
     // only a time step reads it)
-    T a_src = T(0), a_dst = T(0);
-    if (REST_PAIR && (PASS & PASS_STATE)) {
+    float a_src = 0.0f, a_dst = 0.0f;
+    if (PASS & PASS_STATE) {
         a_src = *a.eqs_src;
         a_dst = *a.eqs_target;
         if (a.eqs_dst && x0 == 0 && y0 == 0 && lin == 0) *a.eqs_dst = a_dst;
@@ -618,20 +615,20 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
     auto slot = [&](int row) { return (dir * (row - first) + 2) % R; };
 
     // phi = f_0 + rest into ring slot sl, column j
-    auto put_phi = [&](int sl, int j, T f0, T rest) { phs[sl * WP + j] = f0 + rest; };
+    auto put_phi = [&](int sl, int j, float f0, float rest) { phs[sl * WP + j] = f0 + rest; };
     // phi at row `row` for the own column (keeping the pulled values) and the
     // halo columns, from the thread's own loads.
-    auto phi_row = [&](int row, int sl, T v[9], T &lo) {
+    auto phi_row = [&](int row, int sl, float v[9], float &lo) {
         const unsigned rm = (unsigned)wrap_row(row - 1, ny, small) * nx;
         const unsigned r0 = (unsigned)wrap_row(row, ny, small) * nx;
         const unsigned rp = (unsigned)wrap_row(row + 1, ny, small) * nx;
         pull9<NC>(fsrc, N, rm, r0, rp, xOm, xO, xOp, v);
-        lo = REST_PAIR ? ldp<NC>(fsrc + (9u * N + r0 + xO)) : T(0);
+        lo = ldp<NC>(fsrc + (9u * N + r0 + xO));
         put_phi(sl, tx + 2, v[0], lo + sum_moving(v));
         if (tx < 4) {
-            T h[9];
+            float h[9];
             pull9<NC>(fsrc, N, rm, r0, rp, xHm, xH, xHp, h);
-            const T hlo = REST_PAIR ? ldp<NC>(fsrc + (9u * N + r0 + xH)) : T(0);
+            const float hlo = ldp<NC>(fsrc + (9u * N + r0 + xH));
             put_phi(sl, jH, h[0], hlo + sum_moving(h));
         }
     };
@@ -718,28 +715,28 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
         bph ^= 1u << st;
     };
     // phi row from stage st (thread row ty), keeping the own pulls
-    auto phi_row_seg = [&](int sl, int st, T v[9], T &lo) {
+    auto phi_row_seg = [&](int sl, int st, float v[9], float &lo) {
         const float *F = fbuf(st) + ty * SL::NF * SL::W;
 #pragma unroll
         for (int i = 0; i < 9; ++i) v[i] = F[i * SL::W + tx + 4 - cxv(i)];
         lo = F[9 * SL::W + tx + 4];
         put_phi(sl, tx + 2, v[0], lo + sum_moving(v));
         if (tx < 4) {
-            T h[9];
+            float h[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) h[i] = F[i * SL::W + jH + 2 - cxv(i)];
-            const T hlo = F[9 * SL::W + jH + 2];
+            const float hlo = F[9 * SL::W + jH + 2];
             put_phi(sl, jH, h[0], hlo + sum_moving(h));
         }
     };
 
     // j is the mu ring index; the phi ring index of the same column is j + 1
-    auto mu_at = [&](int sm, int s0, int sp, int j) -> T {
+    auto mu_at = [&](int sm, int s0, int sp, int j) -> float {
         return mu_node(P, phs + sm * WP, phs + s0 * WP, phs + sp * WP, j + 1);
     };
     // mu at the row with ring slot s0; sm / sp are the slots of rows y-1 / y+1
     auto mu_row = [&](int sm, int s0, int sp) {
-        T *mr = mus + s0 * WM;
+        float *mr = mus + s0 * WM;
         mr[tx + 1] = mu_at(sm, s0, sp, tx + 1);
         if (tx < 2) mr[jM] = mu_at(sm, s0, sp, jM);
     };
@@ -748,16 +745,16 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
     // mu and the non-finite flag are exact in the storage type
     if (PASS & PASS_DIAG) {
 #pragma unroll
-        for (int q = 0; q < NACC; ++q) dacc[q][lin] = T(0);
-        facc[0][lin] = T(0);
-        facc[1][lin] = T(INFINITY);
-        facc[2][lin] = T(-INFINITY);
+        for (int q = 0; q < NACC; ++q) dacc[q][lin] = 0.0f;
+        facc[0][lin] = 0.0f;
+        facc[1][lin] = INFINITY;
+        facc[2][lin] = -INFINITY;
         if (lin == 0) *dbad = 0;  // read after the march's barriers
     }
 
     // prologue: phi rows y0-2 .. y0+1 (the own row y0+ty keeps its values),
     // mu rows y0-1 .. y0
-    T fcur[9], fnext[9], locur = T(0), lonext = T(0);
+    float fcur[9], fnext[9], locur = 0.0f, lonext = 0.0f;
     if constexpr (DSEG) {
         // one f buffer: the two phi row pairs one after the other
         if (rseg >= 0 && rseg < NSR) fence_proxy_async_global();
@@ -811,8 +808,8 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
         const int row = first + dir * (t + ty);
         const bool out_ok = col_ok && t + ty < nout;
         const int st = (t / TYB) & 1;
-        T gv[9];
-        T Sprev = T(0);
+        float gv[9];
+        float Sprev = 0.0f;
         const unsigned nrow = (unsigned)wrap_row(row, ny, small) * nx;
         if constexpr (SEG) {
             // this iteration's stage has landed (the other stage, and a
@@ -821,7 +818,7 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
             // the previous iteration is done)
             wait_stage(st);
             if (DSEG && NEED_S && out_ok)
-                Sprev = __ldcg(static_cast<const T *>(a.S) + (nrow + xo));  // from L2
+                Sprev = __ldcg(static_cast<const float *>(a.S) + (nrow + xo));  // from L2
             phi_row_seg(ring(2 + ty), st, fnext, lonext);
             if (t + TYB < nout) bulk_expect(st ^ 1, t + TYB, true);
         } else {
@@ -830,8 +827,8 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
             const unsigned rp = (unsigned)wrap_row(row + 1, ny, small) * nx;
             pull9<NC>(gsrc, N, rm, nrow, rp, xOm, xO, xOp, gv);
             if (NEED_S && out_ok)
-                Sprev = NC ? __ldcs(static_cast<const T *>(a.S) + (nrow + xo))
-                           : __ldcg(static_cast<const T *>(a.S) + (nrow + xo));  // from L2
+                Sprev = NC ? __ldcs(static_cast<const float *>(a.S) + (nrow + xo))
+                           : __ldcg(static_cast<const float *>(a.S) + (nrow + xo));  // from L2
             phi_row(first + dir * (t + 2 + ty), ring(2 + ty), fnext, lonext);
         }
         __syncthreads();
@@ -849,9 +846,9 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
                 for (int i = 0; i < 9; ++i) gv[i] = G[i * SL::W + tx + 4 - cxv(i)];
                 if (STAGE_S) Sprev = stg[st * SL::STAGE + SL::SOFF + ty * TX + tx];
             }
-            d2q9_node<T, PASS, NT>(P, a, phs + sm * WP, phs + s0 * WP, phs + sp * WP, mus + sm * WM,
-                                   mus + s0 * WM, mus + sp * WM, tx + 2, tx + 1, fcur, locur, gv,
-                                   Sprev, a_src, a_dst, nrow + xo, lin, dacc, facc, dbad);
+            d2q9_node<PASS, NT>(P, a, phs + sm * WP, phs + s0 * WP, phs + sp * WP, mus + sm * WM,
+                                mus + s0 * WM, mus + sp * WM, tx + 2, tx + 1, fcur, locur, gv, Sprev,
+                                a_src, a_dst, nrow + xo, lin, dacc, facc, dbad);
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) fcur[i] = fnext[i];
@@ -864,8 +861,8 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<T, TX> &sm, T *dyn, const Ste
         const double d_E = (double)dacc[2][lin] + (double)dacc[3][lin];
         const double d_bud = 1.5 * ((double)dacc[4][lin] + (double)dacc[5][lin]) -
                              0.5 * ((double)dacc[6][lin] + (double)dacc[7][lin]);
-        write_partial<NW, T>(sm.red, lin, d_phi, d_E, facc[0][lin], facc[1][lin], facc[2][lin],
-                             d_bud, *dbad ? T(1) : T(0), a.partials + part);
+        write_partial<NW, float>(sm.red, lin, d_phi, d_E, facc[0][lin], facc[1][lin], facc[2][lin],
+                                 d_bud, *dbad ? 1.0f : 0.0f, a.partials + part);
     }
 }
 
@@ -889,7 +886,7 @@ __device__ __forceinline__ void run_tile(typename SmemOf<T, TX>::type &sm, T *dy
     if constexpr (sizeof(T) == 8)
         d2q9_tile64<TX, PASS, NC>(sm, dyn, P, a, x0, y0, yend, dir, part);
     else
-        d2q9_tile<T, TX, PASS, NC, SEG>(sm, dyn, P, a, x0, y0, yend, dir, part, bph);
+        d2q9_tile<TX, PASS, NC, SEG>(sm, dyn, P, a, x0, y0, yend, dir, part, bph);
 }
 
 // The kernels' dynamic shared memory (tile_dyn_bytes of their tile width).
@@ -990,8 +987,8 @@ __global__ void __launch_bounds__(SHX *SHY, 4)
     __syncthreads();
     if (!ok) return;
     const float *p0 = sm.phs + (ty + 2) * WP, *m0 = sm.mus + (ty + 1) * WM;
-    d2q9_node<float, PASS, NT>(P, a, p0 - WP, p0, p0 + WP, m0 - WM, m0, m0 + WM, tx + 2, tx + 1, f,
-                               lo, gv, Sprev, a_src, a_dst, n, lin, nullptr, nullptr, nullptr);
+    d2q9_node<PASS, NT>(P, a, p0 - WP, p0, p0 + WP, m0 - WM, m0, m0 + WM, tx + 2, tx + 1, f,
+                        lo, gv, Sprev, a_src, a_dst, n, lin, nullptr, nullptr, nullptr);
 }
 
 // Batched: CTA k runs tile k of a flat tile table over many independent grids
@@ -1512,11 +1509,6 @@ cudaError_t seg_attrs()
     return e;
 }
 
-// Most tiles for which d2q9_small64_kernel is used: one per SM.  With two per SM
-// its schedulers hold two warps of about 85 operations each, no fewer than the
-// one warp of 177 that d2q9_tile64 gives them on such a grid, and more in all.
-constexpr int SM64_MAX_TILES = 152;
-
 // Rows per 64-column tile of an FP64 step.  A scheduler's FP64 pipe takes the
 // warps it holds one operation after the other, so a step takes the most tiles
 // that an SM gets times their operations: about 165 for two rows and 69 to
@@ -1557,7 +1549,10 @@ cudaError_t launch_pass(const void *params, const PassArgs &a, const LaunchShape
     if constexpr (sizeof(T) == 8 && !(PASS & (PASS_DIAG | PASS_MACROS))) {
         if constexpr (PASS == PASS_STATE) {
             const dim3 tiles((P.nx + SM64_TX - 1) / SM64_TX, (P.ny + 1) / 2);
-            if (tiles.x * (long long)tiles.y <= SM64_MAX_TILES)
+            // at most one tile per SM: with two, its schedulers hold two warps of
+            // about 85 operations each, no fewer than the one warp of 177 that
+            // d2q9_tile64 gives them on such a grid, and more in all
+            if (tiles.x * (long long)tiles.y <= (s.num_sms > 0 ? s.num_sms : 152))
                 return launch_pdl(d2q9_small64_kernel, tiles, SM64_NT, 0, st, P, a);
         }
         // no partial records: the tiles need not be those of `s`

@@ -602,7 +602,9 @@ __global__ void __launch_bounds__(PAIR_NT, 3)
 // there the two-node form has to load and store single values (twice the
 // requests for the same sectors) and was 2 to 10% slower than this one
 // (177 x 44 x 219 FP16 188 against 170 us per step).  Each value is formed by the same
-// operations in the same order, so both give the same bits.
+// operations in the same order.  Which of them become multiply-adds is the
+// compiler's choice here and written out above, after that choice: a test
+// holds the two forms to the same bits.
 template <class C, int PASS>
 __global__ void __launch_bounds__(TX3 *TY3)
     d3q19_off_pass1_kernel(const StepParams<float> P, PassArgs a, const OffBuf src, const OffBuf dst,
@@ -770,7 +772,6 @@ __global__ void __launch_bounds__(TX3 *TY3)
             const float4 A0 = qa[qslot(zz) * MA + cq];
             flo = -(2.0f / 3.0f) * A0.x + s_f * C::dec(hr(0));
             gv[0] = (1.0f / 3.0f) * A0.y - 3.0f * p_own + s_g * C::dec(kr(0));
-            fv[0] = 0.0f;
         }
 #pragma unroll
         for (int i = 1; i < 19; ++i) {
