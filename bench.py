@@ -96,16 +96,26 @@ def measured_peaks():
 
 
 def kernel_hash():
-    """First 16 hex digits of the sha256 of the kernel sources with comments
-    and blank lines removed: a traffic record belongs to the code it was
-    taken on, whatever happens to the comments since."""
+    """First 16 hex digits of the sha256 of the kernel sources, and of the headers
+    beside them that they include, with comments and blank lines removed: a
+    traffic record belongs to the code it was taken on, whatever happens to the
+    comments since."""
     import re
     h = hashlib.sha256()
-    for rel in KERNEL_SOURCES:
-        with open(os.path.join(ROOT, rel)) as fh:
+    todo, seen = [os.path.join(ROOT, rel) for rel in KERNEL_SOURCES], set()
+    while todo:
+        path = todo.pop(0)
+        if path in seen:
+            continue
+        seen.add(path)
+        with open(path) as fh:
             text = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         text = re.sub(r"//[^\n]*", "", text)
         h.update("\n".join(l.rstrip() for l in text.split("\n") if l.strip()).encode())
+        for name in re.findall(r'^\s*#\s*include\s+"([^"]+)"', text, flags=re.M):
+            header = os.path.join(os.path.dirname(path), name)
+            if os.path.exists(header):  # others are on the include path: the C ABI
+                todo.append(header)
     return h.hexdigest()[:16]
 
 
