@@ -43,14 +43,14 @@ struct TileSmem64 {
 template <int TX, int PASS, bool NC>
 __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                                             const StepParams<double> &P, const PassArgs &a, int x0,
-                                            int y0, int yend, int dir, int part)
+                                            int y0, int yend, int dir, int part, const int tx)
 {
     using SM = TileSmem64<TX>;
     constexpr int WP = SM::WP, WM = SM::WM, NT = SM::NT, NW = (NT + 31) / 32;
     constexpr bool NEED_S = (PASS & (PASS_STATE | PASS_DIAG)) != 0;
     double(*const dacc)[NT] = reinterpret_cast<double(*)[NT]>(dyn);
     double(*const facc)[NT] = dacc + 4;
-    const int tx = threadIdx.x, ty = threadIdx.y, lin = ty * TX + tx;
+    const int ty = threadIdx.y, lin = ty * TX + tx;
     const int nx = P.nx, ny = P.ny;
     const unsigned N = (unsigned)P.N;
     const bool small = ny < 4;

@@ -487,7 +487,7 @@ __device__ __forceinline__ void d2q9_node(const StepParams<float> &P, const Pass
             // f_0 - f_0^eq = (5/9) alpha mu - sum_{i!=0} f_i
             const float ne = fmaf(float(5.0 / 9.0), am, -snz);
             const float d0 =
-                fmaf(float(-5.0 / 9.0), dsh, fmaf(float(-8.0 / 9.0), Sh, -(ne * itf)));
+                fmaf(-dsh, float(5.0 / 9.0), fmaf(-Sh, float(8.0 / 9.0), -ne * itf));
             // (hi, lo) + d0 with an exact two-sum on the high word
             const float sl = locur + d0;
             const float hi = fcur[0] + sl;
@@ -508,9 +508,9 @@ __device__ __forceinline__ void d2q9_node(const StepParams<float> &P, const Pass
         // (the two u.grad rho terms cancel).  Opposite directions share
         // the even part and flip the odd part.
         const float kg = fmaf(-0.5f, itg, 1.0f);
-        const float A = fmaf(-(1.5f * rho), uu, 3.0f * p);
+        const float p3 = 3.0f * p, A = fmaf(-(1.5f * rho), uu, p3);
         // G_0 = 0
-        st_stream(gd + n, fmaf(fmaf(float(4.0 / 9.0), A, -(3.0f * p)) - gv[0], itg, gv[0]));
+        st_stream(gd + n, fmaf(fmaf(float(4.0 / 9.0), A, -p3) - gv[0], itg, gv[0]));
         {
             // two populations per paired instruction: f 1..4 and 5..8 in
             // pairs; g the two axis and the two diagonal direction pairs
@@ -563,7 +563,8 @@ __device__ __forceinline__ void d2q9_node(const StepParams<float> &P, const Pass
 template <int TX, int PASS, bool NC = true, bool SEG = false>
 __device__ __forceinline__ void d2q9_tile(TileSmem<float, TX> &sm, float *dyn,
                                           const StepParams<float> &P, const PassArgs &a, int x0,
-                                          int y0, int yend, int dir, int part, unsigned &bph)
+                                          int y0, int yend, int dir, int part, unsigned &bph,
+                                          const int tx)
 {
     using SM = TileSmem<float, TX>;
     using SL = SegLayout<TX>;
@@ -577,12 +578,12 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<float, TX> &sm, float *dyn,
     float(*const facc)[NT] = dacc + NACC;
     float *const stg = reinterpret_cast<float *>(dyn);
     int *const dbad = &sm.bad;
-    const int lin = threadIdx.y * TX + threadIdx.x;
+    const int lin = threadIdx.y * TX + tx;
 
     const int nx = P.nx, ny = P.ny;
     const unsigned N = (unsigned)P.N;
     const bool small = ny < 4;
-    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int ty = threadIdx.y;
     const float *__restrict__ fsrc = static_cast<const float *>(a.f_src);
     const float *__restrict__ gsrc = static_cast<const float *>(a.g_src);
     constexpr bool NEED_S = (PASS & (PASS_STATE | PASS_DIAG)) != 0;
@@ -869,7 +870,7 @@ __device__ __forceinline__ void d2q9_tile(TileSmem<float, TX> &sm, float *dyn,
 #include "d2q9_fp64.cuh"
 
 // One tile of either storage type (see d2q9_tile; FP64 has a march of its own,
-// and no row-segment staging).
+// and no row-segment staging).  tx: the thread's index along x.
 template <typename T, int TX>
 struct SmemOf {
     using type = TileSmem<T, TX>;
@@ -881,12 +882,12 @@ struct SmemOf<double, TX> {
 template <typename T, int TX, int PASS, bool NC = true, bool SEG = false>
 __device__ __forceinline__ void run_tile(typename SmemOf<T, TX>::type &sm, T *dyn,
                                          const StepParams<T> &P, const PassArgs &a, int x0, int y0,
-                                         int yend, int dir, int part, unsigned &bph)
+                                         int yend, int dir, int part, unsigned &bph, int tx)
 {
     if constexpr (sizeof(T) == 8)
-        d2q9_tile64<TX, PASS, NC>(sm, dyn, P, a, x0, y0, yend, dir, part);
+        d2q9_tile64<TX, PASS, NC>(sm, dyn, P, a, x0, y0, yend, dir, part, tx);
     else
-        d2q9_tile<TX, PASS, NC, SEG>(sm, dyn, P, a, x0, y0, yend, dir, part, bph);
+        d2q9_tile<TX, PASS, NC, SEG>(sm, dyn, P, a, x0, y0, yend, dir, part, bph, tx);
 }
 
 // The kernels' dynamic shared memory (tile_dyn_bytes of their tile width).
@@ -898,15 +899,18 @@ template <typename T, int TX, int PASS>
 __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ctas))
     d2q9_pass_kernel(const StepParams<T> P, PassArgs a, int rows)
 {
-    const int bx = pdl_wait(blockIdx.x);
-    const int y0 = blockIdx.y * rows;
+    // (not the block index: it stays in uniform registers.  1024 x 1024 32.5 us per
+    // step, as without the dependence; 33.5 through the block index)
+    const int tx = pdl_wait(threadIdx.x);
+    __builtin_assume(tx >= 0 && tx < TX);
+    const int bx = blockIdx.x, y0 = blockIdx.y * rows;
     // march direction: alternating between neighbouring row tiles, and
     // reversed on every other step
     const int dir = ((blockIdx.y & 1) ? -1 : 1) * (a.flip ? -1 : 1);
     __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
     run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, bx * TX, y0,
-                          min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + bx, bph);
+                          min(y0 + rows, P.ny), dir, blockIdx.y * gridDim.x + bx, bph, tx);
 }
 
 // The FP32 step of a small or mid-sized grid: one 64 x 4 tile per CTA of as many
@@ -1019,7 +1023,7 @@ __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ct
     __shared__ typename SmemOf<T, TX>::type sm;
     unsigned bph = 0;  // no bulk staging here
     run_tile<T, TX, PASS>(sm, reinterpret_cast<T *>(tile_dyn), P, a, t.x0, t.y0, t.yend,
-                          parity ? -t.dir : t.dir, bx, bph);
+                          parity ? -t.dir : t.dir, bx, bph, threadIdx.x);
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int *p)
@@ -1304,16 +1308,17 @@ __global__ void __launch_bounds__((Occ<T, PASS_STATE, TX>::nth), (Occ<T, PASS_ST
         const bool seg = SEGK && seg_ok<T, TX>(P.nx, a.f_src, a.g_src, a.S);
         if (k == pa.diag_k) {
             if (seg)
-                run_tile<T, TX, PASS_STATE | PASS_DIAG, false, SEGK>(sm, dyn, P, a, t.x0, t.y0,
-                                                                       t.yend, dir, ti, bph);
+                run_tile<T, TX, PASS_STATE | PASS_DIAG, false, SEGK>(
+                    sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph, threadIdx.x);
             else
-                run_tile<T, TX, PASS_STATE | PASS_DIAG, false>(sm, dyn, P, a, t.x0, t.y0, t.yend,
-                                                                 dir, ti, bph);
+                run_tile<T, TX, PASS_STATE | PASS_DIAG, false>(
+                    sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph, threadIdx.x);
         } else if (seg) {
             run_tile<T, TX, PASS_STATE, false, SEGK>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti,
-                                                      bph);
+                                                     bph, threadIdx.x);
         } else {
-            run_tile<T, TX, PASS_STATE, false>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph);
+            run_tile<T, TX, PASS_STATE, false>(sm, dyn, P, a, t.x0, t.y0, t.yend, dir, ti, bph,
+                                               threadIdx.x);
         }
         // every thread read s_stepdone at this pair's top, before the tile's
         // barriers: thread 0 folds in what lane 31 saw, for the next pair, and

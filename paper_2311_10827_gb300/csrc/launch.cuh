@@ -24,17 +24,17 @@
 namespace wblbm {
 
 // Waits until the grid before this one has completed and its stores are
-// visible, and passes on its block index.  The kernels read what that grid
+// visible, and passes on an index.  The kernels read what that grid
 // wrote through the read-only path, and the compiler takes such loads for
 // loads of constants, which a memory clobber does not hold back: only an address
 // formed from a value that the wait itself defines orders them.  So a kernel
-// takes the block index along x from here, and every address of such a load
-// contains it; a load whose address contains no block index takes its pointer
-// through after_wait.
-__device__ __forceinline__ int pdl_wait(unsigned block)
+// takes an index along x, of its block or its thread, from here, and every
+// address of such a load contains it; a load whose address contains neither
+// takes its pointer through after_wait.
+__device__ __forceinline__ int pdl_wait(unsigned index)
 {
-    asm volatile("griddepcontrol.wait;" : "+r"(block)::"memory");
-    return (int)block;
+    asm volatile("griddepcontrol.wait;" : "+r"(index)::"memory");
+    return (int)index;
 }
 // p, not before a pdl_wait above (volatile statements keep their order).
 template <class T>

@@ -1,8 +1,9 @@
 """Kernels launched before the grid in front of them has ended (launch_pdl) read its
 results through the read-only path, and the compiler may place such loads
-anywhere their address is known.  So every one of these kernels takes its block
-index along x from the wait itself, uses no other, and reads nothing before it; a
-pointer that is read without that index goes through after_wait."""
+anywhere their address is known.  So every one of these kernels takes the index
+along x of its block or of its thread from the wait itself, uses no other, and
+reads nothing before it; a pointer that is read without that index goes through
+after_wait."""
 import os
 import re
 
@@ -29,7 +30,7 @@ def kernels(text):
         yield m.group(1), text[i:j], text[j:k]
 
 
-def test_every_kernel_of_launch_pdl_takes_its_block_index_from_the_wait():
+def test_every_kernel_of_launch_pdl_takes_an_index_from_the_wait():
     launched, waiting = set(), {}
     for f, text in sources():
         launched |= set(re.findall(r"launch_pdl\((\w+)", text)) - {"void"}
@@ -39,8 +40,9 @@ def test_every_kernel_of_launch_pdl_takes_its_block_index_from_the_wait():
     assert launched and launched == set(waiting)
     for name, (f, params, body) in waiting.items():
         where = f"{f}: {name}"
-        assert body.count("pdl_wait(blockIdx.x)") == 1 and body.count("pdl_wait(") == 1, where
-        assert body.count("blockIdx.x") == 1, where
+        assert body.count("pdl_wait(") == 1, where
+        index = re.search(r"pdl_wait\((blockIdx\.x|threadIdx\.x)\)", body).group(1)
+        assert body.count(index) == 1, where
         before = body[:body.index("pdl_wait(")]
         # only shared-memory declarations and constants stand before it
         rest = re.sub(r"(__shared__|constexpr|using)[^;]*;", "", before)
@@ -66,5 +68,17 @@ def test_uniform_reads_come_after_the_wait():
 def test_the_wait_defines_the_index():
     with open(os.path.join(CSRC, "launch.cuh")) as fh:
         text = fh.read()
-    assert re.search(r'asm volatile\("griddepcontrol\.wait;" : "\+r"\(block\)\s*::\s*"memory"\)', text)
+    assert re.search(r'asm volatile\("griddepcontrol\.wait;" : "\+r"\(index\)\s*::\s*"memory"\)', text)
     assert re.search(r'asm volatile\("" : "\+l"\(p\)\)', text)
+
+
+def test_the_tiles_take_the_threads_index_from_their_kernel():
+    """A kernel that passes its thread index on: the march has no other."""
+    for f, text in sources():
+        for m in re.finditer(r"void (d2q9_tile\w*)\(([^)]*)\)\s*\{", text):
+            assert re.search(r"\btx$", m.group(2)), m.group(1)
+            k, depth = m.end(), 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[k], 0)
+                k += 1
+            assert "threadIdx.x" not in text[m.end():k], m.group(1)
