@@ -39,8 +39,9 @@ struct TileSmem64 {
 };
 
 // One tile: columns [x0, x0 + TX), rows [y0, yend), marching in direction dir
-// (see d2q9_tile, which this replaces for FP64 storage).
-template <int TX, int PASS, bool NC>
+// (see d2q9_tile, which this replaces for FP64 storage).  INCG: g relaxes by
+// increments (INCR_G).
+template <int TX, int PASS, bool NC, bool INCG>
 __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                                             const StepParams<double> &P, const PassArgs &a, int x0,
                                             int y0, int yend, int dir, int part, const int tx)
@@ -271,27 +272,20 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                     s = E + O;
                     d = E - O;
                 };
-                auto collide_g = [&](auto inc) {
-                    constexpr bool INC = inc.value;
-                    double s, d;
-                    gd[n] = relax64<INC>(gv[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
-                    pair(ux, Fx, qx, s, d);
-                    gd[2 * N + n] = relax64<INC>(gv[2], itg, omg, s);
-                    gd[4 * N + n] = relax64<INC>(gv[4], itg, omg, d);
-                    pair(uy, Fy, qy, s, d);
-                    gd[3 * N + n] = relax64<INC>(gv[3], itg, omg, s);
-                    gd[1 * N + n] = relax64<INC>(gv[1], itg, omg, d);
-                    pair(ux + uy, Fx + Fy, qx + qy, s, d);
-                    gd[5 * N + n] = relax64<INC>(gv[5], itg, omg, 0.25 * s);
-                    gd[7 * N + n] = relax64<INC>(gv[7], itg, omg, 0.25 * d);
-                    pair(uy - ux, Fy - Fx, qy - qx, s, d);
-                    gd[6 * N + n] = relax64<INC>(gv[6], itg, omg, 0.25 * s);
-                    gd[8 * N + n] = relax64<INC>(gv[8], itg, omg, 0.25 * d);
-                };
-                if (P.incr & INCR_G)
-                    collide_g(std::true_type{});
-                else
-                    collide_g(std::false_type{});
+                double s, d;
+                gd[n] = relax64<INCG>(gv[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
+                pair(ux, Fx, qx, s, d);
+                gd[2 * N + n] = relax64<INCG>(gv[2], itg, omg, s);
+                gd[4 * N + n] = relax64<INCG>(gv[4], itg, omg, d);
+                pair(uy, Fy, qy, s, d);
+                gd[3 * N + n] = relax64<INCG>(gv[3], itg, omg, s);
+                gd[1 * N + n] = relax64<INCG>(gv[1], itg, omg, d);
+                pair(ux + uy, Fx + Fy, qx + qy, s, d);
+                gd[5 * N + n] = relax64<INCG>(gv[5], itg, omg, 0.25 * s);
+                gd[7 * N + n] = relax64<INCG>(gv[7], itg, omg, 0.25 * d);
+                pair(uy - ux, Fy - Fx, qy - qx, s, d);
+                gd[6 * N + n] = relax64<INCG>(gv[6], itg, omg, 0.25 * s);
+                gd[8 * N + n] = relax64<INCG>(gv[8], itg, omg, 0.25 * d);
             }
         }
 #pragma unroll
@@ -333,6 +327,7 @@ struct SmallSmem64 {
     double snz[32];               // sum of the moving f of the tile's nodes
     double w[14][32];             // stage 2 .. 4 results per node
 };
+template <bool INCG>
 __global__ void __launch_bounds__(SM64_NT, 4)
     d2q9_small64_kernel(const StepParams<double> P, PassArgs a)
 {
@@ -460,29 +455,22 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         s = E + O;
         d = E - O;
     };
-    auto collide_g = [&](auto inc) {
-        constexpr bool INC = inc.value;
-        double s, d;
-        if (warp == 1) {
-            pair(ux, Fx, qx, s, d);
-            gd[2 * N + n] = relax64<INC>(v[2], itg, omg, s);
-            gd[4 * N + n] = relax64<INC>(v[4], itg, omg, d);
-            pair(uy, Fy, qy, s, d);
-            gd[3 * N + n] = relax64<INC>(v[3], itg, omg, s);
-            gd[1 * N + n] = relax64<INC>(v[1], itg, omg, d);
-        } else if (warp == 2) {
-            pair(ux + uy, Fx + Fy, qx + qy, s, d);
-            gd[5 * N + n] = relax64<INC>(v[5], itg, omg, 0.25 * s);
-            gd[7 * N + n] = relax64<INC>(v[7], itg, omg, 0.25 * d);
-        } else {
-            gd[n] = relax64<INC>(v[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
-            pair(uy - ux, Fy - Fx, qy - qx, s, d);
-            gd[6 * N + n] = relax64<INC>(v[6], itg, omg, 0.25 * s);
-            gd[8 * N + n] = relax64<INC>(v[8], itg, omg, 0.25 * d);
-        }
-    };
-    if (P.incr & INCR_G)
-        collide_g(std::true_type{});
-    else
-        collide_g(std::false_type{});
+    double s, d;
+    if (warp == 1) {
+        pair(ux, Fx, qx, s, d);
+        gd[2 * N + n] = relax64<INCG>(v[2], itg, omg, s);
+        gd[4 * N + n] = relax64<INCG>(v[4], itg, omg, d);
+        pair(uy, Fy, qy, s, d);
+        gd[3 * N + n] = relax64<INCG>(v[3], itg, omg, s);
+        gd[1 * N + n] = relax64<INCG>(v[1], itg, omg, d);
+    } else if (warp == 2) {
+        pair(ux + uy, Fx + Fy, qx + qy, s, d);
+        gd[5 * N + n] = relax64<INCG>(v[5], itg, omg, 0.25 * s);
+        gd[7 * N + n] = relax64<INCG>(v[7], itg, omg, 0.25 * d);
+    } else {
+        gd[n] = relax64<INCG>(v[0], itg, omg, itg * fma(4.0 / 9.0, A, -p3));
+        pair(uy - ux, Fy - Fx, qy - qx, s, d);
+        gd[6 * N + n] = relax64<INCG>(v[6], itg, omg, 0.25 * s);
+        gd[8 * N + n] = relax64<INCG>(v[8], itg, omg, 0.25 * d);
+    }
 }

@@ -100,9 +100,9 @@ __device__ __forceinline__ void write_partial3(int tid, double d_phi, double d_E
 // operations: sums and differences of opposite populations serve the moments,
 // diagonal differences serve two gradient components, a reciprocal is three
 // operations, and a collision is one or two multiply-adds per population on
-// coefficients formed once per node.  100^3 1515 -> 1117 us per step, 200^3 9.0 ->
-// 6.6 ms.
-template <int PASS>
+// coefficients formed once per node (INCG: g relaxes by increments, INCR_G).
+// 100^3 1515 -> 1117 us per step, 200^3 9.0 -> 6.6 ms.
+template <int PASS, bool INCG>
 __global__ void __launch_bounds__(TX3 *TY3)
     d3q19_pass_kernel(const StepParams<double> P, PassArgs a, const double *__restrict__ phif,
                       int planes)
@@ -317,25 +317,18 @@ __global__ void __launch_bounds__(TX3 *TY3)
                 if ((cx || cy) && cz) s = cz > 0 ? s + v[2] : s - v[2];
                 return s;
             };
-            auto collide_g = [&](auto inc) {
-                constexpr bool INC = inc.value;
-                __stcs(gd + n, relax64<INC>(gv[0], itg, omg, itg * fma(T(1.0 / 3.0), A, -p3)));
+            __stcs(gd + n, relax64<INCG>(gv[0], itg, omg, itg * fma(T(1.0 / 3.0), A, -p3)));
 #pragma unroll
-                for (int i = 1; i < 19; ++i) {
-                    const int o = opp(i);
-                    if (o < i) continue;
-                    const T cu = dot(c3x(i), c3y(i), c3z(i), u), cF = dot(c3x(i), c3y(i), c3z(i), F);
-                    const T cq = dot(c3x(i), c3y(i), c3z(i), q);
-                    const T E = fma(cu, fma(e2, cq, e1 * cu), e0), O = fma(o2, cF, o1 * cu);
-                    const T w = i <= 6 ? T(1) : T(0.5);
-                    __stcs(gd + (i * N + n), relax64<INC>(gv[i], itg, omg, w * (E + O)));
-                    __stcs(gd + (o * N + n), relax64<INC>(gv[o], itg, omg, w * (E - O)));
-                }
-            };
-            if (P.incr & INCR_G)
-                collide_g(std::true_type{});
-            else
-                collide_g(std::false_type{});
+            for (int i = 1; i < 19; ++i) {
+                const int o = opp(i);
+                if (o < i) continue;
+                const T cu = dot(c3x(i), c3y(i), c3z(i), u), cF = dot(c3x(i), c3y(i), c3z(i), F);
+                const T cq = dot(c3x(i), c3y(i), c3z(i), q);
+                const T E = fma(cu, fma(e2, cq, e1 * cu), e0), O = fma(o2, cF, o1 * cu);
+                const T w = i <= 6 ? T(1) : T(0.5);
+                __stcs(gd + (i * N + n), relax64<INCG>(gv[i], itg, omg, w * (E + O)));
+                __stcs(gd + (o * N + n), relax64<INCG>(gv[o], itg, omg, w * (E - O)));
+            }
         }
         }  // col_ok
         {
@@ -740,7 +733,11 @@ cudaError_t launch3(const void *params, const PassArgs &a, const LaunchShape &s,
         return launch_pdl(d3q19_pass32_kernel<PASS, false>, grid, block, 0, st, P, a,
                           static_cast<const float *>(phi), s.rows);
     } else {
-        return launch_pdl(d3q19_pass_kernel<PASS>, grid, dim3(TX3, TY3), 0, st, P, a,
+        if constexpr (PASS & PASS_STATE)
+            if (P.incr & INCR_G)
+                return launch_pdl(d3q19_pass_kernel<PASS, true>, grid, dim3(TX3, TY3), 0, st, P, a,
+                                  static_cast<const T *>(phi), s.rows);
+        return launch_pdl(d3q19_pass_kernel<PASS, false>, grid, dim3(TX3, TY3), 0, st, P, a,
                           static_cast<const T *>(phi), s.rows);
     }
 }
@@ -799,7 +796,7 @@ int d3q19_ctas_per_sm(int precision)
     int n = 0;
     cudaError_t e = precision == 0
                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &n, d3q19_pass_kernel<PASS_STATE>, TX3 * TY3, 0)
+                              &n, d3q19_pass_kernel<PASS_STATE, false>, TX3 * TY3, 0)
                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                               &n, d3q19_pass32_kernel<PASS_STATE, true>, PAIR_NT, 0);
     return e == cudaSuccess && n > 0 ? n : 2;

@@ -11,12 +11,21 @@
 
 namespace wblbm {
 
+// What FP64 runs hold beside the scalars.  (The FP32 kernels, at the limit of their
+// registers, get no field that they do not use: it cost 36 bytes of spills.)
+template <typename T>
+struct StepForm {
+};
+template <>
+struct StepForm<double> {
+    int incr;            // INCR_* populations relax by their increments
+};
+
 // Scalars of one run in the compute type T (derived on the host from the
 // paper's parameters; see lbm_create).
 template <typename T>
-struct StepParams {
+struct StepParams : StepForm<T> {
     int nx, ny, nz;
-    int incr;            // FP64: INCR_* populations relax by their increments
     long long N;         // nodes
     T kappa, beta;       // Eqs. beta, suiface_tension
     T phil, phiv, phibar;
@@ -129,9 +138,11 @@ void fill_step_params(StepParams<T> &P, const lbm_grid &g, const lbm_params &p, 
     P.ny = g.ny;
     P.nz = g.nz;
     P.N = (long long)g.nx * g.ny * g.nz;
-    // (nu with a tenth of its range to spare: phi overshoots its phases a little)
-    const double nu = fmax(p.nu_l, p.nu_v) + 0.1 * fabs(p.nu_l - p.nu_v);
-    P.incr = (d.tau_f > 2.0 ? INCR_F : 0) | (0.5 + 3.0 * nu > 2.0 ? INCR_G : 0);
+    if constexpr (sizeof(T) == 8) {
+        // (nu with a tenth of its range to spare: phi overshoots its phases a little)
+        const double nu = fmax(p.nu_l, p.nu_v) + 0.1 * fabs(p.nu_l - p.nu_v);
+        P.incr = (d.tau_f > 2.0 ? INCR_F : 0) | (0.5 + 3.0 * nu > 2.0 ? INCR_G : 0);
+    }
     P.kappa = (T)d.kappa;
     P.beta = (T)d.beta;
     P.phil = (T)p.phi_l;

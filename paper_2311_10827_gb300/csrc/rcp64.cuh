@@ -34,7 +34,7 @@ __device__ __forceinline__ double rcp64(double x)
 // grows with every step, where independent roundings average out.  There (INC)
 // the population is moved by its increment -r x + s, one operation more.  A
 // run's parameters choose (StepParams::incr), not a node's rate: warps on an
-// interface would run both forms (64^3 238 -> 312 us per step).
+// interface would run both forms (64^3 312 us per step against 248).
 template <bool INC>
 __device__ __forceinline__ double relax64(double x, double r, double omr, double s)
 {
