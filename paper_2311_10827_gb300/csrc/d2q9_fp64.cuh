@@ -19,7 +19,7 @@
 //    direction class;
 //  * the halo columns of both thread rows are one warp's extra work instead
 //    of two warps'.
-// About 155 FP64 operations per node against about 250 in the form shared with
+// About 156 FP64 operations per node against about 250 in the form shared with
 // the FP32 kernel before.  Measured with per-step launches, whole runs of 40
 // and 400 steps: 1024 x 1024 505 -> 363 us per step (the operations alone take
 // 255 us), 16 x 128 16.5 -> 9.9 us; with 64-column tiles 341 us.
@@ -242,11 +242,12 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
                 static_cast<double *>(a.S_out)[n] = 0.5 * S2;
                 // Eq. BGK with Eqs. H_i, F_i: f* = f (1 - 1/tau_f) + z w_i + w_i b_i Sh,
                 // z = alpha mu / tau_f, Sh = 1.5 S - 0.5 S_prev, b = -2, -1/2, 1;
-                // the rest population through f_0 - f_0^eq = (5/9) alpha mu - sum f_i
+                // the rest population through f_0 - f_0^eq = (5/9) alpha mu - sum f_i,
+                // its increment formed first: one rounding at its size, which is phi's
                 const double Sh = fma(0.75, S2, -0.5 * Sprev);
                 const double itf = P.inv_tauf, omf = 1.0 - itf;
                 const double z = (itf * P.alpha) * mu;
-                fd[n] = fma(itf, scur, fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, fcur[0])));
+                fd[n] = fcur[0] + fma(itf, scur, fma(-5.0 / 9.0, z, (-8.0 / 9.0) * Sh));
                 const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
                 auto collide_f = [&](auto inc) {
 #pragma unroll
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(SM64_NT, 4)
         const double Sh = fma(0.75, S2, -0.5 * Sprev);
         const double itf = P.inv_tauf, omf = 1.0 - itf;
         const double z = (itf * P.alpha) * m0[k];
-        fd[n] = fma(itf, sm.snz[lane], fma(-5.0 / 9.0, z, fma(-8.0 / 9.0, Sh, v[0])));
+        fd[n] = v[0] + fma(itf, sm.snz[lane], fma(-5.0 / 9.0, z, (-8.0 / 9.0) * Sh));
         const double ka = (1.0 / 9.0) * fma(-0.5, Sh, z), kd = (1.0 / 36.0) * (z + Sh);
         auto collide_f = [&](auto inc) {
 #pragma unroll

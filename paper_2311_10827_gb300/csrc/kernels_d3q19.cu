@@ -292,7 +292,8 @@ __global__ void __launch_bounds__(TX3 *TY3)
             // f* = f (1 - 1/tau_f) + w_i z + w_i b_i Sh, z = alpha mu / tau_f
             const T Sh = fma(T(1.5), S, T(-0.5) * Sprev);
             const T itf = P.inv_tauf, omf = T(1) - itf, z = (itf * P.alpha) * mu;
-            __stcs(fd + n, fma(itf, snz, fma(T(-2.0 / 3.0), z, fma(T(-5.0 / 6.0), Sh, fv[0]))));
+            // (the rest population's increment first: one rounding at its size)
+            __stcs(fd + n, fv[0] + fma(itf, snz, fma(T(-2.0 / 3.0), z, T(-5.0 / 6.0) * Sh)));
             const T ka = T(1.0 / 18.0) * (z - Sh), ke = T(1.0 / 36.0) * fma(T(0.5), Sh, z);
             auto collide_f = [&](auto inc) {
 #pragma unroll
