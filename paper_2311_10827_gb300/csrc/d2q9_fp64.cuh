@@ -11,7 +11,7 @@
 //    h + (2/3) v + (1/6)(v_E + v_W) with h the horizontal second difference,
 //    and the gradient (1/2)(phi_E - phi_W) + (1/12)(v_E - v_W),
 //    (1/3) d + (1/12)(d_E + d_W).  Every term stays a difference of
-//    neighbours, so a uniform phase still gives exact zeros;
+//    neighbours, so a uniform field still gives exact zeros;
 //  * 1/rho and 1/tau_g are three operations each and as accurate as a divide
 //    (rcp64; one reciprocal of rho tau_g for both takes as many, and loses an ulp);
 //  * each collision is one multiply-add per population (two for relaxation
@@ -19,10 +19,10 @@
 //    direction class;
 //  * the halo columns of both thread rows are one warp's extra work instead
 //    of two warps'.
-// About 156 FP64 operations per node against about 250 in the form shared with
-// the FP32 kernel before.  Measured with per-step launches, whole runs of 40
-// and 400 steps: 1024 x 1024 505 -> 363 us per step (the operations alone take
-// 255 us), 16 x 128 16.5 -> 9.9 us; with 64-column tiles 341 us.
+// About 156 FP64 operations per node (165 with tau_g > 2) against about 250 in the
+// form shared with the FP32 kernel before.  Measured, us per step: 1024 x 1024
+// 498 -> 344 (359 with tau_g > 2; the operations alone take 260 and 275), 512 x 512
+// 153 -> 99 (103), 301 x 203 54.9 -> 32.5 (33.7); 128-column tiles were 6% slower.
 #pragma once
 
 // shared memory of one FP64 tile march
@@ -308,12 +308,12 @@ __device__ __forceinline__ void d2q9_tile64(TileSmem64<TX> &sm, double *dyn,
 // The FP64 time step of a grid too small to fill the chip.  A warp takes 64
 // cycles for any FP64 instruction, whatever its active lanes, and each of the
 // SM's four schedulers has one such pipe; with fewer warps than pipes the step
-// takes the operations of one warp, one after the other (7.2 us for the 177 of
+// takes the operations of one warp, one after the other (7.2 us for the 180 of
 // two rows of d2q9_tile64).  Here a tile of 16 x 2 nodes is one CTA of four
 // warps, one per scheduler, that share the node update: every warp holds the 32
 // nodes and does a part of their operations, so that about 85 of them are in
 // sequence.  Each value is formed by the expressions of d2q9_tile64.  16 x 128:
-// 9.5 -> 5.1 us per step.
+// 9.5 -> 4.9 us per step.
 //   1  phi of the tile and two halo rows and columns (one node per thread)
 //   2  v, d of one halo row                 warp 3: rho u's sum, sum of g
 //   3  mu of one halo row and column          (while 1 .. 3 run elsewhere)

@@ -901,7 +901,7 @@ extern __shared__ float4 tile_dyn[];
 // Single grid: CTA (bx, by) owns strip bx and row tile by; even row tiles
 // march down, odd ones up, so neighbouring tiles meet at their shared rows.
 // FP64 has a kernel for each form of g's relaxation: with both in one, 1500 x 1500
-// took 973 us per step instead of 913, or 930 instead of 872 (nu_l = 1, 0.1).
+// took 973 us per step instead of 911, or 930 instead of 871 (nu_l = 1, 0.1).
 template <typename T, int TX, int PASS, bool INCG = false>
 __global__ void __launch_bounds__((Occ<T, PASS, TX>::nth), (Occ<T, PASS, TX>::ctas))
     d2q9_pass_kernel(const StepParams<T> P, PassArgs a, int rows)
@@ -1562,7 +1562,7 @@ cudaError_t launch_pass_g(const StepParams<T> &P, const PassArgs &a, const Launc
         if constexpr (PASS == PASS_STATE) {
             const dim3 tiles((P.nx + SM64_TX - 1) / SM64_TX, (P.ny + 1) / 2);
             // at most one tile per SM: with two, its schedulers hold two warps of
-            // about 85 operations each, no fewer than the one warp of 177 that
+            // about 85 operations each, no fewer than the one warp of 180 that
             // d2q9_tile64 gives them on such a grid, and more in all
             if (tiles.x * (long long)tiles.y <= (s.num_sms > 0 ? s.num_sms : 152))
                 return launch_pdl(d2q9_small64_kernel<INCG>, tiles, SM64_NT, 0, st, P, a);

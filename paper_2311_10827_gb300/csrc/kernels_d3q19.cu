@@ -6,13 +6,14 @@
 // Storage as in 2D: pull scheme, SoA [i][z][y][x], post-collision values at
 // their source node.  A step is two passes:
 //   1. d3q19_phi_kernel: phi = sum_i f_i pulled (one FP field);
-//   2. d3q19_pass_kernel: a CTA owns a TX x TY column tile and marches down
-//      z; phi planes (tile + 2 halo, read from the phi field, mostly L2) and
-//      mu planes (tile + 1) live in shared-memory rings; each node pulls its
-//      19 + 19 populations, recovers the moments and collides.
-// HBM traffic per node (FP32): 84 B for pass 1, 324 B for pass 2.  As in 2D,
-// FP32 storage keeps the rest population as a compensated pair hi + lo (lo in
-// population slot 19) so that its small per-step changes are not lost.
+//   2. d3q19_pass32_kernel (FP32, two nodes per thread) or d3q19_pass_kernel
+//      (FP64, one): a CTA owns a TX x TY column tile and marches down z; phi
+//      planes (tile + 2 halo, read from the phi field, mostly L2) and mu planes
+//      (tile + 1) live in shared-memory rings; each node pulls its 19 + 19
+//      populations, recovers the moments and collides.
+// HBM traffic per node of the FP32 form: 84 B for pass 1, 324 B for pass 2.  As
+// in 2D, FP32 storage keeps the rest population as a compensated pair hi + lo
+// (lo in population slot 19) so that its small per-step changes are not lost.
 #include <float.h>
 #include <math.h>
 
@@ -101,7 +102,8 @@ __device__ __forceinline__ void write_partial3(int tid, double d_phi, double d_E
 // diagonal differences serve two gradient components, a reciprocal is three
 // operations, and a collision is one or two multiply-adds per population on
 // coefficients formed once per node (INCG: g relaxes by increments, INCR_G).
-// 100^3 1515 -> 1117 us per step, 200^3 9.0 -> 6.6 ms.
+// 100 x 75 x 130 1447 -> 1060 us per step (1108 with tau_g > 2), 160^3 4.06 -> 2.96 ms
+// (3.10).
 template <int PASS, bool INCG>
 __global__ void __launch_bounds__(TX3 *TY3)
     d3q19_pass_kernel(const StepParams<double> P, PassArgs a, const double *__restrict__ phif,
@@ -768,9 +770,12 @@ LaunchShape d3q19_shape(int nx, int ny, int nz, int num_sms, int ctas_per_sm)
     // Split z into gz marches of `planes` planes.  A march takes about planes + 2
     // planes of work (it starts by filling its rings), and CTAs that share an SM
     // hide part of each other's waits: two take 1.3 times one's time, three 1.6
-    // (64^3: 256 CTAs of 4 planes 16.7 us, 352 of 3 planes 17.2 us).  An SM works
+    // (FP32, 64^3: 256 CTAs of 4 planes 16.7 us, 352 of 3 planes 17.2 us; the FP64
+    // pass has one CTA per SM, so that k of them take k times one's).  An SM works
     // through its share of the CTAs, `occ` at a time; pick the split with the
-    // least time.
+    // least time.  Against counting waves of CTAs with marches of at least four
+    // planes, over 26 shapes from 24^3 to 320 x 320 x 24 in each of the four formats:
+    // none more than 0.3% slower, 24^3 1.4x (FP64 1.7x), 321 x 24 x 25 1.37x.
     const long long cols = (long long)s.grid_x * s.grid_y;
     const long long occ = ctas_per_sm > 0 ? ctas_per_sm : 2, sms = num_sms > 0 ? num_sms : 152;
     auto share = [](long long k) { return k == 0 ? 0.0 : 1.0 + 0.3 * (double)(k - 1); };
