@@ -961,10 +961,11 @@ __device__ inline double geq_of(const EqData &e, float p, int i)
 // exactly half of it on the edges, the second stores their differences from the
 // neighbours' equilibria.  Of the state only the parity that is initialised is
 // written: phi0 may lie in the other one.  The FP64 pipe bounds both; the scales
-// are powers of two, so the values are multiplied by 1/s_f before their
-// differences are formed, which is exact and rounds to FP32 and to storage as
-// the divided difference does, down to its smallest values (a divide of its
-// own for each of the 19 values made this 13.1 ms at 256^3, against 3.0 ms now).
+// are powers of two, so the values are taken times 1/s_f before their differences
+// are formed, which is exact and rounds to FP32 and to storage as the divided
+// difference does, down to its smallest values, and takes one FP64 operation (a
+// divide of its own for each of the 19 values made this 13.1 ms at 256^3, against
+// 3.0 ms now).
 template <class C>
 __global__ void __launch_bounds__(256)
     d3q19_off_init_macros_k(const StepParams<double> Pd, const StepParams<float> P,
@@ -983,7 +984,7 @@ __global__ void __launch_bounds__(256)
     const double c = __ldg(phi0 + n);
     const double mu = mu_of_field(Pd, phi0, b, c), am = Pd.alpha * mu;
     static_assert(2.0 * w3(7) == w3(1), "edge values are half the face values");
-    fa[n] = inv * (w3(1) * am);
+    fa[n] = (inv * w3(1)) * am;
     const float phi_hi = (float)c, mu_f = (float)mu;
     o.M[n] = phi_hi;
     o.M[N + n] = mu_f;
@@ -997,8 +998,7 @@ __global__ void __launch_bounds__(256)
 
 template <class C>
 __global__ void __launch_bounds__(256)
-    d3q19_off_init_k(const StepParams<float> P, const double *__restrict__ fa, OffBuf o,
-                     double inv)
+    d3q19_off_init_k(const StepParams<float> P, const double *__restrict__ fa, OffBuf o, float inv)
 {
     const unsigned N = (unsigned)P.N, n = blockIdx.x * 256u + threadIdx.x;
     if (n >= N) return;
@@ -1006,7 +1006,7 @@ __global__ void __launch_bounds__(256)
     const unsigned r = n / nx;
     const Nb b = make_nb((int)(n - r * nx), (int)(r % ny), (int)(r / ny), P.nx, P.ny, P.nz);
     const float q0 = P.alpha * o.M[N + n];
-    const double eqa = inv * (double)((float)w3(1) * q0), eqe = inv * (double)((float)w3(7) * q0);
+    const double eqa = (double)((float)w3(1) * q0 * inv), eqe = (double)((float)w3(7) * q0 * inv);
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
         const unsigned m = b.at(c3x(i), c3y(i), c3z(i));
@@ -1231,11 +1231,11 @@ cudaError_t d3q19_off_init(int codec, const void *params64, const void *params32
     if (codec == OFFSET_F16) {
         d3q19_off_init_macros_k<CodecF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp, o, (float *)S, sf,
                                                               sg, inv);
-        d3q19_off_init_k<CodecF16><<<nb, 256, 0, st>>>(P, tmp, o, inv);
+        d3q19_off_init_k<CodecF16><<<nb, 256, 0, st>>>(P, tmp, o, (float)inv);
     } else {
         d3q19_off_init_macros_k<CodecBF16><<<nb, 256, 0, st>>>(Pd, P, phi0, tmp, o, (float *)S, sf,
                                                                sg, inv);
-        d3q19_off_init_k<CodecBF16><<<nb, 256, 0, st>>>(P, tmp, o, inv);
+        d3q19_off_init_k<CodecBF16><<<nb, 256, 0, st>>>(P, tmp, o, (float)inv);
     }
     d3q19_off_prep_k<<<dim3((P.nx + PHI_TX - 1) / PHI_TX, P.ny, P.nz), PHI_TX, 0, st>>>(P, o);
     return cudaGetLastError();
